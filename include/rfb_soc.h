@@ -109,8 +109,9 @@ typedef struct rfb_solve_opts {
     double cfl;             /* C_CFL in (0, 1] (default 0.4) */
     double velocity_scale;  /* beta >= 0: every face velocity is multiplied by it (1) */
     int64_t max_sweeps;     /* give up after this many sweeps (0 = 50,000,000) */
-    int32_t fp32_kernel;    /* RFB_PREC_MIXED only: 0 = chosen by timing the kernels on
-                               the lattice (once per lattice shape, dt mode
+    int32_t fp32_kernel;    /* RFB_PREC_MIXED only: 0 = resident sweeps where the lattice
+                               fits on the chip (local steps), else chosen by timing the
+                               kernels on the lattice (once per lattice shape, dt mode
                                and device in a process), 1 = one sweep per launch,
                                2 = several sweeps per pass (TMA-staged, temporally
                                blocked; local steps: nx % 4 == 0; global step: nx % 16
@@ -525,7 +526,8 @@ rfb_status rfb_selftest_bounded_wait(int64_t spin_limit, int32_t* gave_up);
 /* The FP32 correction kernel the handle's autotuner chose for RFB_PREC_MIXED solves with
  * fp32_kernel = 0 or 2 (or the one a solve forced), as an opts.fp32_kernel value: 0 = not
  * chosen yet, 1 = one sweep per launch, 3 / 4 = two-sweep passes in the persistent /
- * chunked launch shape, 5 / 6 the same with four TMA stages, 7 .. 10 three-sweep passes;
+ * chunked launch shape, 5 / 6 the same with four TMA stages, 7 .. 10 three-sweep passes,
+ * 11 = resident sweeps (fp32_kernel = 0 on a lattice that fits on the chip);
  * and the timed device milliseconds per sweep of the one-sweep kernel and of the fastest
  * pass variant (0 if not timed). Any output pointer may be NULL. */
 rfb_status rfb_soc_tuned_fp32_kernel(const rfb_soc_handle* h, int32_t* kernel,

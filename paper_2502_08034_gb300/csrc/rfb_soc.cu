@@ -6,6 +6,7 @@
 #include "sweep_tb.cuh"
 #include "sweep_dt.cuh"
 #include "sweep_t3.cuh"
+#include "sweep_res.cuh"
 #include "bv_kernels.cuh"
 
 #include <cuda.h>
@@ -135,6 +136,15 @@ struct rfb_soc_handle {
     CUtensorMap tm_delta[2], tm_r, tm_u, tm_v, tm_w, tm_f, tm_t;
     float* tm_delta_ptr[2] = {nullptr, nullptr};
     double tb_tuned_plain_ms = 0, tb_tuned_tb_ms = 0;
+    // resident FP32 sweeps (sweep_res.cuh): bricks of the lattice, inboxes (first use), the
+    // tag of the next launch's words
+    struct ResPlan {
+        int cpt = -1;             // planes of a brick; 0 the lattice does not fit, -1 not planned
+        int bx = 0, by = 0, gx = 0, gy = 0, gz = 0;
+    } res;
+    bool res_used = false;        // the last FP32 correction sweeps were resident ones
+    unsigned long long* d_inbox = nullptr;
+    uint32_t res_tag = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 };
 
@@ -684,10 +694,111 @@ void plain_sweep(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int
     LAUNCHED(h);
 }
 
+// the two correction buffers (and their tensor maps) change places
+void swap_delta(rfb_soc_handle* h) {
+    std::swap(h->d_delta[0], h->d_delta[1]);
+    if (h->tm_ready) {
+        std::swap(h->tm_delta[0], h->tm_delta[1]);
+        std::swap(h->tm_delta_ptr[0], h->tm_delta_ptr[1]);
+    }
+}
+
+// ---- resident sweeps (sweep_res.cuh)
+
+using ResKernel = void (*)(ResArgs);
+template <bool TR>
+ResKernel res_kernel(int cpt) {
+    switch (cpt) {
+        case 2: return sweep32r_kernel<2, TR>;
+        case 4: return sweep32r_kernel<4, TR>;
+        case 6: return sweep32r_kernel<6, TR>;
+        case 8: return sweep32r_kernel<8, TR>;
+        case 10: return sweep32r_kernel<10, TR>;
+        default: return sweep32r_kernel<12, TR>;
+    }
+}
+
+// Whether the resident sweeps take this lattice: its bricks, one per SM, are all on the chip
+// at once (up to about 0.9 M cells). They are the faster ones wherever they fit: 1.9 us a
+// sweep at 528k cells, where launches and passes take 6.2 us. Among the cuts that fit, the one with the least shared-memory work per sweep (the
+// word latency is the same for all).
+bool res_fits(rfb_soc_handle* h) {
+    if (h->res.cpt >= 0) return h->res.cpt > 0;
+    h->res.cpt = 0;
+    int sms = 0, coop = 0;
+    CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    CK(h, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
+    if (!coop) return false;
+    double best = INFINITY;
+    for (int gx = 1; gx <= std::min(h->nx / 2, sms); ++gx) {
+        const int bx = (h->nx + gx - 1) / gx;
+        if ((h->nx + bx - 1) / bx != gx) continue;
+        for (int gy = 1; gy <= std::min(h->ny / 2, sms / gx); ++gy) {
+            const int by = (h->ny + gy - 1) / gy;
+            if ((h->ny + by - 1) / by != gy || bx * by > RES_T ||
+                bx > 64 || bx * (by + 2) > RES_ROWS)
+                continue;
+            for (int cpt : {2, 4, 6, 8, 10, 12}) {
+                const int gz = (h->nz + cpt - 1) / cpt;
+                const int ring = 2 * cpt * (bx + by);
+                if (gx * gy * gz > sms || ring > 2 * RES_RING * RES_T) continue;
+                const double cost = 5.0 * cpt * ((bx * by + 31) / 32) + 0.25 * ring;
+                if (cost < best) {
+                    best = cost;
+                    h->res = {cpt, bx, by, gx, gy, gz};
+                }
+            }
+        }
+    }
+    return h->res.cpt > 0;
+}
+
+// n sweeps (tr: of the transposed operator) from delta = 0; the result is left in d_delta[0].
+// One launch does them all, or 4096 at a time (a launch of some ms).
+void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n, bool tr) {
+    const auto& P = h->res;
+    ResArgs A{};
+    A.nx = h->nx; A.ny = h->ny; A.nz = h->nz;
+    A.bx = P.bx; A.by = P.by;
+    A.gx = P.gx; A.gy = P.gy; A.gz = P.gz;
+    A.u = h->d_u32; A.v = h->d_v32; A.w = h->d_w32; A.dt = h->d_dtc;
+    A.r = h->d_r32;
+    A.omc = (float)(1.0 - op.cfl);
+    A.Dh = C.Dh;
+    A.err = tb_err_word(h);
+    A.stride = res_stride(P.cpt, P.bx, P.by);
+    const int ctas = P.gx * P.gy * P.gz;
+    if (!h->d_inbox) dalloc(h, &h->d_inbox, (size_t)ctas * 2 * A.stride);
+    A.inbox = h->d_inbox;
+    const ResKernel k = tr ? res_kernel<true>(P.cpt) : res_kernel<false>(P.cpt);
+    const int smem = res_smem(P.cpt);
+    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    for (int64_t q = 0; q < n; q += A.n) {
+        A.n = (int)std::min<int64_t>(n - q, 4096);
+        A.in = q ? h->d_delta[0] : nullptr;
+        A.out = h->d_delta[q ? 1 : 0];
+        A.tag = h->res_tag;
+        h->res_tag += (uint32_t)A.n;
+        void* args[] = {&A};
+        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(RES_T), args, smem,
+                                          h->stream));
+        ++h->launches;
+        if (q) swap_delta(h);
+    }
+}
+
+// How a call's FP32 sweeps run: one launch per sweep, passes of the chosen variant (two or
+// three sweeps each, single sweeps for the remainder), or resident sweeps.
+enum class Sweep32 { plain, pass, resident };
+
 // n FP32 correction sweeps delta <- delta + dt (L delta + r), starting from delta = 0.
-// The result is left in d_delta[0]. use_tb: passes of the chosen variant (two or three
-// sweeps each), plain sweeps for the remainder.
-void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, bool use_tb = false) {
+// The result is left in d_delta[0].
+void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Sweep32::plain) {
+    if (how == Sweep32::resident) {
+        res_sweeps(h, op, make_coef<float>(h, op, true, false), n, false);
+        return;
+    }
+    const bool use_tb = how == Sweep32::pass;
     const size_t bytes = (size_t)h->N * sizeof(float);
     CK(h, cudaMemsetAsync(h->d_delta[0], 0, bytes, h->stream));
     CK(h, cudaMemsetAsync(h->d_delta[1], 0, bytes, h->stream));
@@ -709,20 +820,19 @@ void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, bool use_tb = fal
         plain_sweep(h, op, C, cur, local);
         cur ^= 1;
     }
-    if (cur == 1) {
-        std::swap(h->d_delta[0], h->d_delta[1]);
-        if (h->tm_ready) {
-            std::swap(h->tm_delta[0], h->tm_delta[1]);
-            std::swap(h->tm_delta_ptr[0], h->tm_delta_ptr[1]);
-        }
-    }
+    if (cur == 1) swap_delta(h);
 }
 
 // n FP32 correction sweeps of the transposed operator (adjoint), delta <- delta +
 // dt (L^T delta + r), from delta = 0; the result is left in d_delta[0] (nx % 4 == 0).
-// With local steps: passes of the step-field kernels (two or three sweeps each, the
-// variant the autotuner chose), plain sweeps for the remainder.
+// With local steps: resident sweeps where the lattice fits and no pass variant was chosen
+// before, else passes of the step-field kernels (two or three sweeps each, the variant the
+// autotuner chose), plain sweeps for the remainder.
 void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n) {
+    if (op.dt_mode == RFB_DT_LOCAL && h->tb_variant < 0 && res_fits(h)) {
+        res_sweeps(h, op, C, n, true);
+        return;
+    }
     const size_t bytes = (size_t)h->N * sizeof(float);
     CK(h, cudaMemsetAsync(h->d_delta[0], 0, bytes, h->stream));
     CK(h, cudaMemsetAsync(h->d_delta[1], 0, bytes, h->stream));
@@ -749,13 +859,7 @@ void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C
         LAUNCHED(h);
         cur ^= 1;
     }
-    if (cur == 1) {
-        std::swap(h->d_delta[0], h->d_delta[1]);
-        if (h->tm_ready) {
-            std::swap(h->tm_delta[0], h->tm_delta[1]);
-            std::swap(h->tm_delta_ptr[0], h->tm_delta_ptr[1]);
-        }
-    }
+    if (cur == 1) swap_delta(h);
 }
 
 // Choices of the FP32-kernel autotuner, kept for the process by lattice shape (dims,
@@ -801,11 +905,12 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
     for (float& m : ms) m = INFINITY;
     for (int cand = tb_only ? 1 : 0; cand <= nvar; ++cand) {
         if (cand > 0) h->tb_variant = cand - 1;
-        sweeps32(h, op, 6, cand > 0);   // warm-up (and tensor maps)
+        const Sweep32 how = cand > 0 ? Sweep32::pass : Sweep32::plain;
+        sweeps32(h, op, 6, how);   // warm-up (and tensor maps)
         for (int rep = 0; rep < 2; ++rep) {   // the faster of two timings
             float t = 0.f;
             CK(h, cudaEventRecord(h->ev[0], h->stream));
-            sweeps32(h, op, 12, cand > 0);
+            sweeps32(h, op, 12, how);
             CK(h, cudaEventRecord(h->ev[1], h->stream));
             CK(h, cudaEventSynchronize(h->ev[1]));
             CK(h, cudaEventElapsedTime(&t, h->ev[0], h->ev[1]));
@@ -945,10 +1050,14 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
         fill_result(h, op, &r, n_unknown);
         joined = true;
     };
-    // FP32 kernel: one-sweep or two-sweep passes (forced by opts or autotuned once)
-    bool use_tb = false;
+    // FP32 kernel: resident sweeps where the lattice fits on the chip (local steps), else
+    // one-sweep launches or passes (forced by opts or autotuned once)
+    bool use_tb = false, use_res = false;
     if (mixed) {
-        if (o.fp32_kernel == 2) {
+        use_res = o.fp32_kernel == 0 && op.dt_mode == RFB_DT_LOCAL && res_fits(h);
+        h->res_used = use_res;
+        if (use_res) {
+        } else if (o.fp32_kernel == 2) {
             if (h->tb_variant < 0) tune_fp32_kernel(h, op, true);
             use_tb = true;
         } else if (o.fp32_kernel >= 3) {
@@ -963,10 +1072,11 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
             if (h->tb_mode < 0) tune_fp32_kernel(h, op);
             use_tb = h->tb_mode == 1;
         }
-        if (use_tb) CK(h, cudaMemsetAsync(tb_err_word(h), 0, sizeof(unsigned int), h->stream));
+        if (use_tb || use_res) CK(h, cudaMemsetAsync(tb_err_word(h), 0, sizeof(unsigned int), h->stream));
     }
     // sweeps per pass: the default interval and the shortened ones are whole passes
     const int depth = use_tb ? tb_depth(h) : 1;
+    const Sweep32 how = use_res ? Sweep32::resident : use_tb ? Sweep32::pass : Sweep32::plain;
     if (o.check_every == 0) every = std::max<int64_t>(depth, every / depth * depth);
     // Check interval: `every` sweeps, shortened near the end. The residual of these
     // transport problems does not decay geometrically early on (it stays up while the
@@ -1013,7 +1123,7 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
         }
         const int64_t n = std::min(next_every, limit - done);
         CK(h, cudaEventRecord(h->ev[0], h->stream));
-        if (mixed) sweeps32(h, op, n, use_tb);
+        if (mixed) sweeps32(h, op, n, how);
         else sweeps64(h, op, umt, n);
         CK(h, cudaEventRecord(h->ev[1], h->stream));
         if (df) {
@@ -1055,13 +1165,14 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
     r.check_ms = check_ms;
     r.time_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0)
                     .count();
-    if (use_tb) {
+    if (use_tb || use_res) {
         unsigned int bad = 0;
         CK(h, cudaMemcpyAsync(&bad, tb_err_word(h), sizeof bad, cudaMemcpyDeviceToHost,
                               h->stream));
         CK(h, cudaStreamSynchronize(h->stream));
         if (bad) {
-            set_err(h, "a TMA stage of the two-sweep kernel did not arrive in time");
+            set_err(h, use_res ? "a neighbour's word of the resident sweeps did not arrive in time"
+                               : "a TMA stage of the two-sweep kernel did not arrive in time");
             st = RFB_ERR_CUDA;
         }
     }
@@ -1085,7 +1196,8 @@ void free_all(rfb_soc_handle* h) {
     // the arena holds flags .. partials; the rest are allocated on first use
     void* ptrs[] = {h->d_arena, h->d_m,    h->d_m32,  h->d_lam[0], h->d_lam[1], h->d_g,
                     h->d_grad,  h->d_L64,  h->d_L2F,  h->d_eta,    h->d_elec,   h->d_sdf[0],
-                    h->d_sdf[1], h->d_gdf,  h->d_stage,  h->d_bv,     h->d_bvpart};
+                    h->d_sdf[1], h->d_gdf,  h->d_stage,  h->d_bv,     h->d_bvpart,
+                    h->d_inbox};
     for (void* p : ptrs)   // back to the pool, in the handle's stream order
         if (p) cudaFreeAsync(p, h->stream);
     cudaStreamSynchronize(h->stream);
@@ -2227,7 +2339,8 @@ rfb_status rfb_soc_tuned_fp32_kernel(const rfb_soc_handle* h, int32_t* kernel,
                                      double* blocked_ms_per_sweep) {
     if (!h) return RFB_ERR_INVALID_ARG;
     int32_t k = 0;
-    if (h->tb_mode == 0) k = 1;
+    if (h->res_used) k = 11;
+    else if (h->tb_mode == 0) k = 1;
     else if (h->tb_mode == 1 || h->tb_variant >= 0) {
         const int v = std::max(h->tb_variant, 0);
         k = (v & 4 ? (v & 2 ? 9 : 7) : (v & 2 ? 5 : 3)) + (v & 1);

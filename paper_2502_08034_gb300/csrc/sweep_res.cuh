@@ -1,0 +1,287 @@
+// FP32 correction sweeps of a lattice that fits on the chip (local steps): one launch
+// applies all the sweeps of a correction cycle.
+//
+// What bounds a small lattice is not its traffic but the fixed cost of a launch and the
+// latency of one dependent round through L2 per sweep: one launch per sweep takes 6.1 us on
+// every lattice from 16x16x32 to 92x92x100 (the rate at which the host can launch), of which a
+// 64^3 lattice's traffic is 1.1 us. Here the lattice is cut into bricks of bx x by columns
+// and CPT planes, one per CTA of a cooperative launch (all resident together). A thread owns
+// a column of CPT cells and keeps their weights a_f, dt r and values in registers for the
+// whole cycle; z neighbours are its own registers, x and y neighbours come from a
+// double-buffered copy of the brick in shared memory. Only faces travel: after each sweep a
+// CTA stores the new values of its faces into its neighbours' inboxes in global memory, each
+// as one 64-bit word (value, sweep tag), and polls its own inbox for the words of that
+// sweep. Value and tag arrive together (one 64-bit access), so a sweep costs one
+// store-to-load latency and one block barrier instead of a launch, with no fence and no
+// grid-wide barrier.
+//
+// Inboxes have two slots (sweep parity). A CTA overwrites the slot of sweep v with sweep
+// v + 2 only after it computed v + 2, which needed the neighbour's words of v + 1, and the
+// neighbour sends those after the barrier that follows its reads of v (the z faces pair
+// thread with thread and need no barrier). Tags grow from launch to launch (the handle keeps
+// the count), so a slot is never cleared.
+//
+// Every update is dt_coef and dt_update with the operands and the order of the one-sweep
+// kernel, so n sweeps here are bitwise n launches of sweep32d_kernel.
+//
+// Measured (us per sweep in cycles of 200; launches before, resident now): 16x16x32 6.2 and
+// 0.83, 64^3 6.2 and 1.28, 80x60x110 6.2 and 1.91. About 0.75 us of it is the word latency
+// (the smallest lattices); the rest is the shared-memory and issue time of a CTA's cells.
+#pragma once
+
+#include "sweep_dt.cuh"
+
+namespace rfb {
+
+constexpr int RES_T = 512;         // threads of a CTA: at most bx * by = 512 columns
+constexpr int RES_RING = 2;        // pairs of x / y halo words polled per thread, at most
+// Shared memory of one plane of the brick: its rows without padding, one row below and one
+// above (a column's index is its thread's, so a warp's accesses never share a bank), then as
+// much again for the columns left and right of the brick, each at its neighbour's index (the
+// bank that its reader leaves free). With padded rows of bx + 2 every access of a warp that
+// spans two rows took two turns: 528k cells 1.96 us a sweep. The pitch is fixed, so that a
+// column's cells are immediate offsets and take no address registers.
+constexpr int RES_ROWS = 640;      // bx * (by + 2) at most
+constexpr int RES_PLANE = 2 * RES_ROWS;
+// polls of one wait before it gives up (each a round trip to L2: about a second)
+constexpr unsigned RES_SPIN_LIMIT = 1u << 21;
+
+struct ResArgs {
+    int nx, ny, nz;
+    int bx, by;                    // columns of a brick (its planes: CPT)
+    int gx, gy, gz;                // bricks
+    const float* __restrict__ u;   // FP32 face velocities * beta / h (low faces)
+    const float* __restrict__ v;
+    const float* __restrict__ w;   // nz + 1 planes
+    const float* __restrict__ dt;  // per-cell step (0: not updated)
+    const float* __restrict__ r;   // forcing
+    const float* __restrict__ in;  // delta before the first sweep (nullptr: 0 everywhere)
+    float* __restrict__ out;       // delta after the last sweep (another buffer than `in`)
+    float omc, Dh;
+    int n;                         // sweeps
+    uint32_t tag;                  // the words of sweep v carry tag + v
+    unsigned long long* inbox;     // CTAs x 2 slots x stride words
+    int stride;
+    unsigned int* err;             // set if a neighbour's word never arrives
+};
+
+// words of one inbox slot: the z faces, then the x and y faces
+__host__ __device__ constexpr int res_stride(int cpt, int bx, int by) {
+    return 2 * RES_T + 2 * cpt * (bx + by);
+}
+// From ten cells a column dt r is kept in shared memory (its own words only): the weights of
+// ten or twelve cells and dt r spill at 128 registers a thread (148 bytes at twelve).
+__host__ __device__ constexpr bool res_dtr_shared(int cpt) { return cpt >= 10; }
+// bytes of the two copies of a brick and its ring of neighbour columns, then dt r
+__host__ __device__ constexpr int res_smem(int cpt) {
+    return (2 * cpt * RES_PLANE + (res_dtr_shared(cpt) ? cpt * RES_T : 0)) * (int)sizeof(float);
+}
+
+__device__ __forceinline__ void res_send(unsigned long long* p, float x, uint32_t tag) {
+    const unsigned long long word = ((unsigned long long)tag << 32) | __float_as_uint(x);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(word) : "memory");
+}
+// two words of a column's neighbouring cells (each 64-bit word by itself is whole)
+__device__ __forceinline__ void res_send2(unsigned long long* p, float x, float y, uint32_t tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p),
+                 "l"(t | __float_as_uint(x)), "l"(t | __float_as_uint(y))
+                 : "memory");
+}
+__device__ __forceinline__ unsigned long long res_peek(const unsigned long long* p) {
+    unsigned long long word;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(p) : "memory");
+    return word;
+}
+
+__device__ __forceinline__ void res_peek2(const unsigned long long* p,
+                                          unsigned long long (&w)[2]) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
+                 : "=l"(w[0]), "=l"(w[1])
+                 : "l"(p)
+                 : "memory");
+}
+
+template <int CPT, bool TR>   // CPT even
+__global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
+    extern __shared__ float res_s[];
+    const int t = threadIdx.x;
+    const int bx = A.bx, by = A.by;
+    constexpr int plane = RES_PLANE, copy = CPT * RES_PLANE;
+    const int b = blockIdx.x;
+    const int ix = b % A.gx, iy = (b / A.gx) % A.gy, iz = b / (A.gx * A.gy);
+    const int x = t % bx, y = t / bx;
+    const bool mine = y < by;                          // owns a column
+    const int i = ix * bx + x, j = iy * by + y, k0 = iz * CPT;
+    for (int q = t; q < 2 * copy; q += RES_T) res_s[q] = 0.f;
+
+    // weights of the column (a cell outside the lattice has none: it stays 0)
+    constexpr bool DTR_S = res_dtr_shared(CPT);
+    CoefD kc[CPT];
+    float dtr[DTR_S ? 1 : CPT], d[CPT];
+    float* const dtr_s = res_s + 2 * copy + t;
+    const int64_t nxny = (int64_t)A.nx * A.ny;
+    const int64_t c0 = i + (int64_t)A.nx * j + nxny * k0;
+    const bool in_xy = mine && i < A.nx && j < A.ny;
+#pragma unroll
+    for (int e = 0; e < CPT; ++e) {
+        const bool in = in_xy && k0 + e < A.nz;
+        const int64_t c = c0 + nxny * e;
+        const float dt = in ? __ldg(A.dt + c) : 0.f;
+        const float uL = in ? __ldg(A.u + c) : 0.f;
+        const float uH = in && i + 1 < A.nx ? __ldg(A.u + c + 1) : 0.f;
+        const float vL = in ? __ldg(A.v + c) : 0.f;
+        const float vH = in && j + 1 < A.ny ? __ldg(A.v + c + A.nx) : 0.f;
+        const float wL = in ? __ldg(A.w + c) : 0.f;
+        const float wH = in ? __ldg(A.w + c + nxny) : 0.f;
+        kc[e] = dt_coef<TR>(dt, A.Dh, uL, uH, vL, vH, wL, wH);
+        const float f = dt * (in ? __ldg(A.r + c) : 0.f);
+        if (DTR_S) dtr_s[e * RES_T] = f;
+        else dtr[DTR_S ? 0 : e] = f;
+        d[e] = in && A.in ? __ldg(A.in + c) : 0.f;
+    }
+
+    // halo words of this thread: the two z faces of its column (bits 0 and 1 of `want`, set
+    // where there is a neighbour) and up to RES_RING pairs of the x and y faces (bits 2, ..)
+    const int nfx = CPT * by, nfy = CPT * bx;          // words of one x face, one y face (a
+                                                       // column's CPT words together)
+    uint32_t want = 0;
+    if (mine && iz > 0) want |= 1u;
+    if (mine && iz + 1 < A.gz) want |= 2u;
+    int dst[RES_RING];
+#pragma unroll
+    for (int m = 0; m < RES_RING; ++m) {
+        int q = 2 * (t + m * RES_T);
+        dst[m] = 0;
+        if (q >= 2 * (nfx + nfy)) continue;
+        if (q < 2 * nfx) {
+            const bool hi = q >= nfx;
+            if (hi) q -= nfx;
+            dst[m] = (q % CPT) * plane + RES_ROWS + (q / CPT + 1) * bx + (hi ? bx : -1);
+            if (hi ? ix + 1 < A.gx : ix > 0) want |= 4u << m;
+        } else {
+            q -= 2 * nfx;
+            const bool hi = q >= nfy;
+            if (hi) q -= nfy;
+            dst[m] = (q % CPT) * plane + (hi ? by + 1 : 0) * bx + q / CPT;
+            if (hi ? iy + 1 < A.gy : iy > 0) want |= 4u << m;
+        }
+    }
+    // words this column sends to, from slot 0 (-1: no neighbour there; a brick is at least
+    // two columns wide each way, so a column is on one x face and one y face at most)
+    auto box = [&](int c) { return c * 2 * A.stride; };
+    const int own = box(b);
+    int to_zm = -1, to_zp = -1, to_x = -1, to_y = -1;
+    if (mine) {
+        if (iz > 0) to_zm = box(b - A.gx * A.gy) + RES_T + t;
+        if (iz + 1 < A.gz) to_zp = box(b + A.gx * A.gy) + t;
+        if (x == 0 && ix > 0) to_x = box(b - 1) + 2 * RES_T + nfx + y * CPT;
+        if (x == bx - 1 && ix + 1 < A.gx) to_x = box(b + 1) + 2 * RES_T + y * CPT;
+        if (y == 0 && iy > 0) to_y = box(b - A.gx) + 2 * RES_T + 2 * nfx + nfy + x * CPT;
+        if (y == by - 1 && iy + 1 < A.gy) to_y = box(b + A.gx) + 2 * RES_T + 2 * nfx + x * CPT;
+    }
+    const int o = bx + t;                              // this column in a plane, its x neighbours
+    const int oxm = x == 0 ? RES_ROWS + o - 1 : o - 1;
+    const int oxp = x == bx - 1 ? RES_ROWS + o + 1 : o + 1;
+    float zlo = 0.f, zhi = 0.f;                        // values below and above the column
+    bool good = true;
+    __syncthreads();
+    if (A.in) {                                        // the brick and its ring before sweep 1
+        if (in_xy && k0 > 0) zlo = __ldg(A.in + c0 - nxny);
+        if (in_xy && k0 + CPT < A.nz) zhi = __ldg(A.in + c0 + nxny * CPT);
+        for (int q = t; q < copy; q += RES_T) {
+            // row yy of the brick (0: the row below it); the second half of a plane holds the
+            // columns left (index -1 of row yy) and right (index bx) of the brick
+            const int e = q / plane, p = q % plane, r = p % RES_ROWS;
+            int yy = r / bx, xx = r % bx;
+            if (p >= RES_ROWS) {
+                if (xx == bx - 1) { ++yy; xx = -1; }
+                else if (xx == 0) { --yy; xx = bx; }
+                else continue;
+                if (yy < 1 || yy > by) continue;
+            }
+            const int gi = ix * bx + xx, gj = iy * by + yy - 1, gk = k0 + e;
+            if (yy < by + 2 && gi >= 0 && gi < A.nx && gj >= 0 && gj < A.ny && gk < A.nz)
+                res_s[q] = __ldg(A.in + gi + (int64_t)A.nx * gj + nxny * gk);
+        }
+        __syncthreads();
+    }
+    for (int ver = 1; ver <= A.n; ++ver) {
+        const float* Sr = res_s + ((ver - 1) & 1) * copy;       // the brick before this sweep
+        float* Sh = res_s + (ver & 1) * copy;                   // and after
+        float* Sw = Sh + o;
+        const uint32_t tag = A.tag + (uint32_t)ver;
+        unsigned long long* const slot = A.inbox + (ver & 1) * A.stride;
+        const bool more = ver < A.n;
+        if (mine) {
+            // every value first (loads and arithmetic of the cells overlap), then the words,
+            // then the brick's copy
+            float prev = zlo;
+#pragma unroll
+            for (int e = 0; e < CPT; ++e) {
+                const int q = e * plane;
+                const float val = dt_update(
+                    kc[e], A.omc, d[e], DTR_S ? dtr_s[e * RES_T] : dtr[DTR_S ? 0 : e], Sr[q + oxm],
+                    Sr[q + oxp], Sr[q + o - bx], Sr[q + o + bx], prev, e + 1 < CPT ? d[e + 1 < CPT ? e + 1 : e] : zhi);
+                prev = d[e];
+                d[e] = val;
+            }
+            if (more) {
+                if (to_zm >= 0) res_send(slot + to_zm, d[0], tag);
+                if (to_zp >= 0) res_send(slot + to_zp, d[CPT - 1], tag);
+                if (to_x >= 0) {
+#pragma unroll
+                    for (int e = 0; e < CPT; e += 2) res_send2(slot + to_x + e, d[e], d[e + 1], tag);
+                }
+                if (to_y >= 0) {
+#pragma unroll
+                    for (int e = 0; e < CPT; e += 2) res_send2(slot + to_y + e, d[e], d[e + 1], tag);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < CPT; ++e) Sw[e * plane] = d[e];
+        }
+        if (!more) break;
+        // wait for the neighbours' words of this sweep
+        uint32_t pend = good ? want : 0u;
+        const unsigned long long* in = slot + own;
+        for (unsigned spin = 0; pend; ++spin) {
+            unsigned long long zw[2], word[RES_RING][2];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+                if (pend & (1u << m)) zw[m] = res_peek(in + t + m * RES_T);
+#pragma unroll
+            for (int m = 0; m < RES_RING; ++m)
+                if (pend & (4u << m)) res_peek2(in + 2 * RES_T + 2 * (t + m * RES_T), word[m]);
+            if ((pend & 1u) && (uint32_t)(zw[0] >> 32) == tag) {
+                zlo = __uint_as_float((uint32_t)zw[0]);
+                pend &= ~1u;
+            }
+            if ((pend & 2u) && (uint32_t)(zw[1] >> 32) == tag) {
+                zhi = __uint_as_float((uint32_t)zw[1]);
+                pend &= ~2u;
+            }
+#pragma unroll
+            for (int m = 0; m < RES_RING; ++m)
+                if ((pend & (4u << m)) && (uint32_t)(word[m][0] >> 32) == tag &&
+                    (uint32_t)(word[m][1] >> 32) == tag) {
+                    Sh[dst[m]] = __uint_as_float((uint32_t)word[m][0]);
+                    Sh[dst[m] + plane] = __uint_as_float((uint32_t)word[m][1]);
+                    pend &= ~(4u << m);
+                }
+            if (pend && spin >= RES_SPIN_LIMIT) {      // give up, and wait no more
+                atomicExch(A.err, 1u);
+                good = false;
+                break;
+            }
+        }
+        __syncthreads();
+    }
+    if (in_xy) {
+#pragma unroll
+        for (int e = 0; e < CPT; ++e)
+            if (k0 + e < A.nz) A.out[c0 + nxny * e] = d[e];
+    }
+}
+
+}  // namespace rfb

@@ -398,10 +398,11 @@ class Solver:
         return int(lib().rfb_soc_kernel_launches(self.h))
 
     def tuned_fp32_kernel(self):
-        """(name, plain ms/sweep, blocked ms/sweep) chosen by the autotuner."""
+        """(name, plain ms/sweep, blocked ms/sweep) chosen by the autotuner ("resident":
+        the lattice fits on the chip and nothing was timed)."""
         k, a, b = c_int32(), c_double(), c_double()
         self._check(lib().rfb_soc_tuned_fp32_kernel(self.h, byref(k), byref(a), byref(b)))
-        names = {0: None, 1: "plain"}
+        names = {0: None, 1: "plain", 11: "resident"}
         names.update({v: k for k, v in FP32_KERNEL.items() if v >= 3})
         return names[k.value], a.value, b.value
 
