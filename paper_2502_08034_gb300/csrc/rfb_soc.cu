@@ -69,7 +69,7 @@ struct rfb_soc_handle {
     float* d_dtc = nullptr;
     double* d_partials = nullptr;
     double* d_red = nullptr;
-    double* h_red = nullptr;                // pinned, NRED doubles
+    double* h_red = nullptr;                // pinned: NRED doubles and the wait error word
     unsigned long long* d_err = nullptr;
     int s_cur = 0, t_cur = 0;
     bool have_state = false;
@@ -136,15 +136,15 @@ struct rfb_soc_handle {
     CUtensorMap tm_delta[2], tm_r, tm_u, tm_v, tm_w, tm_f, tm_t;
     float* tm_delta_ptr[2] = {nullptr, nullptr};
     double tb_tuned_plain_ms = 0, tb_tuned_tb_ms = 0;
-    // resident FP32 sweeps (sweep_res.cuh): bricks of the lattice, inboxes (first use), the
-    // tag of the next launch's words
+    // resident sweeps (sweep_res.cuh), FP32 and FP64: bricks of the lattice, inboxes (first
+    // use), the tag of the next launch's words
     struct ResPlan {
         int cpt = -1;             // planes of a brick; 0 the lattice does not fit, -1 not planned
         int bx = 0, by = 0, gx = 0, gy = 0, gz = 0;
-    } res;
+        unsigned long long* inbox = nullptr;
+        uint32_t tag = 0;
+    } res, res64;
     bool res_used = false;        // the last FP32 correction sweeps were resident ones
-    unsigned long long* d_inbox = nullptr;
-    uint32_t res_tag = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 };
 
@@ -274,12 +274,27 @@ Coef<T> make_coef(const rfb_soc_handle* h, const OpPoint& op, bool correction, b
     return C;
 }
 
+// set by a sweep kernel whose bounded wait gave up; read back with every reduction
+unsigned int* wait_err_word(rfb_soc_handle* h) {
+    return reinterpret_cast<unsigned int*>(h->d_err + 3);
+}
+
 void reduce_readback(rfb_soc_handle* h, int min_slot0) {
-    finalize_kernel<<<1, 256, 0, h->stream>>>(h->d_partials, h->nblocks, h->d_red, min_slot0);
+    finalize_kernel<<<1, 256, 0, h->stream>>>(h->d_partials, h->nblocks, h->d_red, min_slot0,
+                                              wait_err_word(h));
     LAUNCHED(h);
-    CK(h, cudaMemcpyAsync(h->h_red, h->d_red, NRED * sizeof(double), cudaMemcpyDeviceToHost,
-                          h->stream));
+    CK(h, cudaMemcpyAsync(h->h_red, h->d_red, (NRED + 1) * sizeof(double),
+                          cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
+}
+
+// After a reduction: whether a bounded wait of the sweeps before it gave up (a TMA stage of a
+// pass, or a neighbour's word of the resident sweeps); the word is cleared for the next call.
+bool wait_gave_up(rfb_soc_handle* h) {
+    if (h->h_red[NRED] == 0.0) return false;
+    CK(h, cudaMemsetAsync(wait_err_word(h), 0, sizeof(unsigned int), h->stream));
+    set_err(h, "the sweep kernel waited too long for a TMA stage or for a neighbour's values");
+    return true;
 }
 
 // Face velocities times beta / h (FP64 and FP32 copies) for the velocity scale beta;
@@ -454,6 +469,96 @@ void check_df(rfb_soc_handle* h, const OpPoint& op, bool umt, bool fuse) {
     reduce_readback(h, 0);
 }
 
+// ---- resident sweeps (sweep_res.cuh)
+
+// The cut of the lattice into at most one brick per SM (cpt 0 if there is none) with the least
+// work per sweep in its fullest CTA: whole warps of columns times planes, and a little for
+// the side faces. ring: values of the side faces a CTA can poll.
+void res_plan(rfb_soc_handle* h, rfb_soc_handle::ResPlan& P, const std::vector<int>& cpts,
+              int ring_most) {
+    if (P.cpt >= 0) return;
+    P.cpt = 0;
+    int sms = 0, coop = 0;
+    CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    CK(h, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
+    if (!coop) return;
+    double best = INFINITY;
+    for (int gx = 1; gx <= std::min(h->nx / 2, sms); ++gx) {
+        const int bx = (h->nx + gx - 1) / gx;
+        if ((h->nx + bx - 1) / bx != gx || bx > 64) continue;
+        for (int gy = 1; gy <= std::min(h->ny / 2, sms / gx); ++gy) {
+            const int by = (h->ny + gy - 1) / gy;
+            if ((h->ny + by - 1) / by != gy || bx * by > RES_T || bx * (by + 2) > RES_ROWS) continue;
+            for (int cpt : cpts) {
+                const int gz = (h->nz + cpt - 1) / cpt;
+                const int ring = 2 * cpt * (bx + by);
+                if (gx * gy * gz > sms || ring > ring_most) continue;
+                const double cost = 5.0 * cpt * ((bx * by + 31) / 32) + 0.25 * ring;
+                if (cost < best) {
+                    best = cost;
+                    P.cpt = cpt;
+                    P.bx = bx; P.by = by;
+                    P.gx = gx; P.gy = gy; P.gz = gz;
+                }
+            }
+        }
+    }
+}
+
+template <bool ADJ>
+void (*res64_kernel(int cpt))(Res64Args) {
+    switch (cpt) {
+        case 2: return sweep64r_kernel<2, ADJ>;
+        case 3: return sweep64r_kernel<3, ADJ>;
+        case 4: return sweep64r_kernel<4, ADJ>;
+        case 5: return sweep64r_kernel<5, ADJ>;
+        default: return sweep64r_kernel<6, ADJ>;
+    }
+}
+
+// The resident FP64 sweeps are the faster ones wherever the lattice fits (up to about 0.46 M
+// cells): 7.9 us a sweep at 396k cells, where launches take 12.3.
+bool res64_fits(rfb_soc_handle* h) {
+    res_plan(h, h->res64, {2, 3, 4, 5, 6}, RES64_RING * RES_T);
+    return h->res64.cpt > 0;
+}
+
+// n FP64 sweeps from buf[cur] (adjoint: transposed steps with source g), 2048 a launch; the
+// result is left in buf[cur]
+void res64_sweeps(rfb_soc_handle* h, const OpPoint& op, double** buf, int& cur, int64_t n,
+                  const double* g) {
+    auto& P = h->res64;
+    Res64Args A{};
+    A.L = lattice(h);
+    A.bx = P.bx; A.by = P.by;
+    A.gx = P.gx; A.gy = P.gy; A.gz = P.gz;
+    A.K = h->K;
+    A.dtc = op.dt_mode == RFB_DT_LOCAL ? h->d_dtc : nullptr;
+    A.dt = op.dt;
+    A.g = g;
+    A.umt = op.umt;
+    A.err = wait_err_word(h);
+    A.stride = res64_stride(P.cpt, P.bx, P.by);
+    const int ctas = P.gx * P.gy * P.gz;
+    if (!P.inbox) dalloc(h, &P.inbox, (size_t)ctas * 4 * A.stride);
+    A.inbox = P.inbox;
+    const auto k = g ? res64_kernel<true>(P.cpt) : res64_kernel<false>(P.cpt);
+    const int smem = res64_smem(P.cpt);
+    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    for (int64_t q = 0; q < n; q += A.n) {
+        A.n = (int)std::min<int64_t>(n - q, 2048);
+        A.in = buf[cur];
+        A.out = buf[cur ^ 1];
+        A.tag = P.tag;
+        P.tag += (uint32_t)A.n;
+        void* args[] = {&A};
+        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(RES_T), args, smem,
+                                          h->stream));
+        ++h->launches;
+        cur ^= 1;
+    }
+}
+
 // n FP64 sweeps on s (or t for U_mt), ping-pong, with the assembled operator
 void sweeps64(rfb_soc_handle* h, const OpPoint& op, bool umt, int64_t n) {
     double** buf = umt ? h->d_t : h->d_s;
@@ -462,6 +567,10 @@ void sweeps64(rfb_soc_handle* h, const OpPoint& op, bool umt, int64_t n) {
     const float* dtc = op.dt_mode == RFB_DT_LOCAL ? h->d_dtc : nullptr;
     Lattice L = lattice(h);
     const Coef<double> C = make_coef<double>(h, op, false, false);
+    if (!C.nl && n > 1 && res64_fits(h)) {
+        res64_sweeps(h, op, buf, cur, n, nullptr);
+        return;
+    }
     for (int64_t q = 0; q < n; ++q) {
         if (C.nl)
             sweep64c_kernel<true><<<h->grid, h->block, 0, h->stream>>>(
@@ -595,8 +704,6 @@ void tb_prepare(rfb_soc_handle* h) {
     h->tm_ready = true;
 }
 
-unsigned int* tb_err_word(rfb_soc_handle* h) { return reinterpret_cast<unsigned int*>(h->d_err + 3); }
-
 // sweeps of one pass of the chosen variant
 int tb_depth(const rfb_soc_handle* h) { return h->tb_variant >= 4 ? 3 : 2; }
 
@@ -616,7 +723,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
         A.d_out = h->d_delta[cur ^ 1];
         A.omc = (float)(1.0 - op.cfl);
         A.Dh = C.Dh;
-        A.err = tb_err_word(h);
+        A.err = wait_err_word(h);
         const bool four = (v & 2) != 0;
         if (v >= 4) {
             if (tr && four)
@@ -657,7 +764,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
     A.d_out = h->d_delta[cur ^ 1];
     A.Dh = C.Dh; A.gDh = C.gDh; A.dt = C.dt; A.cfl = (float)op.cfl; A.umt = C.umt;
     for (int q = 0; q < 8; ++q) A.tB[q] = C.rB[q];
-    A.err = tb_err_word(h);
+    A.err = wait_err_word(h);
     if (local)
         sweep32tb_kernel<true><<<S.grid, TB_THREADS, TB_SMEM, h->stream>>>(
             td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_f, A);
@@ -703,7 +810,7 @@ void swap_delta(rfb_soc_handle* h) {
     }
 }
 
-// ---- resident sweeps (sweep_res.cuh)
+// ---- resident FP32 sweeps
 
 using ResKernel = void (*)(ResArgs);
 template <bool TR>
@@ -718,45 +825,17 @@ ResKernel res_kernel(int cpt) {
     }
 }
 
-// Whether the resident sweeps take this lattice: its bricks, one per SM, are all on the chip
-// at once (up to about 0.9 M cells). They are the faster ones wherever they fit: 1.9 us a
-// sweep at 528k cells, where launches and passes take 6.2 us. Among the cuts that fit, the one with the least shared-memory work per sweep (the
-// word latency is the same for all).
+// The resident FP32 sweeps are the faster ones wherever the lattice fits (up to about 0.9 M
+// cells): 1.9 us a sweep at 528k cells, where launches and passes take 6.2 us.
 bool res_fits(rfb_soc_handle* h) {
-    if (h->res.cpt >= 0) return h->res.cpt > 0;
-    h->res.cpt = 0;
-    int sms = 0, coop = 0;
-    CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-    CK(h, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
-    if (!coop) return false;
-    double best = INFINITY;
-    for (int gx = 1; gx <= std::min(h->nx / 2, sms); ++gx) {
-        const int bx = (h->nx + gx - 1) / gx;
-        if ((h->nx + bx - 1) / bx != gx) continue;
-        for (int gy = 1; gy <= std::min(h->ny / 2, sms / gx); ++gy) {
-            const int by = (h->ny + gy - 1) / gy;
-            if ((h->ny + by - 1) / by != gy || bx * by > RES_T ||
-                bx > 64 || bx * (by + 2) > RES_ROWS)
-                continue;
-            for (int cpt : {2, 4, 6, 8, 10, 12}) {
-                const int gz = (h->nz + cpt - 1) / cpt;
-                const int ring = 2 * cpt * (bx + by);
-                if (gx * gy * gz > sms || ring > 2 * RES_RING * RES_T) continue;
-                const double cost = 5.0 * cpt * ((bx * by + 31) / 32) + 0.25 * ring;
-                if (cost < best) {
-                    best = cost;
-                    h->res = {cpt, bx, by, gx, gy, gz};
-                }
-            }
-        }
-    }
+    res_plan(h, h->res, {2, 4, 6, 8, 10, 12}, 2 * RES_RING * RES_T);
     return h->res.cpt > 0;
 }
 
 // n sweeps (tr: of the transposed operator) from delta = 0; the result is left in d_delta[0].
 // One launch does them all, or 4096 at a time (a launch of some ms).
 void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n, bool tr) {
-    const auto& P = h->res;
+    auto& P = h->res;
     ResArgs A{};
     A.nx = h->nx; A.ny = h->ny; A.nz = h->nz;
     A.bx = P.bx; A.by = P.by;
@@ -765,11 +844,11 @@ void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int6
     A.r = h->d_r32;
     A.omc = (float)(1.0 - op.cfl);
     A.Dh = C.Dh;
-    A.err = tb_err_word(h);
+    A.err = wait_err_word(h);
     A.stride = res_stride(P.cpt, P.bx, P.by);
     const int ctas = P.gx * P.gy * P.gz;
-    if (!h->d_inbox) dalloc(h, &h->d_inbox, (size_t)ctas * 2 * A.stride);
-    A.inbox = h->d_inbox;
+    if (!P.inbox) dalloc(h, &P.inbox, (size_t)ctas * 2 * A.stride);
+    A.inbox = P.inbox;
     const ResKernel k = tr ? res_kernel<true>(P.cpt) : res_kernel<false>(P.cpt);
     const int smem = res_smem(P.cpt);
     CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -777,8 +856,8 @@ void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int6
         A.n = (int)std::min<int64_t>(n - q, 4096);
         A.in = q ? h->d_delta[0] : nullptr;
         A.out = h->d_delta[q ? 1 : 0];
-        A.tag = h->res_tag;
-        h->res_tag += (uint32_t)A.n;
+        A.tag = P.tag;
+        P.tag += (uint32_t)A.n;
         void* args[] = {&A};
         CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(RES_T), args, smem,
                                           h->stream));
@@ -1072,7 +1151,6 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
             if (h->tb_mode < 0) tune_fp32_kernel(h, op);
             use_tb = h->tb_mode == 1;
         }
-        if (use_tb || use_res) CK(h, cudaMemsetAsync(tb_err_word(h), 0, sizeof(unsigned int), h->stream));
     }
     // sweeps per pass: the default interval and the shortened ones are whole passes
     const int depth = use_tb ? tb_depth(h) : 1;
@@ -1141,6 +1219,7 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
         CK(h, cudaEventElapsedTime(&ms_c, h->ev[1], h->ev[2]));
         sweep_ms += ms_s;
         check_ms += ms_c;
+        if (wait_gave_up(h)) { st = RFB_ERR_CUDA; break; }
         const double res_before = r.residual;
         done += n;
         ++r.checks;
@@ -1165,17 +1244,7 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
     r.check_ms = check_ms;
     r.time_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0)
                     .count();
-    if (use_tb || use_res) {
-        unsigned int bad = 0;
-        CK(h, cudaMemcpyAsync(&bad, tb_err_word(h), sizeof bad, cudaMemcpyDeviceToHost,
-                              h->stream));
-        CK(h, cudaStreamSynchronize(h->stream));
-        if (bad) {
-            set_err(h, use_res ? "a neighbour's word of the resident sweeps did not arrive in time"
-                               : "a TMA stage of the two-sweep kernel did not arrive in time");
-            st = RFB_ERR_CUDA;
-        }
-    }
+    if (wait_gave_up(h)) st = RFB_ERR_CUDA;
     if (res) *res = r;
     return st;
 }
@@ -1197,7 +1266,7 @@ void free_all(rfb_soc_handle* h) {
     void* ptrs[] = {h->d_arena, h->d_m,    h->d_m32,  h->d_lam[0], h->d_lam[1], h->d_g,
                     h->d_grad,  h->d_L64,  h->d_L2F,  h->d_eta,    h->d_elec,   h->d_sdf[0],
                     h->d_sdf[1], h->d_gdf,  h->d_stage,  h->d_bv,     h->d_bvpart,
-                    h->d_inbox};
+                    h->res.inbox, h->res64.inbox};
     for (void* p : ptrs)   // back to the pool, in the handle's stream order
         if (p) cudaFreeAsync(p, h->stream);
     cudaStreamSynchronize(h->stream);
@@ -1324,7 +1393,7 @@ rfb_status rfb_soc_create(const int32_t dims[3], double dx, const uint8_t* fiber
                 {(void**)&h->d_delta[0], n4}, {(void**)&h->d_delta[1], n4},
                 {(void**)&h->d_r32, n4}, {(void**)&h->d_dtc, n4},
                 {(void**)&h->d_err, 4 * sizeof(unsigned long long)},
-                {(void**)&h->d_red, NRED * sizeof(double)},
+                {(void**)&h->d_red, (NRED + 1) * sizeof(double)},
                 {(void**)&h->d_partials, (size_t)h->nblocks * NRED * sizeof(double)}};
             auto up = [](size_t b) { return (b + 255) / 256 * 256; };
             size_t total = 0;
@@ -1336,7 +1405,8 @@ rfb_status rfb_soc_create(const int32_t dims[3], double dx, const uint8_t* fiber
                 off += up(q.bytes);
             }
         }
-        CK(h, cudaMallocHost((void**)&h->h_red, NRED * sizeof(double)));
+        CK(h, cudaMallocHost((void**)&h->h_red, (NRED + 1) * sizeof(double)));
+        h->h_red[NRED] = 0.0;
         for (cudaEvent_t& e : h->ev) CK(h, cudaEventCreate(&e));
 
         // staging: the inputs on the device (copied when they are host arrays)
@@ -2202,7 +2272,6 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
                 LAUNCHED(h);
                 check64();
             };
-            CK(h, cudaMemsetAsync(tb_err_word(h), 0, sizeof(unsigned int), h->stream));
             df_check(false);
             bool joined = false;
             while (true) {
@@ -2230,14 +2299,6 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
                 join_and_check();
                 if (!bad && h->h_red[6] > 0) st = RFB_ERR_NONFINITE;
             }
-            unsigned int tb_bad = 0;
-            CK(h, cudaMemcpyAsync(&tb_bad, tb_err_word(h), sizeof tb_bad, cudaMemcpyDeviceToHost,
-                                  h->stream));
-            CK(h, cudaStreamSynchronize(h->stream));
-            if (tb_bad) {
-                set_err(h, "a TMA stage of the two-sweep kernel did not arrive in time");
-                st = RFB_ERR_CUDA;
-            }
         }
         while (!mixed) {
             adjoint64c_kernel<1><<<h->grid, h->block, 0, h->stream>>>(
@@ -2258,7 +2319,9 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
                 break;
             }
             const int64_t n = std::min(every, o.max_sweeps - done);
-            for (int64_t q = 0; q < n; ++q) {
+            const bool resident = res64_fits(h);
+            if (resident) res64_sweeps(h, op, h->d_lam, cur, n, h->d_g);
+            for (int64_t q = 0; q < n && !resident; ++q) {
                 adjoint64c_kernel<0><<<h->grid, h->block, 0, h->stream>>>(
                     lattice(h), h->K, C.dtc, op.dt, h->d_lam[cur], h->d_lam[cur ^ 1], h->d_g,
                     nullptr, op.umt, h->kchunk);
@@ -2275,6 +2338,7 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
             umt ? nullptr : h->d_grad, h->d_partials, h->kchunk);
         LAUNCHED(h);
         reduce_readback(h, 0);
+        if (wait_gave_up(h)) st = RFB_ERR_CUDA;
         double dbeta = jscale * h->h_red[0] / op.beta;
         if (obj == RFB_OBJ_U) dbeta -= fwd.U / op.beta;
         if (umt) CK(h, cudaMemsetAsync(h->d_grad, 0, N * 8, h->stream));

@@ -1501,11 +1501,13 @@ stats_kernel(const uint8_t* __restrict__ flags, const double* __restrict__ w,
 }
 
 // Sum (slots 0..6) / max (slot 7) of the per-block partials, in a fixed order.
-// min_slot0: slot 0 is reduced with min instead of a sum (diag_kernel).
+// min_slot0: slot 0 is reduced with min instead of a sum (diag_kernel). err (nullable): the
+// word of the sweeps' bounded waits, passed on in slot NRED.
 __global__ void __launch_bounds__(256)
 finalize_kernel(const double* __restrict__ partials, int64_t nblocks, double* __restrict__ out,
-                int min_slot0) {
+                int min_slot0, const unsigned int* __restrict__ err = nullptr) {
     __shared__ double sh[256];
+    if (err && threadIdx.x == 0) out[NRED] = (double)*err;
     for (int q = 0; q < NRED; ++q) {
         const bool is_max = (q == NRED - 1);
         const bool is_min = (q == 0 && min_slot0);

@@ -284,4 +284,246 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
     }
 }
 
+// ---------------------------------------------------------------------------------
+// Resident FP64 sweeps with the assembled operator, s <- s + dt RHS(s) (ADJ: the transposed
+// step lam <- lam + dt (L^T lam + g)). The scheme of the FP32 kernel: bricks, columns of CPT
+// cells per thread, faces as tagged words, here two 64-bit words a value (its halves). What
+// bounds it is the FP64 pipe: 8 DFMA a cell at 2 lanes a clock and SM, 2.9 us for 48x48x96,
+// so the whole warps a cut takes decide its time and shared memory costs nothing beside it.
+// Operands and order are those of sweep64c_kernel and adjoint64c_kernel: bitwise the same.
+//
+// Measured (us per sweep, launches before and resident now): 16x16x32 8.2 and 1.6, 32x32x64 8.2
+// and 2.0, 48x48x96 10.3 and 4.6, 64^3 10.2 and 5.7, 60x60x110 12.3 and 7.9.
+// ---------------------------------------------------------------------------------
+constexpr int RES64_RING = 3;      // x / y halo values polled per thread, at most
+// coefficients of a cell kept in shared memory (the last ones; registers hold the others):
+// eight doubles for five or six cells do not fit beside the values at 128 registers
+__host__ __device__ constexpr int res64_shared(int cpt) { return cpt >= 6 ? 3 : cpt >= 5 ? 2 : 0; }
+__host__ __device__ constexpr int res64_smem(int cpt) {
+    return (2 * cpt * RES_PLANE + cpt * res64_shared(cpt) * RES_T) * (int)sizeof(double);
+}
+// 16-byte entries of one inbox slot
+__host__ __device__ constexpr int res64_stride(int cpt, int bx, int by) {
+    return 2 * RES_T + 2 * cpt * (bx + by);
+}
+
+struct Res64Args {
+    Lattice L;
+    int bx, by, gx, gy, gz;        // as in ResArgs
+    L64 K;
+    const float* __restrict__ dtc; // per-cell step, nullptr: dt
+    double dt;
+    const double* __restrict__ in; // before the first sweep
+    double* __restrict__ out;      // after the last (another buffer)
+    const double* __restrict__ g;  // ADJ: the source
+    int umt, n;
+    uint32_t tag;
+    unsigned long long* inbox;     // CTAs x 2 slots x stride entries of two words
+    int stride;
+    unsigned int* err;
+};
+
+__device__ __forceinline__ void res_send64(unsigned long long* p, double x, uint32_t tag) {
+    const unsigned long long t = (unsigned long long)tag << 32, v = __double_as_longlong(x);
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p),
+                 "l"(t | (v & 0xffffffffull)), "l"(t | (v >> 32))
+                 : "memory");
+}
+__device__ __forceinline__ bool res_take64(const unsigned long long (&w)[2], uint32_t tag,
+                                           double* x) {
+    if ((uint32_t)(w[0] >> 32) != tag || (uint32_t)(w[1] >> 32) != tag) return false;
+    *x = __longlong_as_double((long long)((w[0] & 0xffffffffull) | (w[1] << 32)));
+    return true;
+}
+
+template <int CPT, bool ADJ>   // CPT >= 2
+__global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
+    extern __shared__ double res_s64[];
+    constexpr int plane = RES_PLANE, copy = CPT * RES_PLANE;
+    constexpr int NS = res64_shared(CPT), NR = 8 - NS;
+    const int t = threadIdx.x;
+    const int nx = A.L.nx, ny = A.L.ny, nz = A.L.nz;
+    const int bx = A.bx, by = A.by;
+    const int b = blockIdx.x;
+    const int ix = b % A.gx, iy = (b / A.gx) % A.gy, iz = b / (A.gx * A.gy);
+    const int x = t % bx, y = t / bx;
+    const int i = ix * bx + x, j = iy * by + y, k0 = iz * CPT;
+    const int64_t nxny = A.L.nxny, N = nxny * nz;
+    const int64_t c0 = i + (int64_t)nx * j + nxny * k0;
+    // every column of the brick runs (one outside the lattice holds 0 and is not updated),
+    // except whole warps of threads without one
+    const bool mine = y < by;
+    const bool in_xy = mine && i < nx && j < ny;
+
+    // coefficients in the order of use: diagonal, source, then the six neighbours
+    double kr[CPT][NR], d[CPT], dt[CPT];
+    double* const ks = res_s64 + 2 * copy + t;
+    uint32_t upd = 0;
+#pragma unroll
+    for (int e = 0; e < CPT; ++e) {
+        const bool in = in_xy && k0 + e < nz;
+        const int64_t c = c0 + nxny * e;
+        const unsigned f = in ? A.L.flags[c] : 0u;
+        const bool u = (f & F_FLUID) && !(A.umt && (f & F_ELEC));
+        if (u) upd |= 1u << e;
+        double q[8];
+        q[0] = u ? A.K.diag[c] : 0.0;
+        if (ADJ) {   // from each neighbour's row the coefficient that points back here
+            q[1] = u ? A.g[c] : 0.0;
+            q[2] = u && i > 0 ? A.K.f[1][c - 1] : 0.0;
+            q[3] = u && i + 1 < nx ? A.K.f[0][c + 1] : 0.0;
+            q[4] = u && j > 0 ? A.K.f[3][c - nx] : 0.0;
+            q[5] = u && j + 1 < ny ? A.K.f[2][c + nx] : 0.0;
+            q[6] = u && c >= nxny ? A.K.f[5][c - nxny] : 0.0;
+            q[7] = u && c + nxny < N ? A.K.f[4][c + nxny] : 0.0;
+        } else {
+            q[1] = u ? A.K.b[c] : 0.0;
+#pragma unroll
+            for (int m = 0; m < 6; ++m) q[2 + m] = u ? A.K.f[m][c] : 0.0;
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            if (m < NR) kr[e][m < NR ? m : 0] = q[m];
+            else ks[(e * NS + m - NR) * RES_T] = q[m];
+        }
+        dt[e] = u ? (A.dtc ? (double)A.dtc[c] : A.dt) : 0.0;
+        d[e] = in ? A.in[c] : 0.0;
+    }
+    // the brick and the columns around it before the first sweep (0 outside the lattice)
+    for (int q = t; q < 2 * copy; q += RES_T) {
+        const int e = q % copy / plane, p = q % plane, r = p % RES_ROWS;
+        int yy = r / bx, xx = r % bx;
+        bool at = q < copy;
+        if (p >= RES_ROWS) {
+            if (xx == bx - 1) { ++yy; xx = -1; }
+            else if (xx == 0) { --yy; xx = bx; }
+            else at = false;
+            if (yy < 1 || yy > by) at = false;
+        }
+        const int gi = ix * bx + xx, gj = iy * by + yy - 1, gk = k0 + e;
+        at = at && yy < by + 2 && gi >= 0 && gi < nx && gj >= 0 && gj < ny && gk < nz;
+        res_s64[q] = at ? A.in[gi + (int64_t)nx * gj + nxny * gk] : 0.0;
+    }
+    double zlo = in_xy && k0 > 0 ? A.in[c0 - nxny] : 0.0;
+    double zhi = in_xy && k0 + CPT < nz ? A.in[c0 + nxny * CPT] : 0.0;
+
+    const int nfx = CPT * by, nfy = CPT * bx;
+    uint32_t want = 0;
+    if (mine && iz > 0) want |= 1u;
+    if (mine && iz + 1 < A.gz) want |= 2u;
+    int dst[RES64_RING];
+#pragma unroll
+    for (int m = 0; m < RES64_RING; ++m) {
+        int q = t + m * RES_T;
+        dst[m] = 0;
+        if (q >= 2 * (nfx + nfy)) continue;
+        if (q < 2 * nfx) {
+            const bool hi = q >= nfx;
+            if (hi) q -= nfx;
+            dst[m] = (q % CPT) * plane + RES_ROWS + (q / CPT + 1) * bx + (hi ? bx : -1);
+            if (hi ? ix + 1 < A.gx : ix > 0) want |= 4u << m;
+        } else {
+            q -= 2 * nfx;
+            const bool hi = q >= nfy;
+            if (hi) q -= nfy;
+            dst[m] = (q % CPT) * plane + (hi ? by + 1 : 0) * bx + q / CPT;
+            if (hi ? iy + 1 < A.gy : iy > 0) want |= 4u << m;
+        }
+    }
+    auto box = [&](int c) { return c * 2 * A.stride; };
+    const int own = box(b);
+    int to_zm = -1, to_zp = -1, to_x = -1, to_y = -1;
+    if (mine) {
+        if (iz > 0) to_zm = box(b - A.gx * A.gy) + RES_T + t;
+        if (iz + 1 < A.gz) to_zp = box(b + A.gx * A.gy) + t;
+        if (x == 0 && ix > 0) to_x = box(b - 1) + 2 * RES_T + nfx + y * CPT;
+        if (x == bx - 1 && ix + 1 < A.gx) to_x = box(b + 1) + 2 * RES_T + y * CPT;
+        if (y == 0 && iy > 0) to_y = box(b - A.gx) + 2 * RES_T + 2 * nfx + nfy + x * CPT;
+        if (y == by - 1 && iy + 1 < A.gy) to_y = box(b + A.gx) + 2 * RES_T + 2 * nfx + x * CPT;
+    }
+    const int o = bx + t;
+    const int oxm = x == 0 ? RES_ROWS + o - 1 : o - 1;
+    const int oxp = x == bx - 1 ? RES_ROWS + o + 1 : o + 1;
+    bool good = true;
+    __syncthreads();
+    for (int ver = 1; ver <= A.n; ++ver) {
+        const double* Sr = res_s64 + ((ver - 1) & 1) * copy;
+        double* Sh = res_s64 + (ver & 1) * copy;
+        const uint32_t tag = A.tag + (uint32_t)ver;
+        unsigned long long* const slot = A.inbox + 2 * ((ver & 1) * A.stride);
+        const bool more = ver < A.n;
+        if (mine) {
+            auto coef = [&](int e, int m) {
+                return m < NR ? kr[e][m < NR ? m : 0] : ks[(e * NS + m - NR) * RES_T];
+            };
+            auto update = [&](int e, double zm, double zp) {
+                const double* P = Sr + e * plane;
+                double r = fma(coef(e, 0), d[e], coef(e, 1));
+                r = fma(coef(e, 2), P[oxm], r);
+                r = fma(coef(e, 3), P[oxp], r);
+                r = fma(coef(e, 4), P[o - bx], r);
+                r = fma(coef(e, 5), P[o + bx], r);
+                r = fma(coef(e, 6), zm, r);
+                r = fma(coef(e, 7), zp, r);
+                const double val = fma(dt[e], r, d[e]);
+                return (upd >> e) & 1u ? val : d[e];
+            };
+            // the z faces first: their words travel while the other cells are computed
+            const double lo = update(0, zlo, d[1]);
+            if (more && to_zm >= 0) res_send64(slot + 2 * to_zm, lo, tag);
+            const double hi = update(CPT - 1, d[CPT - 2], zhi);
+            if (more && to_zp >= 0) res_send64(slot + 2 * to_zp, hi, tag);
+            double prev = d[0];
+            d[0] = lo;
+#pragma unroll
+            for (int e = 1; e < CPT - 1; ++e) {
+                const double val = update(e, prev, d[e + 1]);
+                prev = d[e];
+                d[e] = val;
+            }
+            d[CPT - 1] = hi;
+            if (more && to_x >= 0) {
+#pragma unroll
+                for (int e = 0; e < CPT; ++e) res_send64(slot + 2 * (to_x + e), d[e], tag);
+            }
+            if (more && to_y >= 0) {
+#pragma unroll
+                for (int e = 0; e < CPT; ++e) res_send64(slot + 2 * (to_y + e), d[e], tag);
+            }
+#pragma unroll
+            for (int e = 0; e < CPT; ++e) Sh[e * plane + o] = d[e];
+        }
+        if (!more) break;
+        uint32_t pend = good ? want : 0u;
+        const unsigned long long* in = slot + 2 * own;
+        for (unsigned spin = 0; pend; ++spin) {
+            unsigned long long word[2 + RES64_RING][2];
+#pragma unroll
+            for (int m = 0; m < 2 + RES64_RING; ++m)
+                if (pend & (1u << m)) res_peek2(in + 2 * (t + m * RES_T), word[m]);
+#pragma unroll
+            for (int m = 0; m < 2 + RES64_RING; ++m) {
+                double val;
+                if ((pend & (1u << m)) && res_take64(word[m], tag, &val)) {
+                    if (m == 0) zlo = val;
+                    else if (m == 1) zhi = val;
+                    else Sh[dst[m >= 2 ? m - 2 : 0]] = val;
+                    pend &= ~(1u << m);
+                }
+            }
+            if (pend && spin >= RES_SPIN_LIMIT) {
+                atomicExch(A.err, 1u);
+                good = false;
+                break;
+            }
+        }
+        __syncthreads();
+    }
+    if (in_xy) {
+#pragma unroll
+        for (int e = 0; e < CPT; ++e)
+            if (k0 + e < nz) A.out[c0 + nxny * e] = d[e];
+    }
+}
+
 }  // namespace rfb
