@@ -115,6 +115,8 @@ struct rfb_soc_handle {
     int kchunk = 8;
     dim3 grid, block;
     int64_t nblocks = 0;
+    int skchunk = 8;          // FP64 sweeps: the same tiles, their own z chunks
+    dim3 sgrid;
     int vkchunk = 8;          // vectorised FP32 sweep (nx % 4 == 0)
     dim3 vgrid, vblock;
     // temporally blocked FP32 sweep (nx % 16 == 0, no area multiplier)
@@ -572,12 +574,10 @@ void sweeps64(rfb_soc_handle* h, const OpPoint& op, bool umt, int64_t n) {
         return;
     }
     for (int64_t q = 0; q < n; ++q) {
-        if (C.nl)
-            sweep64c_kernel<true><<<h->grid, h->block, 0, h->stream>>>(
-                L, h->K, dtc, op.dt, buf[cur], buf[cur ^ 1], op.umt, h->kchunk, C, op.cfl);
-        else
-            sweep64c_kernel<false><<<h->grid, h->block, 0, h->stream>>>(
-                L, h->K, dtc, op.dt, buf[cur], buf[cur ^ 1], op.umt, h->kchunk, C, op.cfl);
+        const auto k = C.nl ? (dtc ? sweep64c_kernel<true, true> : sweep64c_kernel<true, false>)
+                            : (dtc ? sweep64c_kernel<false, true> : sweep64c_kernel<false, false>);
+        k<<<h->sgrid, h->block, 0, h->stream>>>(L, h->K, dtc, op.dt, buf[cur], buf[cur ^ 1],
+                                                op.umt, h->skchunk, C, op.cfl);
         LAUNCHED(h);
         cur ^= 1;
     }
@@ -1369,6 +1369,14 @@ rfb_status rfb_soc_create(const int32_t dims[3], double dx, const uint8_t* fiber
         h->kchunk = kc;
         h->grid = dim3(gx, gy, (nz + kc - 1) / kc);
         h->nblocks = (int64_t)h->grid.x * h->grid.y * h->grid.z;
+        // FP64 sweeps: two planes a block. Their FP64 pipe and memory stream are both near
+        // three quarters of their rates, so what helps is many blocks and an even share per SM
+        // (128x128x256, us per sweep with chunks of 1, 2, 4, 8, 16, 32 planes: 73.8, 69.7,
+        // 71.7, 74.3, 85, 84; 200x192x256: 180, 171, 172, 175, 183, -; 8 before)
+        {
+            h->skchunk = std::max(2, (nz + 65534) / 65535);
+            h->sgrid = dim3(gx, gy, (nz + h->skchunk - 1) / h->skchunk);
+        }
         {
             h->vblock = dim3(VBX, VBY, 1);
             const int vx = (nx / 4 + VBX - 1) / VBX, vy = (ny + VBY - 1) / VBY;
@@ -2322,9 +2330,9 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
             const bool resident = res64_fits(h);
             if (resident) res64_sweeps(h, op, h->d_lam, cur, n, h->d_g);
             for (int64_t q = 0; q < n && !resident; ++q) {
-                adjoint64c_kernel<0><<<h->grid, h->block, 0, h->stream>>>(
+                adjoint64c_kernel<0><<<h->sgrid, h->block, 0, h->stream>>>(
                     lattice(h), h->K, C.dtc, op.dt, h->d_lam[cur], h->d_lam[cur ^ 1], h->d_g,
-                    nullptr, op.umt, h->kchunk);
+                    nullptr, op.umt, h->skchunk);
                 LAUNCHED(h);
                 cur ^= 1;
             }
