@@ -33,7 +33,8 @@
 
 namespace rfb {
 
-constexpr int RES_T = 512;         // threads of a CTA: at most bx * by = 512 columns
+constexpr int RES_T = 512;         // most threads of a CTA, columns of a brick (a launch has
+                                   // the whole warps that its bricks need)
 constexpr int RES_RING = 2;        // pairs of x / y halo words polled per thread, at most
 // Shared memory of one plane of the brick: its rows without padding, one row below and one
 // above (a column's index is its thread's, so a warp's accesses never share a bank), then as
@@ -44,7 +45,7 @@ constexpr int RES_RING = 2;        // pairs of x / y halo words polled per threa
 constexpr int RES_ROWS = 640;      // bx * (by + 2) at most
 constexpr int RES_PLANE = 2 * RES_ROWS;
 // polls of one wait before it gives up (each a round trip to L2: about a second)
-constexpr unsigned RES_SPIN_LIMIT = 1u << 21;
+constexpr unsigned RES_SPIN_LIMIT = 1u << 20;
 
 struct ResArgs {
     int nx, ny, nz;
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
     const int x = t % bx, y = t / bx;
     const bool mine = y < by;                          // owns a column
     const int i = ix * bx + x, j = iy * by + y, k0 = iz * CPT;
-    for (int q = t; q < 2 * copy; q += RES_T) res_s[q] = 0.f;
+    for (int q = t; q < 2 * copy; q += (int)blockDim.x) res_s[q] = 0.f;
 
     // weights of the column (a cell outside the lattice has none: it stays 0)
     constexpr bool DTR_S = res_dtr_shared(CPT);
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
     int dst[RES_RING];
 #pragma unroll
     for (int m = 0; m < RES_RING; ++m) {
-        int q = 2 * (t + m * RES_T);
+        int q = 2 * (t + m * (int)blockDim.x);
         dst[m] = 0;
         if (q >= 2 * (nfx + nfy)) continue;
         if (q < 2 * nfx) {
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
     if (A.in) {                                        // the brick and its ring before sweep 1
         if (in_xy && k0 > 0) zlo = __ldg(A.in + c0 - nxny);
         if (in_xy && k0 + CPT < A.nz) zhi = __ldg(A.in + c0 + nxny * CPT);
-        for (int q = t; q < copy; q += RES_T) {
+        for (int q = t; q < copy; q += (int)blockDim.x) {
             // row yy of the brick (0: the row below it); the second half of a plane holds the
             // columns left (index -1 of row yy) and right (index bx) of the brick
             const int e = q / plane, p = q % plane, r = p % RES_ROWS;
@@ -244,15 +245,17 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
         if (!more) break;
         // wait for the neighbours' words of this sweep
         uint32_t pend = good ? want : 0u;
+        __syncwarp();                  // the warp's own words are sent before it starts polling
         const unsigned long long* in = slot + own;
-        for (unsigned spin = 0; pend; ++spin) {
+        // a warp stays together until all its lanes have their words
+        for (unsigned spin = 0; __any_sync(0xffffffffu, pend != 0u); ++spin) {
             unsigned long long zw[2], word[RES_RING][2];
 #pragma unroll
             for (int m = 0; m < 2; ++m)
                 if (pend & (1u << m)) zw[m] = res_peek(in + t + m * RES_T);
 #pragma unroll
             for (int m = 0; m < RES_RING; ++m)
-                if (pend & (4u << m)) res_peek2(in + 2 * RES_T + 2 * (t + m * RES_T), word[m]);
+                if (pend & (4u << m)) res_peek2(in + 2 * RES_T + 2 * (t + m * (int)blockDim.x), word[m]);
             if ((pend & 1u) && (uint32_t)(zw[0] >> 32) == tag) {
                 zlo = __uint_as_float((uint32_t)zw[0]);
                 pend &= ~1u;
@@ -269,10 +272,10 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
                     Sh[dst[m] + plane] = __uint_as_float((uint32_t)word[m][1]);
                     pend &= ~(4u << m);
                 }
-            if (pend && spin >= RES_SPIN_LIMIT) {      // give up, and wait no more
+            if (spin >= RES_SPIN_LIMIT && pend) {      // give up, and wait no more
                 atomicExch(A.err, 1u);
                 good = false;
-                break;
+                pend = 0;
             }
         }
         __syncthreads();
@@ -390,7 +393,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
         d[e] = in ? A.in[c] : 0.0;
     }
     // the brick and the columns around it before the first sweep (0 outside the lattice)
-    for (int q = t; q < 2 * copy; q += RES_T) {
+    for (int q = t; q < 2 * copy; q += (int)blockDim.x) {
         const int e = q % copy / plane, p = q % plane, r = p % RES_ROWS;
         int yy = r / bx, xx = r % bx;
         bool at = q < copy;
@@ -414,7 +417,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
     int dst[RES64_RING];
 #pragma unroll
     for (int m = 0; m < RES64_RING; ++m) {
-        int q = t + m * RES_T;
+        int q = t + m * (int)blockDim.x;
         dst[m] = 0;
         if (q >= 2 * (nfx + nfy)) continue;
         if (q < 2 * nfx) {
@@ -495,12 +498,17 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
         }
         if (!more) break;
         uint32_t pend = good ? want : 0u;
+        __syncwarp();                  // the warp's own words are sent before it starts polling
         const unsigned long long* in = slot + 2 * own;
-        for (unsigned spin = 0; pend; ++spin) {
+        // a warp stays together until all its lanes have their words
+        for (unsigned spin = 0; __any_sync(0xffffffffu, pend != 0u); ++spin) {
             unsigned long long word[2 + RES64_RING][2];
 #pragma unroll
             for (int m = 0; m < 2 + RES64_RING; ++m)
-                if (pend & (1u << m)) res_peek2(in + 2 * (t + m * RES_T), word[m]);
+                if (pend & (1u << m))
+                    res_peek2(in + 2 * (m < 2 ? t + m * RES_T
+                                              : 2 * RES_T + t + (m - 2) * (int)blockDim.x),
+                              word[m]);
 #pragma unroll
             for (int m = 0; m < 2 + RES64_RING; ++m) {
                 double val;
@@ -511,10 +519,10 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
                     pend &= ~(1u << m);
                 }
             }
-            if (pend && spin >= RES_SPIN_LIMIT) {
+            if (spin >= RES_SPIN_LIMIT && pend) {
                 atomicExch(A.err, 1u);
                 good = false;
-                break;
+                pend = 0;
             }
         }
         __syncthreads();
