@@ -8,6 +8,7 @@
 #include "sweep_t3.cuh"
 #include "sweep_res.cuh"
 #include "bv_kernels.cuh"
+#include "bv_res.cuh"
 
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -143,9 +144,13 @@ struct rfb_soc_handle {
     struct ResPlan {
         int cpt = -1;             // planes of a brick; 0 the lattice does not fit, -1 not planned
         int bx = 0, by = 0, gx = 0, gy = 0, gz = 0;
+        int threads = 0;          // whole warps for a brick's columns and its polled side faces
         unsigned long long* inbox = nullptr;
         uint32_t tag = 0;
-    } res, res64;
+    } res, res64, res_cg, res_bv;
+    unsigned long long* cg_rows = nullptr;   // reduction rows of the resident potential solve
+    double* cg_out = nullptr;                // its result
+    uint32_t cg_rtag = 0;
     bool res_used = false;        // the last FP32 correction sweeps were resident ones
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 };
@@ -475,32 +480,36 @@ void check_df(rfb_soc_handle* h, const OpPoint& op, bool umt, bool fuse) {
 
 // The cut of the lattice into at most one brick per SM (cpt 0 if there is none) with the least
 // work per sweep in its fullest CTA: whole warps of columns times planes, and a little for
-// the side faces. ring: values of the side faces a CTA can poll.
+// the side faces. ring: side-face words a thread polls at most, for `values` words a cell;
+// most: threads of a CTA at most.
 void res_plan(rfb_soc_handle* h, rfb_soc_handle::ResPlan& P, const std::vector<int>& cpts,
-              int ring_most) {
-    if (P.cpt >= 0) return;
+              int ring, int values = 1, int most = RES_T) {
+    if (P.cpt > 0) return;
     P.cpt = 0;
     int sms = 0, coop = 0;
     CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     CK(h, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
     if (!coop) return;
+    sms = std::min(sms, 32 * RES_LANE);
     double best = INFINITY;
     for (int gx = 1; gx <= std::min(h->nx / 2, sms); ++gx) {
         const int bx = (h->nx + gx - 1) / gx;
         if ((h->nx + bx - 1) / bx != gx || bx > 64) continue;
         for (int gy = 1; gy <= std::min(h->ny / 2, sms / gx); ++gy) {
             const int by = (h->ny + gy - 1) / gy;
-            if ((h->ny + by - 1) / by != gy || bx * by > RES_T || bx * (by + 2) > RES_ROWS) continue;
+            if ((h->ny + by - 1) / by != gy || bx * by > most || bx * (by + 2) > RES_ROWS) continue;
             for (int cpt : cpts) {
                 const int gz = (h->nz + cpt - 1) / cpt;
-                const int ring = 2 * cpt * (bx + by);
-                if (gx * gy * gz > sms || ring > ring_most) continue;
-                const double cost = 5.0 * cpt * ((bx * by + 31) / 32) + 0.25 * ring;
+                const int side = 2 * cpt * (bx + by);
+                const int poll = (side * values + ring - 1) / ring;
+                if (gx * gy * gz > sms || poll > most) continue;
+                const double cost = 5.0 * cpt * ((bx * by + 31) / 32) + 0.25 * side;
                 if (cost < best) {
                     best = cost;
                     P.cpt = cpt;
                     P.bx = bx; P.by = by;
                     P.gx = gx; P.gy = gy; P.gz = gz;
+                    P.threads = (std::max(bx * by, poll) + 31) / 32 * 32;
                 }
             }
         }
@@ -521,7 +530,7 @@ void (*res64_kernel(int cpt))(Res64Args) {
 // The resident FP64 sweeps are the faster ones wherever the lattice fits (up to about 0.46 M
 // cells): 7.9 us a sweep at 396k cells, where launches take 12.3.
 bool res64_fits(rfb_soc_handle* h) {
-    res_plan(h, h->res64, {2, 3, 4, 5, 6}, RES64_RING * RES_T);
+    if (h->res64.cpt < 0) res_plan(h, h->res64, {2, 3, 4, 5, 6}, RES64_RING);
     return h->res64.cpt > 0;
 }
 
@@ -554,7 +563,7 @@ void res64_sweeps(rfb_soc_handle* h, const OpPoint& op, double** buf, int& cur, 
         A.tag = P.tag;
         P.tag += (uint32_t)A.n;
         void* args[] = {&A};
-        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(RES_T), args, smem,
+        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads), args, smem,
                                           h->stream));
         ++h->launches;
         cur ^= 1;
@@ -828,7 +837,7 @@ ResKernel res_kernel(int cpt) {
 // The resident FP32 sweeps are the faster ones wherever the lattice fits (up to about 0.9 M
 // cells): 1.9 us a sweep at 528k cells, where launches and passes take 6.2 us.
 bool res_fits(rfb_soc_handle* h) {
-    res_plan(h, h->res, {2, 4, 6, 8, 10, 12}, 2 * RES_RING * RES_T);
+    if (h->res.cpt < 0) res_plan(h, h->res, {2, 4, 6, 8, 10, 12}, 2 * RES_RING);
     return h->res.cpt > 0;
 }
 
@@ -859,7 +868,7 @@ void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int6
         A.tag = P.tag;
         P.tag += (uint32_t)A.n;
         void* args[] = {&A};
-        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(RES_T), args, smem,
+        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads), args, smem,
                                           h->stream));
         ++h->launches;
         if (q) swap_delta(h);
@@ -1266,7 +1275,8 @@ void free_all(rfb_soc_handle* h) {
     void* ptrs[] = {h->d_arena, h->d_m,    h->d_m32,  h->d_lam[0], h->d_lam[1], h->d_g,
                     h->d_grad,  h->d_L64,  h->d_L2F,  h->d_eta,    h->d_elec,   h->d_sdf[0],
                     h->d_sdf[1], h->d_gdf,  h->d_stage,  h->d_bv,     h->d_bvpart,
-                    h->res.inbox, h->res64.inbox};
+                    h->res.inbox, h->res64.inbox, h->res_cg.inbox,
+                    h->res_bv.inbox, h->cg_rows, h->cg_out};
     for (void* p : ptrs)   // back to the pool, in the handle's stream order
         if (p) cudaFreeAsync(p, h->stream);
     cudaStreamSynchronize(h->stream);
@@ -1702,6 +1712,103 @@ rfb_status rfb_soc_solve_nernst(rfb_soc_handle* h, double s_in, double eta, doub
 
 namespace {
 
+// ---- resident Butler-Volmer kernels (bv_res.cuh)
+
+void (*bv_cgr(int cpt, int threads))(BVCgArgs) {
+    if (threads <= 256)
+        return cpt == 2 ? bv_cgr_kernel<2, 256> : cpt == 3 ? bv_cgr_kernel<3, 256>
+                                                           : bv_cgr_kernel<4, 256>;
+    return cpt == 2 ? bv_cgr_kernel<2, RES_T> : cpt == 3 ? bv_cgr_kernel<3, RES_T>
+                                                         : bv_cgr_kernel<4, RES_T>;
+}
+ResCut res_cut(const rfb_soc_handle::ResPlan& P) { return {P.bx, P.by, P.gx, P.gy, P.gz}; }
+
+// They are the faster ones wherever the lattice fits (the potential solve up to about 0.3 M
+// cells, the species sweeps 0.15 M): a solve of 16x18x24 takes 237 ms instead of 1000. Bricks
+// of up to 256 columns first: their threads have twice the registers.
+bool bv_cg_fits(rfb_soc_handle* h) {
+    auto& P = h->res_cg;
+    if (P.cpt < 0) res_plan(h, P, {2, 3, 4}, BV_RING, 1, 256);
+    if (P.cpt == 0) res_plan(h, P, {2, 3, 4}, BV_RING);
+    return P.cpt > 0;
+}
+bool bv_sweep_fits(rfb_soc_handle* h) {
+    auto& P = h->res_bv;
+    if (P.cpt < 0) res_plan(h, P, {BVS_CPT}, BV_RING, 3, 256);
+    if (P.cpt == 0) res_plan(h, P, {BVS_CPT}, BV_RING, 3);
+    return P.cpt > 0;
+}
+
+// n species sweeps at the potential phi from buf[v][cur] into buf[v][cur ^ 1] and on, 2048 a
+// launch
+void bv_res_sweeps(rfb_soc_handle* h, const BVArgs& B, const double* phi, double* (&buf)[3][2],
+                   int& cur, int64_t n) {
+    auto& P = h->res_bv;
+    BVSweepArgs A{};
+    A.B = B;
+    A.cut = res_cut(P);
+    A.phi = phi;
+    A.stride = res64_stride(P.cpt, P.bx, P.by);
+    A.err = wait_err_word(h);
+    const int ctas = P.gx * P.gy * P.gz, smem = bv_sweep_smem();
+    if (!P.inbox) dalloc(h, &P.inbox, (size_t)ctas * 12 * A.stride);
+    A.inbox = P.inbox;
+    const auto k = P.threads <= 256 ? bv_sweepr_kernel<256> : bv_sweepr_kernel<RES_T>;
+    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    for (int64_t q = 0; q < n; q += A.n) {
+        A.n = (int)std::min<int64_t>(n - q, 2048);
+        for (int v = 0; v < 3; ++v) {
+            A.C[v] = buf[v][cur];
+            A.C2[v] = buf[v][cur ^ 1];
+        }
+        A.tag = P.tag;
+        P.tag += (uint32_t)A.n;
+        void* args[] = {&A};
+        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads),
+                                          args, smem, h->stream));
+        ++h->launches;
+        cur ^= 1;
+    }
+}
+
+// One potential solve: out receives the iterations, the looks without progress and the
+// BV_STATS values of the last look.
+void bv_res_potential(rfb_soc_handle* h, const BVArgs& B, const double* kcell, const double* kmem,
+                      const double* bphi, double* phi, double tol, int max_it,
+                      double (&out)[BV_CG_OUT]) {
+    auto& P = h->res_cg;
+    BVCgArgs A{};
+    A.B = B;
+    A.cut = res_cut(P);
+    A.kcell = kcell; A.kmem = kmem; A.bphi = bphi; A.phi = phi;
+    A.tol = tol;
+    A.max_it = max_it;
+    A.stride = res64_stride(P.cpt, P.bx, P.by);
+    A.err = wait_err_word(h);
+    const int ctas = P.gx * P.gy * P.gz, smem = bv_cg_smem(P.cpt);
+    if (!P.inbox) {
+        dalloc(h, &P.inbox, (size_t)ctas * 4 * A.stride);
+        dalloc(h, &h->cg_rows, (size_t)ctas * 4);
+        dalloc(h, &h->cg_out, BV_CG_OUT);
+    }
+    A.inbox = P.inbox;
+    A.rows = h->cg_rows;
+    A.out = h->cg_out;
+    A.tag = P.tag;
+    A.rtag = h->cg_rtag;
+    const auto k = bv_cgr(P.cpt, P.threads);
+    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    void* args[] = {&A};
+    CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads), args, smem,
+                                      h->stream));
+    ++h->launches;
+    CK(h, cudaMemcpyAsync(out, h->cg_out, sizeof out, cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+    // the next launch's words follow this one's
+    P.tag += (uint32_t)out[2 + BV_STATS];
+    h->cg_rtag += (uint32_t)out[3 + BV_STATS];
+}
+
 // N-double fields of the Butler-Volmer state in h->d_bv: 0-1 O, 2-3 R, 4-5 H
 // (ping-pong), 6 phi, 7 phi before the last potential solve, 8 right-hand side of the
 // potential equation, 9 kappa_c, 10 membrane kappa, 11-14 CG r, z, p, q; then 1/diag.
@@ -1809,19 +1916,23 @@ rfb_status rfb_soc_solve_bv(rfb_soc_handle* h, double s_in, double eta, double t
                                  : std::pow(h->nz * h->h, 2) / h->D;
         const double scale[3] = {c0, c0, P.c_H_in};
         std::vector<double> hp((size_t)BV_NB * BV_STATS);
-        double hred[NRED];
+        const int nb = (int)std::min<int64_t>(BV_NB, (N + BV_TPB - 1) / BV_TPB);
+        const bool res_cg = bv_cg_fits(h), res_sweep = bv_sweep_fits(h);
+        double hred[NRED + 1];
         rfb_bv_result r{};
         rfb_status st = RFB_OK;
         auto check = [&]() {   // species residuals and outputs at (C, phi)
             const int cur = h->bv_cur;
-            bv_check_kernel<<<BV_NB, BV_TPB, 0, h->stream>>>(
+            bv_check_kernel<<<nb, BV_TPB, 0, h->stream>>>(
                 A, bv_field(h, 0 + cur), bv_field(h, 2 + cur), bv_field(h, 4 + cur),
                 bv_field(h, 6), bv_field(h, 8), bv_field(h, 9), bv_field(h, 10), part);
             LAUNCHED(h);
-            finalize_kernel<<<1, 256, 0, h->stream>>>(part, BV_NB, h->d_red, 0);
+            finalize_kernel<<<1, 256, 0, h->stream>>>(part, nb, h->d_red, 0, wait_err_word(h));
             LAUNCHED(h);
             CK(h, cudaMemcpyAsync(hred, h->d_red, sizeof hred, cudaMemcpyDeviceToHost, h->stream));
             CK(h, cudaStreamSynchronize(h->stream));
+            h->h_red[NRED] = hred[NRED];
+            if (wait_gave_up(h)) throw Fail{RFB_ERR_CUDA};
             double resid = 0.0;
             for (int q = 0; q < 3; ++q)
                 resid = std::max(resid, tau * std::sqrt(hred[q] / (double)h->n_fluid) / scale[q]);
@@ -1838,6 +1949,22 @@ rfb_status rfb_soc_solve_bv(rfb_soc_handle* h, double s_in, double eta, double t
         bool cg_ok = false;
         auto potential = [&](double bmax) -> double {
             double* phi = bv_field(h, 6);
+            if (res_cg) {
+                double o[BV_CG_OUT];
+                bv_res_potential(h, A, bv_field(h, 9), bv_field(h, 10), bv_field(h, 8), phi,
+                                 P.cg_rtol * bmax, P.max_cg, o);
+                const double* st6 = o + 2;
+                r.cg_iterations += (int64_t)o[0];
+                r.phi_mean = st6[2] / (double)h->n_fluid;
+                r.phi_min = st6[3];
+                r.phi_max = st6[4];
+                cg_ok = st6[0] <= std::max(P.cg_rtol * bmax, 64.0 * 2.2e-16 * st6[5]) ||
+                        o[1] >= 20;
+                if (!cg_ok && std::isfinite(st6[0]))
+                    set_err(h, "potential solve: max residual %.3e after %d iterations", st6[0],
+                            (int)o[0]);
+                return std::isfinite(st6[0]) ? st6[1] : INFINITY;
+            }
             CK(h, cudaMemcpyAsync(bv_field(h, 7), phi, N * 8, cudaMemcpyDeviceToDevice, h->stream));
             double* rr = bv_field(h, 11);
             double* zz = bv_field(h, 12);
@@ -1936,7 +2063,13 @@ rfb_status rfb_soc_solve_bv(rfb_soc_handle* h, double s_in, double eta, double t
                 break;
             }
             const int64_t n = std::min<int64_t>(P.cycle, o.max_sweeps - done);
-            for (int64_t q = 0; q < n; ++q) {
+            if (res_sweep) {
+                double* buf[3][2];
+                for (int v = 0; v < 3; ++v)
+                    for (int c = 0; c < 2; ++c) buf[v][c] = bv_field(h, 2 * v + c);
+                bv_res_sweeps(h, A, bv_field(h, 6), buf, h->bv_cur, n);
+            }
+            for (int64_t q = 0; q < n && !res_sweep; ++q) {
                 const int cur = h->bv_cur;
                 bv_sweep_kernel<<<flat_grid(N), BV_TPB, 0, h->stream>>>(
                     A, bv_field(h, 0 + cur), bv_field(h, 2 + cur), bv_field(h, 4 + cur),
