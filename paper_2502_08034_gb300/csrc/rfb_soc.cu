@@ -286,12 +286,13 @@ unsigned int* wait_err_word(rfb_soc_handle* h) {
     return reinterpret_cast<unsigned int*>(h->d_err + 3);
 }
 
+// The totals of d_partials into h_red, written there by the kernel (pinned memory, mapped into
+// the device's address space): no copy. ev[2] marks the end of the reduction on the stream.
 void reduce_readback(rfb_soc_handle* h, int min_slot0) {
-    finalize_kernel<<<1, 256, 0, h->stream>>>(h->d_partials, h->nblocks, h->d_red, min_slot0,
-                                              wait_err_word(h));
+    finalize_kernel<<<1, FIN_T, 0, h->stream>>>(h->d_partials, h->nblocks, h->h_red, min_slot0,
+                                                wait_err_word(h));
     LAUNCHED(h);
-    CK(h, cudaMemcpyAsync(h->h_red, h->d_red, (NRED + 1) * sizeof(double),
-                          cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaEventRecord(h->ev[2], h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
 }
 
@@ -1129,8 +1130,6 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
         CK(h, cudaEventRecord(h->ev[1], h->stream));
         df_end(h, umt);
         check(h, op, umt);
-        CK(h, cudaEventRecord(h->ev[2], h->stream));
-        CK(h, cudaEventSynchronize(h->ev[2]));
         float ms_c = 0.f;
         CK(h, cudaEventElapsedTime(&ms_c, h->ev[1], h->ev[2]));
         check_ms += ms_c;
@@ -1186,8 +1185,6 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
             df_end(h, umt);
             CK(h, cudaEventRecord(h->ev[1], h->stream));
             check_forcing64(h, op, umt, false);
-            CK(h, cudaEventRecord(h->ev[2], h->stream));
-            CK(h, cudaEventSynchronize(h->ev[2]));
             float ms_c = 0.f;
             CK(h, cudaEventElapsedTime(&ms_c, h->ev[1], h->ev[2]));
             check_ms += ms_c;
@@ -1221,8 +1218,6 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
         } else {
             check(h, op, umt);
         }
-        CK(h, cudaEventRecord(h->ev[2], h->stream));   // check() synchronised the stream
-        CK(h, cudaEventSynchronize(h->ev[2]));
         float ms_s = 0.f, ms_c = 0.f;
         CK(h, cudaEventElapsedTime(&ms_s, h->ev[0], h->ev[1]));
         CK(h, cudaEventElapsedTime(&ms_c, h->ev[1], h->ev[2]));
@@ -1469,7 +1464,7 @@ rfb_status rfb_soc_create(const int32_t dims[3], double dx, const uint8_t* fiber
             stats_kernel<<<sblocks, 256, 0, h->stream>>>(h->d_flags, h->d_w, h->d_m, N, nxny,
                                                          h->d_partials);
             LAUNCHED(h);
-            finalize_kernel<<<1, 256, 0, h->stream>>>(h->d_partials, sblocks, h->d_red, 0);
+            finalize_kernel<<<1, FIN_T, 0, h->stream>>>(h->d_partials, sblocks, h->d_red, 0);
             LAUNCHED(h);
             unsigned long long herr[4];
             CK(h, cudaMemcpyAsync(herr, h->d_err, sizeof herr, cudaMemcpyDeviceToHost,
@@ -1685,8 +1680,6 @@ rfb_status rfb_soc_solve_nernst(rfb_soc_handle* h, double s_in, double eta, doub
             }
             CK(h, cudaEventRecord(h->ev[1], h->stream));
             check(h, op, false);
-            CK(h, cudaEventRecord(h->ev[2], h->stream));
-            CK(h, cudaEventSynchronize(h->ev[2]));
             float ms_s = 0.f, ms_c = 0.f;
             CK(h, cudaEventElapsedTime(&ms_s, h->ev[0], h->ev[1]));
             CK(h, cudaEventElapsedTime(&ms_c, h->ev[1], h->ev[2]));
@@ -1927,7 +1920,7 @@ rfb_status rfb_soc_solve_bv(rfb_soc_handle* h, double s_in, double eta, double t
                 A, bv_field(h, 0 + cur), bv_field(h, 2 + cur), bv_field(h, 4 + cur),
                 bv_field(h, 6), bv_field(h, 8), bv_field(h, 9), bv_field(h, 10), part);
             LAUNCHED(h);
-            finalize_kernel<<<1, 256, 0, h->stream>>>(part, nb, h->d_red, 0, wait_err_word(h));
+            finalize_kernel<<<1, FIN_T, 0, h->stream>>>(part, nb, h->d_red, 0, wait_err_word(h));
             LAUNCHED(h);
             CK(h, cudaMemcpyAsync(hred, h->d_red, sizeof hred, cudaMemcpyDeviceToHost, h->stream));
             CK(h, cudaStreamSynchronize(h->stream));
@@ -2255,7 +2248,7 @@ rfb_status rfb_soc_set_area_mult(rfb_soc_handle* h, const double* m, rfb_mem_kin
         stats_kernel<<<sblocks, 256, 0, h->stream>>>(h->d_flags, h->d_w, src, h->N, h->nxny,
                                                      h->d_partials);
         LAUNCHED(h);
-        finalize_kernel<<<1, 256, 0, h->stream>>>(h->d_partials, sblocks, h->d_red, 0);
+        finalize_kernel<<<1, FIN_T, 0, h->stream>>>(h->d_partials, sblocks, h->d_red, 0);
         LAUNCHED(h);
         CK(h, cudaMemcpyAsync(h->h_red, h->d_red, NRED * sizeof(double), cudaMemcpyDeviceToHost,
                               h->stream));
@@ -2649,7 +2642,7 @@ extern "C" rfb_status rfb_soc_current_noalloc(rfb_soc_handle* h, rfb_solve_resul
         check_kernel<false, false><<<h->grid, h->block, 0, h->stream>>>(
             lattice(h), C, h->d_s[h->s_cur], nullptr, nullptr, nullptr, partials, h->kchunk);
         LAUNCHED(h);
-        finalize_kernel<<<1, 256, 0, h->stream>>>(partials, h->nblocks, sums, 0);
+        finalize_kernel<<<1, FIN_T, 0, h->stream>>>(partials, h->nblocks, sums, 0);
         LAUNCHED(h);
         double host_sums[NRED];
         CK(h, cudaMemcpyAsync(host_sums, sums, sizeof host_sums, cudaMemcpyDeviceToHost,
@@ -2886,7 +2879,7 @@ void batch_check_items(rfb_batch* b, bool fused) {
 
 void batch_check(rfb_batch* b, bool fused, int sweeps_done) {
     batch_check_items(b, fused);
-    batch_finalize_kernel<<<(int)b->hs.size(), 256, 0, b->stream>>>(
+    batch_finalize_kernel<<<(int)b->hs.size(), FIN_T, 0, b->stream>>>(
         b->d_insts, b->d_item_begin, b->d_partials, b->d_ctl, fused ? 1 : 0, sweeps_done);
     BLAUNCHED(b);
 }

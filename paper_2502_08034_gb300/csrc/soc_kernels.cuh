@@ -101,6 +101,12 @@ __device__ __forceinline__ T reaction(const Coef<T>& C, const T* tA, const T* tB
 __device__ __forceinline__ bool positive(double q) { return __double_as_longlong(q) > 0; }
 __device__ __forceinline__ bool positive(float q) { return q > 0.0f; }
 
+// max(q, 0) and max(-q, 0) on the integer pipe
+__device__ __forceinline__ double upward(double q) { return positive(q) ? q : 0.0; }
+__device__ __forceinline__ double downward(double q) {
+    return __double_as_longlong(q) < 0 ? -q : 0.0;
+}
+
 __device__ __forceinline__ int n_wall_of(unsigned f, int i, int j, int k, int nx, int ny,
                                          int nz) {
     int dom = 6 - (i == 0) - (i == nx - 1) - (j == 0) - (j == ny - 1) - (k == 0) -
@@ -140,9 +146,9 @@ __device__ __forceinline__ T cell_rhs(const Coef<T>& C, const T* tA, const T* tB
 template <typename T>
 __device__ __forceinline__ T cell_diag(const Coef<T>& C, const T* tB, unsigned f, T uL, T uH,
                                        T vL, T vH, T wL, T wH, bool inlet, int nw, T mult) {
-    T d = (uH > T(0) ? uH : T(0)) + (uL < T(0) ? -uL : T(0));
-    d += (vH > T(0) ? vH : T(0)) + (vL < T(0) ? -vL : T(0));
-    d += (wH > T(0) ? wH : T(0)) + (wL < T(0) ? -wL : T(0));
+    T d = upward(uH) + downward(uL);
+    d += upward(vH) + downward(vL);
+    d += upward(wH) + downward(wL);
     d += C.Dh * T(__popc(f & F_NBRS));
     if (inlet) d += C.gDh;
     d += mult * tB[nw];
@@ -529,6 +535,7 @@ struct L64 {
 };
 
 __device__ __forceinline__ void block_reduce_store(double (&acc)[NRED], double* out);
+__device__ __forceinline__ void note_rhs(double r, double (&acc)[NRED]);
 
 __global__ void assemble64_kernel(Lattice L, Coef<double> C, L64 K) {
     __shared__ double tA[8], tB[8];
@@ -549,21 +556,20 @@ __global__ void assemble64_kernel(Lattice L, Coef<double> C, L64 K) {
             const double wL = C.w[c], wH = C.w[c + nxny];
             const double Dh = C.Dh;
             // inflow coefficients (upwind) and diffusion to fluid neighbours
-            a[0] = fmax(uL, 0.0) + ((f & F_XM) ? Dh : 0.0);
-            a[1] = fmax(-uH, 0.0) + ((f & F_XP) ? Dh : 0.0);
-            a[2] = fmax(vL, 0.0) + ((f & F_YM) ? Dh : 0.0);
-            a[3] = fmax(-vH, 0.0) + ((f & F_YP) ? Dh : 0.0);
-            a[4] = (k > 0) ? fmax(wL, 0.0) + ((f & F_ZM) ? Dh : 0.0) : 0.0;
-            a[5] = fmax(-wH, 0.0) + ((f & F_ZP) ? Dh : 0.0);
-            const double outflow = (fmax(-uL, 0.0) + fmax(uH, 0.0)) +
-                                   (fmax(-vL, 0.0) + fmax(vH, 0.0)) +
-                                   (fmax(-wL, 0.0) + fmax(wH, 0.0));
+            a[0] = upward(uL) + ((f & F_XM) ? Dh : 0.0);
+            a[1] = downward(uH) + ((f & F_XP) ? Dh : 0.0);
+            a[2] = upward(vL) + ((f & F_YM) ? Dh : 0.0);
+            a[3] = downward(vH) + ((f & F_YP) ? Dh : 0.0);
+            a[4] = (k > 0) ? upward(wL) + ((f & F_ZM) ? Dh : 0.0) : 0.0;
+            a[5] = downward(wH) + ((f & F_ZP) ? Dh : 0.0);
+            const double outflow = (downward(uL) + upward(uH)) + (downward(vL) + upward(vH)) +
+                                   (downward(wL) + upward(wH));
             const int nw = n_wall_of(f, i, j, k, nx, ny, nz);
             const double mult = C.m ? C.m[c] : 1.0;
             dg = -(outflow + Dh * (double)__popc(f & F_NBRS) + (k == 0 ? C.gDh : 0.0) +
                    mult * tB[nw]);
             bb = mult * tA[nw];
-            if (k == 0) bb += (fmax(wL, 0.0) + C.gDh) * C.s_in;
+            if (k == 0) bb += (upward(wL) + C.gDh) * C.s_in;
         }
 #pragma unroll
         for (int q = 0; q < 6; ++q) K.f[q][c] = a[q];
@@ -870,12 +876,7 @@ adjoint64c_kernel(Lattice L, L64 K, const float* __restrict__ dtc, double dt_glo
                     const double dt = dtc ? widen(dtc[c]) : dt_global;
                     lam_out[c] = fma(dt, r, l_cur);
                 } else {
-                    if (isfinite(r)) {
-                        acc[0] += r * r;
-                        acc[7] = fmax(acc[7], fabs(r));
-                    } else {
-                        acc[6] += 1.0;
-                    }
+                    note_rhs(r, acc);
                     acc[1] += g[c] * g[c];
                 }
             }
@@ -893,32 +894,91 @@ adjoint64c_kernel(Lattice L, L64 K, const float* __restrict__ dtc, double dt_glo
 // ---------------------------------------------------------------------------------
 // Block reduction helpers (fixed order => deterministic)
 // ---------------------------------------------------------------------------------
-__device__ __forceinline__ double warp_sum(double x) {
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    return x;
-}
-__device__ __forceinline__ double warp_max(double x) {
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_down_sync(0xffffffffu, x, o));
-    return x;
+// One right-hand side into the reductions: sum of squares (0), count of non-finite values (6),
+// largest magnitude (7); compared and classified on the integer pipe.
+__device__ __forceinline__ void note_rhs(double r, double (&acc)[NRED]) {
+    const long long b = __double_as_longlong(r) & 0x7fffffffffffffffll;
+    if (b < 0x7ff0000000000000ll) {
+        acc[0] += r * r;
+        if (b > __double_as_longlong(acc[7])) acc[7] = __longlong_as_double(b);
+    } else {
+        acc[6] += 1.0;
+    }
 }
 
-// slots 0..NRED-2 are sums, slot NRED-1 is a max
+// largest of the warp's numbers x >= 0 (their bits order them)
+__device__ __forceinline__ double warp_max(double x) {
+    const unsigned hi = __double2hiint(x), lo = __double2loint(x);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    return __hiloint2double((int)mh, (int)__reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u));
+}
+__device__ __forceinline__ double larger_bits(double a, double b) {   // a, b >= 0
+    return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
+
+// Sums (slots 0..6) and the maximum of numbers >= 0 (slot 7) over a block, fixed order. A
+// warp's seven sums are reduced and scattered together: in each of three steps a lane passes
+// half of its slots to its partner and keeps the sums of the others, so nine FP64 additions
+// leave one slot per four lanes (five per slot, 35, reduced one by one: with the maximum's
+// they were two thirds of the FP64 time of a check on a small lattice).
 __device__ __forceinline__ void block_reduce_store(double (&acc)[NRED], double* out) {
     __shared__ double sh[BX * BY / 32][NRED];
     const int tid = threadIdx.y * BX + threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
+    const double vmax = warp_max(acc[NRED - 1]);
+    double v[NRED];
 #pragma unroll
-    for (int q = 0; q < NRED - 1; ++q) acc[q] = warp_sum(acc[q]);
-    acc[NRED - 1] = warp_max(acc[NRED - 1]);
-    if (lane == 0) {
+    for (int q = 0; q < NRED; ++q) v[q] = q < NRED - 1 ? acc[q] : 0.0;
 #pragma unroll
-        for (int q = 0; q < NRED; ++q) sh[wid][q] = acc[q];
+    for (int n = NRED / 2; n >= 1; n >>= 1) {          // lane distances 16, 8, 4
+        const bool up = lane & (4 * n);
+#pragma unroll
+        for (int q = 0; q < n; ++q) {
+            const double keep = up ? v[n + q] : v[q], pass = up ? v[q] : v[n + q];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, pass, 4 * n);
+        }
     }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    if ((lane & 3) == 0) sh[wid][lane >> 2] = lane == 28 ? vmax : v[0];
     __syncthreads();
     if (tid < NRED) {
         double r = sh[0][tid];
         for (int w = 1; w < BX * BY / 32; ++w)
-            r = (tid == NRED - 1) ? fmax(r, sh[w][tid]) : r + sh[w][tid];
+            r = (tid == NRED - 1) ? larger_bits(r, sh[w][tid]) : r + sh[w][tid];
+        out[tid] = r;
+    }
+}
+static_assert(NRED == 8 && BX * BY / 32 == 8, "eight slots, eight warps");
+
+// The same for the double-float checks, whose threads hold FP32 sums of squares (slots 0 and,
+// with G, 1), a count (6) and a maximum (7); the other slots are 0.
+template <bool G>
+__device__ __forceinline__ void block_reduce_df(float sum2, float sumg, int bad, float vmax,
+                                                double* out) {
+    __shared__ double sh[2][BX * BY / 32];
+    __shared__ unsigned shu[2][BX * BY / 32];
+    const int tid = threadIdx.y * BX + threadIdx.x;
+    const int lane = tid & 31, wid = tid >> 5;
+    const unsigned nbad = __reduce_add_sync(0xffffffffu, (unsigned)bad);
+    const unsigned big = __reduce_max_sync(0xffffffffu, __float_as_uint(vmax));
+    double a = widen(sum2), g = G ? widen(sumg) : 0.0;
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (G) g += __shfl_xor_sync(0xffffffffu, g, o);
+    }
+    if (lane == 0) { sh[0][wid] = a; sh[1][wid] = g; shu[0][wid] = nbad; shu[1][wid] = big; }
+    __syncthreads();
+    if (tid < NRED) {
+        double r = 0.0;
+        unsigned n = 0, m = 0;
+        for (int w = 0; w < BX * BY / 32; ++w) {
+            if (tid == 0 || (G && tid == 1)) r += sh[tid][w];
+            n += shu[0][w];
+            m = max(m, shu[1][w]);
+        }
+        if (tid == 6) r = (double)n;
+        if (tid == 7) r = widen(__uint_as_float(m));
         out[tid] = r;
     }
 }
@@ -994,12 +1054,7 @@ __device__ __forceinline__ void check_column(const Lattice& L, const Coef<double
                 double r = cell_rhs<double>(C, tA, tB, s_cur, sxm, sxp, sym, syp, szm, szp, uL, uH,
                                             vL, vH, wL, wH, k == 0, outlet, nw, mult);
                 if (!pinned) {
-                    if (isfinite(r)) {
-                        acc[0] += r * r;
-                        acc[7] = fmax(acc[7], fabs(r));
-                    } else {
-                        acc[6] += 1.0;
-                    }
+                    note_rhs(r, acc);
                     if (WRITE_R) r_out[c] = (float)r;
                 } else if (WRITE_R) {
                     r_out[c] = 0.0f;
@@ -1077,12 +1132,7 @@ check64c_kernel(Lattice L, Coef<double> C, L64 K, const double* __restrict__ s,
                     double r = rhs64(K, c, s_cur, val(c + oxm), val(c + oxp), val(c + oym),
                                      val(c + oyp), s_prev, s_next);
                     if (C.nl) r += src;   // mode 1: the operator holds transport only
-                    if (isfinite(r)) {
-                        acc[0] += r * r;
-                        acc[7] = fmax(acc[7], fabs(r));
-                    } else {
-                        acc[6] += 1.0;
-                    }
+                    note_rhs(r, acc);
                     if (WRITE_R) r_out[c] = (float)r;
                 } else if (WRITE_R) {
                     r_out[c] = 0.0f;
@@ -1233,10 +1283,9 @@ check_df_kernel(Lattice L, L2F K, const float2* __restrict__ s, const float* __r
         check_df_column<FUSE>(L, K, s, delta, s_new, r_out, umt, i, j, kb,
                               min(kb + kchunk, L.nz), sum2, vmax, bad);
     }
-    double acc[NRED] = {(double)sum2, 0.0, 0.0, 0.0, 0.0, 0.0, (double)bad, (double)vmax};
     const int64_t bid = (int64_t)blockIdx.x + (int64_t)gridDim.x *
                         ((int64_t)blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
-    block_reduce_store(acc, partials + bid * NRED);
+    block_reduce_df<false>(sum2, 0.f, bad, vmax, partials + bid * NRED);
 }
 
 // Adjoint defect r = g + L^T lam in double-float (lam [+ delta] as pairs): (L^T lam)_c
@@ -1296,11 +1345,9 @@ check_df_adjoint_kernel(Lattice L, L2F K, const float2* __restrict__ lam,
             l_cur = l_next;
         }
     }
-    double acc[NRED] = {(double)sum2, (double)sumg, 0.0, 0.0, 0.0, 0.0, (double)bad,
-                        (double)vmax};
     const int64_t bid = (int64_t)blockIdx.x + (int64_t)gridDim.x *
                         ((int64_t)blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
-    block_reduce_store(acc, partials + bid * NRED);
+    block_reduce_df<true>(sum2, sumg, bad, vmax, partials + bid * NRED);
 }
 
 // Batched FP64 check (FUSE: state = s64[cur] + delta[0] written to s64[cur ^ 1], FP32
@@ -1371,9 +1418,59 @@ batch_check_df_kernel(const BatchInst* __restrict__ insts, const BatchItem* __re
                                           it.kb, it.ke, sum2, vmax, bad);
             }
         }
-        double acc[NRED] = {(double)sum2, 0.0, 0.0, 0.0, 0.0, 0.0, (double)bad, (double)vmax};
-        block_reduce_store(acc, partials + (int64_t)w * NRED);
+        block_reduce_df<false>(sum2, 0.f, bad, vmax, partials + (int64_t)w * NRED);
     }
+}
+
+// Sum (slots 0..6) / max (slot 7, numbers >= 0) of n rows of partials by one block of FIN_T
+// threads, in a fixed order: thread t takes slot t % 8 of every (FIN_T / 8)-th row (coalesced),
+// then lanes, warps and the last eight rows are added. min_slot0: slot 0 is the smallest
+// instead of the sum (numbers >= 0). The result is in the first warp: thread q holds slot q.
+constexpr int FIN_T = 1024;
+__device__ __forceinline__ double finalize_rows(const double* __restrict__ rows, int64_t n,
+                                                bool min_slot0) {
+    __shared__ double sh[2][FIN_T / 32][NRED];
+    const int t = threadIdx.x, q = t % NRED;
+    const bool is_max = q == NRED - 1, is_min = q == 0 && min_slot0;
+    auto add = [&](double a, double b) {
+        if (is_max) return larger_bits(a, b);
+        if (is_min) return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+        return a + b;
+    };
+    double a = is_min ? 1e300 : 0.0;
+#pragma unroll 4
+    for (int64_t b = t / NRED; b < n; b += FIN_T / NRED) a = add(a, rows[b * NRED + q]);
+    a = add(a, __shfl_xor_sync(0xffffffffu, a, 8));
+    a = add(a, __shfl_xor_sync(0xffffffffu, a, 16));
+    if ((t & 31) < NRED) sh[0][t >> 5][q] = a;
+    __syncthreads();
+    if (t < (FIN_T / 32) * NRED) {                     // 32 rows left
+        a = sh[0][t / NRED][q];
+        a = add(a, __shfl_xor_sync(0xffffffffu, a, 8));
+        a = add(a, __shfl_xor_sync(0xffffffffu, a, 16));
+        if ((t & 31) < NRED) sh[1][t >> 5][q] = a;
+    }
+    __syncthreads();
+    if (t < 32) {                                      // eight rows left
+        a = sh[1][t >> 3][q];
+        a = add(a, sh[1][(t >> 3) + 4][q]);
+        a = add(a, __shfl_xor_sync(0xffffffffu, a, 8));
+        a = add(a, __shfl_xor_sync(0xffffffffu, a, 16));
+    }
+    return a;
+}
+static_assert(FIN_T / 32 == 32 && NRED == 8, "32, then 8 rows");
+
+// The totals of a reduction into out (device or mapped host memory). One slot after the other
+// by a shared-memory tree with a barrier a level, it took 17 to 19 us beside checks of 26 to
+// 110 us; now about 5. err (nullable): the word of the sweeps' bounded waits, passed on in
+// slot NRED.
+__global__ void __launch_bounds__(FIN_T)
+finalize_kernel(const double* __restrict__ partials, int64_t nblocks, double* __restrict__ out,
+                int min_slot0, const unsigned int* __restrict__ err = nullptr) {
+    if (err && threadIdx.x == NRED) out[NRED] = (double)*err;
+    const double a = finalize_rows(partials, nblocks, min_slot0);
+    if (threadIdx.x < NRED) out[threadIdx.x] = a;
 }
 
 // Per-lattice sums of the item partials (one block per lattice, fixed order), then the
@@ -1391,35 +1488,19 @@ struct BatchCtl {
     int nonfinite;
 };
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(FIN_T)
 batch_finalize_kernel(BatchInst* __restrict__ insts, const int* __restrict__ item_begin,
                       const double* __restrict__ partials, BatchCtl* __restrict__ ctl,
                       int fused, int sweeps_done) {
-    __shared__ double sh[256];
     const int q_inst = blockIdx.x;
     BatchInst& I = insts[q_inst];
     const int was_active = I.active;
     __syncthreads();
     if (!was_active) return;   // uniform per block
     const int b0 = item_begin[q_inst], b1 = item_begin[q_inst + 1];
-    for (int q = 0; q < NRED; ++q) {
-        const bool is_max = (q == NRED - 1);
-        double a = 0.0;
-        for (int b = b0 + threadIdx.x; b < b1; b += 256) {
-            const double x = partials[(int64_t)b * NRED + q];
-            a = is_max ? fmax(a, x) : a + x;
-        }
-        sh[threadIdx.x] = a;
-        __syncthreads();
-        for (int sft = 128; sft > 0; sft >>= 1) {
-            if (threadIdx.x < sft)
-                sh[threadIdx.x] = is_max ? fmax(sh[threadIdx.x], sh[threadIdx.x + sft])
-                                         : sh[threadIdx.x] + sh[threadIdx.x + sft];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) ctl[q_inst].sums[q] = sh[0];
-        __syncthreads();
-    }
+    const double a = finalize_rows(partials + (int64_t)b0 * NRED, b1 - b0, false);
+    if (threadIdx.x < NRED) ctl[q_inst].sums[threadIdx.x] = a;
+    __syncthreads();
     if (threadIdx.x == 0) {
         BatchCtl& k = ctl[q_inst];
         if (fused) I.cur ^= 1;
@@ -1444,6 +1525,7 @@ diag_kernel(Lattice L, Coef<double> C, double cfl, float* __restrict__ dtc,
     double acc[NRED];
 #pragma unroll
     for (int q = 0; q < NRED; ++q) acc[q] = 0.0;
+    double dmin = 1e300;
     if (i < L.nx && j < L.ny) {
         const int kb = blockIdx.z * kchunk;
         const int ke = min(kb + kchunk, L.nz);
@@ -1463,27 +1545,28 @@ diag_kernel(Lattice L, Coef<double> C, double cfl, float* __restrict__ dtc,
             const int nw = n_wall_of(f, i, j, k, nx, L.ny, L.nz);
             double mult = C.m ? C.m[c] : 1.0;
             double d = cell_diag<double>(C, tB, f, uL, uH, vL, vH, wL, wH, k == 0, nw, mult);
-            acc[7] = fmax(acc[7], d);
-            acc[0] = (acc[0] == 0.0 || d < acc[0]) ? d : acc[0];
+            acc[7] = larger_bits(acc[7], d);
+            if (positive(d) && __double_as_longlong(d) < __double_as_longlong(dmin)) dmin = d;
             if (dtc) dtc[c] = d > 0.0 ? __double2float_rz(cfl / d) : 0.0f;
         }
     }
-    // slot 0 carries a min: reduce it as -max(-x) by negating around the max slot
-    __shared__ double mins[BX * BY];
+    // slot 0 carries the smallest diagonal instead of a sum
+    __shared__ double mins[BX * BY / 32];
     const int tid = threadIdx.y * BX + threadIdx.x;
-    mins[tid] = acc[0] == 0.0 ? 1e300 : acc[0];
-    acc[0] = 0.0;
-    __syncthreads();
-    for (int sft = BX * BY / 2; sft > 0; sft >>= 1) {
-        if (tid < sft) mins[tid] = fmin(mins[tid], mins[tid + sft]);
-        __syncthreads();
+    {
+        const unsigned hi = __double2hiint(dmin), lo = __double2loint(dmin);
+        const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+        const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : 0xffffffffu);
+        if ((tid & 31) == 0) mins[tid >> 5] = __hiloint2double((int)mh, (int)ml);
     }
-    const double bmin = mins[0];
-    __syncthreads();
     const int64_t bid = (int64_t)blockIdx.x + (int64_t)gridDim.x *
                         ((int64_t)blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
-    block_reduce_store(acc, partials + bid * NRED);
-    if (tid == 0) partials[bid * NRED + 0] = bmin;
+    block_reduce_store(acc, partials + bid * NRED);    // synchronises the block
+    if (tid == 0) {
+        for (int w = 1; w < BX * BY / 32; ++w)
+            if (__double_as_longlong(mins[w]) < __double_as_longlong(mins[0])) mins[0] = mins[w];
+        partials[bid * NRED + 0] = mins[0];
+    }
 }
 
 __global__ void fill_kernel(double* __restrict__ a, double v, int64_t n) {
@@ -1518,38 +1601,6 @@ stats_kernel(const uint8_t* __restrict__ flags, const double* __restrict__ w,
         }
     }
     block_reduce_store(acc, partials + (int64_t)blockIdx.x * NRED);
-}
-
-// Sum (slots 0..6) / max (slot 7) of the per-block partials, in a fixed order.
-// min_slot0: slot 0 is reduced with min instead of a sum (diag_kernel). err (nullable): the
-// word of the sweeps' bounded waits, passed on in slot NRED.
-__global__ void __launch_bounds__(256)
-finalize_kernel(const double* __restrict__ partials, int64_t nblocks, double* __restrict__ out,
-                int min_slot0, const unsigned int* __restrict__ err = nullptr) {
-    __shared__ double sh[256];
-    if (err && threadIdx.x == 0) out[NRED] = (double)*err;
-    for (int q = 0; q < NRED; ++q) {
-        const bool is_max = (q == NRED - 1);
-        const bool is_min = (q == 0 && min_slot0);
-        double a = is_min ? 1e300 : 0.0;
-        for (int64_t b = threadIdx.x; b < nblocks; b += 256) {
-            double x = partials[b * NRED + q];
-            a = is_max ? fmax(a, x) : is_min ? fmin(a, x) : a + x;
-        }
-        sh[threadIdx.x] = a;
-        __syncthreads();
-        for (int sft = 128; sft > 0; sft >>= 1) {
-            if (threadIdx.x < sft) {
-                double x = sh[threadIdx.x + sft];
-                sh[threadIdx.x] = is_max ? fmax(sh[threadIdx.x], x)
-                                         : is_min ? fmin(sh[threadIdx.x], x)
-                                                  : sh[threadIdx.x] + x;
-            }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[q] = sh[0];
-        __syncthreads();
-    }
 }
 
 // ---------------------------------------------------------------------------------
