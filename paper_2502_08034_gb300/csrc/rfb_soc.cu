@@ -751,18 +751,20 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
             LAUNCHED(h);
             return;
         }
-        if (tr && four)
-            sweep32tbd_kernel<true, 4><<<S.grid, TB_THREADS, tbd_smem<4>(), h->stream>>>(
-                td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A);
-        else if (tr)
-            sweep32tbd_kernel<true, 3><<<S.grid, TB_THREADS, tbd_smem<3>(), h->stream>>>(
-                td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A);
-        else if (four)
-            sweep32tbd_kernel<false, 4><<<S.grid, TB_THREADS, tbd_smem<4>(), h->stream>>>(
-                td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A);
-        else
-            sweep32tbd_kernel<false, 3><<<S.grid, TB_THREADS, tbd_smem<3>(), h->stream>>>(
-                td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A);
+        const auto k = tr ? (four ? sweep32tbd_kernel<true, 4> : sweep32tbd_kernel<true, 3>)
+                          : (four ? sweep32tbd_kernel<false, 4> : sweep32tbd_kernel<false, 3>);
+        // a pass may start its blocks while the pass before it runs out (sweep_dt.cuh)
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = S.grid;
+        cfg.blockDim = dim3(TB_THREADS);
+        cfg.dynamicSmemBytes = four ? tbd_smem<4>() : tbd_smem<3>();
+        cfg.stream = h->stream;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        CK(h, cudaLaunchKernelEx(&cfg, k, td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A));
         LAUNCHED(h);
         return;
     }

@@ -227,12 +227,22 @@ __device__ __forceinline__ void tbd_ring_drain(TBDRing<NST, TXI>& R) {
         if (R.pend & (1u << s)) (void)R.wait(s);
 }
 
+// Programmatic dependent launch: the next launch of the stream may start its blocks where this
+// one's have ended, and waits (grid_wait) for all of this one before it touches what this one
+// writes. A launch without the attribute waits at its start and grid_wait returns at once.
+__device__ __forceinline__ void grid_release() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Two sweeps over planes kb .. ke-1 of one tile of lattice F, from F.d_in into F.d_out.
 // Every stage issued is waited for, so the ring is empty when it returns; false if a
-// wait gave up (the CTA decides together at its step barrier).
+// wait gave up (the CTA decides together at its step barrier). early: the first segment of a
+// launch that may have started before the pass before it has ended; what no pass writes
+// (forcing, velocities, step) is fetched at once, delta after that pass.
 template <bool TR, int NST, int TXI = 128>
 __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField& F, int tile,
-                                            int kb, int ke) {
+                                            int kb, int ke, bool early = false) {
     using G = TBDGeom<TXI>;
     const int tid = threadIdx.x;
     const int tx = tid % G::GX, ty = tid / G::GX;
@@ -248,21 +258,29 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
     const int y0 = TB_TYI * (tile / gx) - 2;
     const int i0 = x0 + bxx, j = y0 + byy;
     const bool in_dom = i0 >= 0 && i0 < nx && j >= 0 && j < ny;
-    auto issue = [&](int p, int s) {                   // plane p -> stage s
+    auto issue_delta = [&](int p, int s) {
+        if (tid == 0) tma_load_3d(R.stage(s), F.d, x0, y0, p, &R.bar[s]);
+    };
+    auto issue_rest = [&](int p, int s) {
         R.pend |= 1u << s;
         if (tid != 0) return;                          // one thread issues the copies
         unsigned char* S = R.stage(s);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_expect_tx(&R.bar[s], G::STAGE);
-        tma_load_3d(S, F.d, x0, y0, p, &R.bar[s]);
         tma_load_3d(S + G::F32, F.r, x0, y0, p, &R.bar[s]);
         tma_load_3d(S + 2 * G::F32, F.u, x0, y0, p, &R.bar[s]);
         tma_load_3d(S + 3 * G::F32, F.v, x0, y0, p, &R.bar[s]);
         tma_load_3d(S + 4 * G::F32, F.w, x0, y0, p, &R.bar[s]);
         tma_load_3d(S + 5 * G::F32, F.t, x0, y0, p, &R.bar[s]);
     };
+    auto issue = [&](int p, int s) {                   // plane p -> stage s
+        issue_rest(p, s);
+        issue_delta(p, s);
+    };
     __syncthreads();   // the previous segment's readers are done with every stage
-    for (int s = 0; s < NST; ++s) issue(kb - 1 + s, s);                 // kb-1, kb, ...
+    for (int s = 0; s < NST; ++s) issue_rest(kb - 1 + s, s);            // kb-1, kb, ...
+    if (early) grid_wait();
+    for (int s = 0; s < NST; ++s) issue_delta(kb - 1 + s, s);
 
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 l1_m2 = zero4, l1_m1 = zero4;               // own level 1 at z-2, z-1
@@ -359,6 +377,11 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
 // (chunk, tile) item it touches; positions past nz in the last chunk are skipped. With
 // one chunk and per = tiles * nz / CTAs this is a persistent launch with equal shares;
 // with per = lc every CTA takes one item and neighbouring tiles run together.
+//
+// Programmatic dependent launches took the pass (us per sweep, chunked, four stages) from 7.18
+// to 5.89 on 96x100x150, 12.29 to 10.63 on 128x128x256, 20.5 to 18.8 on 160x160x200 and 42.7
+// to 41.0 on 256^3: a block's barriers, tensor maps and first five fields are in place when
+// the pass before it ends, and the last partial wave overlaps them.
 template <bool TR, int NST>
 __global__ void __launch_bounds__(TB_THREADS, 1)
 sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constant__ CUtensorMap tm_r,
@@ -366,13 +389,14 @@ sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constan
                   const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_t,
                   TBDArgs A) {
     extern __shared__ unsigned char smem_raw[];
+    grid_release();
     TBDRing<NST> R = tbd_ring_init<NST>(smem_raw, A.err);
     const TBDField F{&tm_d, &tm_r, &tm_u, &tm_v, &tm_w, &tm_t, A.nx, A.ny, A.nz,
                      A.d_in, A.d_out, A.omc, A.Dh};
     const int gx = (A.nx + TB_TXI - 1) / TB_TXI;
     const int tiles = gx * ((A.ny + TB_TYI - 1) / TB_TYI);
     const int64_t q1 = min((int64_t)(blockIdx.x + 1) * A.per, A.total);
-    bool ok = true;
+    bool ok = true, first = true;
     for (int64_t q = (int64_t)blockIdx.x * A.per; q < q1 && ok;) {
         const int64_t item = q / A.lc;
         const int zl = (int)(q % A.lc);
@@ -382,7 +406,8 @@ sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constan
         if (kb >= A.nz) { q = item_end; continue; }   // padding of a short last chunk
         const int ke = (int)min((int64_t)A.nz, kb + (min(q1, item_end) - q));
         q = min(q1, item_end);
-        ok = tbd_segment<TR, NST>(R, F, tile, kb, ke);
+        ok = tbd_segment<TR, NST>(R, F, tile, kb, ke, first);
+        first = false;
     }
     if (!ok) tbd_ring_drain<NST>(R);
 }
