@@ -39,13 +39,16 @@ def pass_kernel(kname):
     """(sweeps per launch, kernel description) of an FP32 kernel name of the binding."""
     if not kname or kname == "plain":
         return 1, "sweep32d_kernel (one sweep)"
+    if kname == "resident":
+        return 200, "sweep32r_kernel (resident: the sweeps of a correction cycle in one launch)"
     shape = kname.rsplit("_", 1)[1]
     if kname.startswith("three_sweep"):
         return 3, ("sweep32t3_kernel (three-sweep TMA-staged pass, coefficients of the older "
                    "levels in tensor memory, %s launch, %d delta stages)" % (
                        shape, 5 if kname.startswith("three_sweep5") else 4))
-    return 2, ("sweep32tbd_kernel (two-sweep TMA-staged pass, %s launch, %d TMA stages)" % (
-        shape, 4 if kname.startswith("blocked4") else 3))
+    return 2, ("sweep32tbd_kernel (two-sweep TMA-staged pass, %s launch, %d TMA stages%s)" % (
+        shape, 4 if kname.startswith("blocked4") else 3,
+        ", 64-column tiles" if "narrow" in kname else ""))
 FALLBACK_HBM_GBS = 6800.0
 
 

@@ -527,7 +527,8 @@ rfb_status rfb_selftest_bounded_wait(int64_t spin_limit, int32_t* gave_up);
  * fp32_kernel = 0 or 2 (or the one a solve forced), as an opts.fp32_kernel value: 0 = not
  * chosen yet, 1 = one sweep per launch, 3 / 4 = two-sweep passes in the persistent /
  * chunked launch shape, 5 / 6 the same with four TMA stages, 7 .. 10 three-sweep passes,
- * 11 = resident sweeps (fp32_kernel = 0 on a lattice that fits on the chip);
+ * 11 = resident sweeps (fp32_kernel = 0 on a lattice that fits on the chip), 12 / 13 =
+ * two-sweep passes with 64-column tiles, persistent / chunked (chosen by timing only);
  * and the timed device milliseconds per sweep of the one-sweep kernel and of the fastest
  * pass variant (0 if not timed). Any output pointer may be NULL. */
 rfb_status rfb_soc_tuned_fp32_kernel(const rfb_soc_handle* h, int32_t* kernel,

@@ -130,13 +130,16 @@ struct rfb_soc_handle {
         int64_t total = 0;    // tiles x chunks x lc
         int64_t per = 0;      // positions per CTA
         dim3 grid;
-    } tb_launch[4];           // 2, 3: the same shapes for the three-sweep pass
+    } tb_launch[6];           // 2, 3: the same shapes for the three-sweep pass; 4, 5: for the
+                              // two-sweep pass with 64-column tiles (two CTAs per SM)
     int tb_variant = -1;      // -1 not chosen yet; bit 0 the launch shape; step-field
                               // passes only: bit 1 one more TMA stage of delta (two-sweep:
                               // four instead of three; three-sweep: five instead of four),
-                              // bit 2 three sweeps per pass instead of two
+                              // bit 2 three sweeps per pass instead of two; 8, 9: two
+                              // sweeps, 64-column tiles
     bool tm_ready = false;
     CUtensorMap tm_delta[2], tm_r, tm_u, tm_v, tm_w, tm_f, tm_t;
+    CUtensorMap tmn_delta[2], tmn_r, tmn_u, tmn_v, tmn_w, tmn_t;   // 72-column boxes
     float* tm_delta_ptr[2] = {nullptr, nullptr};
     double tb_tuned_plain_ms = 0, tb_tuned_tb_ms = 0;
     // resident sweeps (sweep_res.cuh), FP32 and FP64: bricks of the lattice, inboxes (first
@@ -659,6 +662,12 @@ void tb_prepare(rfb_soc_handle* h) {
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, tbd_smem<4>()));
         CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<true, 4>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, tbd_smem<4>()));
+        CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<false, 3, 64>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   tbd_smem<3, 64>()));
+        CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<true, 3, 64>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   tbd_smem<3, 64>()));
         CK(h, cudaFuncSetAttribute(sweep32t3_kernel<false, 4>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, t3_smem<4>()));
         CK(h, cudaFuncSetAttribute(sweep32t3_kernel<true, 4>,
@@ -680,7 +689,18 @@ void tb_prepare(rfb_soc_handle* h) {
     if (h->nx % 16 == 0)   // the mask byte of the global-step pass
         tb_encode(h, &h->tm_f, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_mask32, h->nz, TB_BWM);
     tb_encode(h, &h->tm_t, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_dtc, h->nz, TB_BW);
-    // One CTA per SM fits (152 to 227 KB of shared memory each).
+    {
+        constexpr int bw = TBDGeom<64>::BW;
+        for (int q = 0; q < 2; ++q)
+            tb_encode(h, &h->tmn_delta[q], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_delta[q],
+                      h->nz, bw);
+        tb_encode(h, &h->tmn_r, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_r32, h->nz, bw);
+        tb_encode(h, &h->tmn_u, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_u32, h->nz, bw);
+        tb_encode(h, &h->tmn_v, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_v32, h->nz, bw);
+        tb_encode(h, &h->tmn_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_w32, h->nz + 1, bw);
+        tb_encode(h, &h->tmn_t, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_dtc, h->nz, bw);
+    }
+    // One CTA per SM fits (152 to 227 KB of shared memory each), two with 64-column tiles.
     // Shape 0, persistent: the tile-major (tile, plane) space in equal shares of at least
     // 16 planes (every z segment pays a prologue of k planes, k the sweeps of a pass): no
     // partial last wave, but CTAs on neighbouring tiles run at different planes and do not
@@ -689,23 +709,23 @@ void tb_prepare(rfb_soc_handle* h) {
     // neighbouring tiles run together; the chunk count minimises waves x (chunk + k).
     int sms = 152;
     CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-    for (int k = 2; k <= 3; ++k) {
-        const int rows = k == 2 ? TB_TYI : T3_TYI;
-        const int64_t tiles = (int64_t)((h->nx + TB_TXI - 1) / TB_TXI) *
-                              ((h->ny + rows - 1) / rows);
-        auto& P = h->tb_launch[2 * (k - 2)];
+    for (int g = 0; g < 3; ++g) {                      // pairs of tb_launch
+        const int k = g == 1 ? 3 : 2, rows = g == 1 ? T3_TYI : TB_TYI;
+        const int txi = g == 2 ? 64 : TB_TXI, slots = g == 2 ? 2 * sms : sms;
+        const int64_t tiles = (int64_t)((h->nx + txi - 1) / txi) * ((h->ny + rows - 1) / rows);
+        auto& P = h->tb_launch[2 * g];
         P.lc = h->nz;
         P.total = tiles * h->nz;
-        P.per = std::max<int64_t>((P.total + sms - 1) / sms, 16);
+        P.per = std::max<int64_t>((P.total + slots - 1) / slots, 16);
         P.grid = dim3((unsigned)((P.total + P.per - 1) / P.per));
         int best_c = 1;
         double best = INFINITY;
         for (int c = 1; c <= std::max(1, h->nz / 8); ++c) {
             const int lc = (h->nz + c - 1) / c, cc = (h->nz + lc - 1) / lc;
-            const double cost = std::ceil((double)(tiles * cc) / sms) * (lc + k);
+            const double cost = std::ceil((double)(tiles * cc) / slots) * (lc + k);
             if (cost < best) { best = cost; best_c = cc; }
         }
-        auto& Q = h->tb_launch[2 * (k - 2) + 1];
+        auto& Q = h->tb_launch[2 * g + 1];
         Q.lc = (h->nz + best_c - 1) / best_c;
         Q.total = tiles * best_c * Q.lc;
         Q.per = Q.lc;
@@ -715,19 +735,22 @@ void tb_prepare(rfb_soc_handle* h) {
 }
 
 // sweeps of one pass of the chosen variant
-int tb_depth(const rfb_soc_handle* h) { return h->tb_variant >= 4 ? 3 : 2; }
+int tb_depth(const rfb_soc_handle* h) {
+    return h->tb_variant >= 4 && h->tb_variant < 8 ? 3 : 2;
+}
 
 // one pass (two or three sweeps) from delta[cur] into delta[cur ^ 1] (tr: of the
 // transposed operator; local steps only)
 void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur, bool local,
              bool tr = false) {
-    const CUtensorMap& td = (h->d_delta[cur] == h->tm_delta_ptr[0]) ? h->tm_delta[0]
-                                                                     : h->tm_delta[1];
+    const int at = h->d_delta[cur] == h->tm_delta_ptr[0] ? 0 : 1;
+    const CUtensorMap& td = h->tm_delta[at];
     if (local) {
         TBDArgs A{};
         A.nx = h->nx; A.ny = h->ny; A.nz = h->nz;
         const int v = std::max(h->tb_variant, 0);
-        const auto& S = h->tb_launch[v >= 4 ? 2 + (v & 1) : v & 1];
+        const bool narrow = v >= 8;
+        const auto& S = h->tb_launch[(narrow ? 4 : v >= 4 ? 2 : 0) + (v & 1)];
         A.lc = S.lc; A.total = S.total; A.per = S.per;
         A.d_in = h->d_delta[cur];
         A.d_out = h->d_delta[cur ^ 1];
@@ -735,7 +758,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
         A.Dh = C.Dh;
         A.err = wait_err_word(h);
         const bool four = (v & 2) != 0;
-        if (v >= 4) {
+        if (v >= 4 && !narrow) {
             if (tr && four)
                 sweep32t3_kernel<true, 5><<<S.grid, T3_THREADS, t3_smem<5>(), h->stream>>>(
                     td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A);
@@ -751,20 +774,26 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
             LAUNCHED(h);
             return;
         }
-        const auto k = tr ? (four ? sweep32tbd_kernel<true, 4> : sweep32tbd_kernel<true, 3>)
-                          : (four ? sweep32tbd_kernel<false, 4> : sweep32tbd_kernel<false, 3>);
+        const auto k =
+            narrow ? (tr ? sweep32tbd_kernel<true, 3, 64> : sweep32tbd_kernel<false, 3, 64>)
+            : tr   ? (four ? sweep32tbd_kernel<true, 4> : sweep32tbd_kernel<true, 3>)
+                   : (four ? sweep32tbd_kernel<false, 4> : sweep32tbd_kernel<false, 3>);
         // a pass may start its blocks while the pass before it runs out (sweep_dt.cuh)
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchAttribute at1{};
+        at1.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at1.val.programmaticStreamSerializationAllowed = 1;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = S.grid;
-        cfg.blockDim = dim3(TB_THREADS);
-        cfg.dynamicSmemBytes = four ? tbd_smem<4>() : tbd_smem<3>();
+        cfg.blockDim = dim3(narrow ? TBDGeom<64>::THREADS : TB_THREADS);
+        cfg.dynamicSmemBytes = narrow ? tbd_smem<3, 64>() : four ? tbd_smem<4>() : tbd_smem<3>();
         cfg.stream = h->stream;
-        cfg.attrs = &at;
+        cfg.attrs = &at1;
         cfg.numAttrs = 1;
-        CK(h, cudaLaunchKernelEx(&cfg, k, td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A));
+        if (narrow)
+            CK(h, cudaLaunchKernelEx(&cfg, k, h->tmn_delta[at], h->tmn_r, h->tmn_u, h->tmn_v,
+                                     h->tmn_w, h->tmn_t, A));
+        else
+            CK(h, cudaLaunchKernelEx(&cfg, k, td, h->tm_r, h->tm_u, h->tm_v, h->tm_w, h->tm_t, A));
         LAUNCHED(h);
         return;
     }
@@ -818,6 +847,7 @@ void swap_delta(rfb_soc_handle* h) {
     std::swap(h->d_delta[0], h->d_delta[1]);
     if (h->tm_ready) {
         std::swap(h->tm_delta[0], h->tm_delta[1]);
+        std::swap(h->tmn_delta[0], h->tmn_delta[1]);
         std::swap(h->tm_delta_ptr[0], h->tm_delta_ptr[1]);
     }
 }
@@ -970,11 +1000,9 @@ std::map<TuneKey, TuneVal> g_tune_cache;
 std::mutex g_tune_mu;
 
 // Project-written autotuner for one lattice: time (twice, keeping the faster) 12 plain
-// sweeps and 12 sweeps of each
-// launch shape of the two-sweep pass (with local steps: with three and with four TMA
-// stages, and the three-sweep pass with four and five delta stages) by CUDA events on
-// the current forcing and keep the fastest (tb_only: choose between the pass variants
-// only).
+// sweeps and 12 sweeps of each launch shape of the two-sweep pass (with local steps: with
+// three and with four TMA stages, and with 64-column tiles) by CUDA events on the current
+// forcing and keep the fastest (tb_only: choose between the pass variants only).
 void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false) {
     if (!tb_eligible(h, op.dt_mode == RFB_DT_LOCAL)) { h->tb_mode = 0; return; }
     const TuneKey key{h->nx, h->ny, h->nz, h->d_m32 != nullptr,
@@ -990,13 +1018,17 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
             return;
         }
     }
-    // candidates: plain, then pass variants 0 .. nvar-1 (12 sweeps: whole passes of each)
-    const int nvar = op.dt_mode == RFB_DT_LOCAL ? 8 : 2;
-    float ms[9];
+    // candidates: plain (-1), then pass variants (12 sweeps: whole passes of each). Not the
+    // three-sweep passes: since passes overlap their ends the two-sweep ones are faster on every
+    // lattice measured (us per sweep of the best of each: 128x128x256 10.6 and 13.7, 160x160x200
+    // 18.8 and 23.2, 192^3 22.7 and 26.6, 256^3 41.0 and 42.3, 256x256x512 75 and 87).
+    std::vector<int> cands = {0, 1};
+    if (op.dt_mode == RFB_DT_LOCAL) cands = {0, 1, 2, 3, 8, 9};
+    float ms[10], plain_ms = INFINITY;
     for (float& m : ms) m = INFINITY;
-    for (int cand = tb_only ? 1 : 0; cand <= nvar; ++cand) {
-        if (cand > 0) h->tb_variant = cand - 1;
-        const Sweep32 how = cand > 0 ? Sweep32::pass : Sweep32::plain;
+    auto time_one = [&](int v, float& best) {
+        const Sweep32 how = v < 0 ? Sweep32::plain : Sweep32::pass;
+        if (v >= 0) h->tb_variant = v;
         sweeps32(h, op, 6, how);   // warm-up (and tensor maps)
         for (int rep = 0; rep < 2; ++rep) {   // the faster of two timings
             float t = 0.f;
@@ -1005,17 +1037,19 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
             CK(h, cudaEventRecord(h->ev[1], h->stream));
             CK(h, cudaEventSynchronize(h->ev[1]));
             CK(h, cudaEventElapsedTime(&t, h->ev[0], h->ev[1]));
-            ms[cand] = std::min(ms[cand], t);
+            best = std::min(best, t);
         }
-    }
+    };
+    if (!tb_only) time_one(-1, plain_ms);
+    for (int v : cands) time_one(v, ms[v]);
     int bestv = 0;
-    for (int v = 1; v < nvar; ++v)
-        if (ms[1 + v] < ms[1 + bestv]) bestv = v;
+    for (int v : cands)
+        if (ms[v] < ms[bestv]) bestv = v;
     h->tb_variant = bestv;
-    const float tb = ms[1 + bestv];
-    h->tb_tuned_plain_ms = ms[0] / 12;
+    const float tb = ms[bestv];
+    h->tb_tuned_plain_ms = tb_only ? INFINITY : plain_ms / 12;
     h->tb_tuned_tb_ms = tb / 12;
-    if (!tb_only) h->tb_mode = tb < ms[0] ? 1 : 0;
+    if (!tb_only) h->tb_mode = tb < plain_ms ? 1 : 0;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_cache[key] = TuneVal{tb_only ? -1 : h->tb_mode, h->tb_variant, h->tb_tuned_plain_ms,
                                 h->tb_tuned_tb_ms};
@@ -2543,7 +2577,7 @@ rfb_status rfb_soc_tuned_fp32_kernel(const rfb_soc_handle* h, int32_t* kernel,
     else if (h->tb_mode == 0) k = 1;
     else if (h->tb_mode == 1 || h->tb_variant >= 0) {
         const int v = std::max(h->tb_variant, 0);
-        k = (v & 4 ? (v & 2 ? 9 : 7) : (v & 2 ? 5 : 3)) + (v & 1);
+        k = (v >= 8 ? 12 : v & 4 ? (v & 2 ? 9 : 7) : (v & 2 ? 5 : 3)) + (v & 1);
     }
     if (kernel) *kernel = k;
     if (plain_ms_per_sweep) *plain_ms_per_sweep = h->tb_tuned_plain_ms;

@@ -382,18 +382,22 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
 // to 5.89 on 96x100x150, 12.29 to 10.63 on 128x128x256, 20.5 to 18.8 on 160x160x200 and 42.7
 // to 41.0 on 256^3: a block's barriers, tensor maps and first five fields are in place when
 // the pass before it ends, and the last partial wave overlaps them.
-template <bool TR, int NST>
-__global__ void __launch_bounds__(TB_THREADS, 1)
+//
+// TXI = 64 (three stages, two CTAs per SM): lattices that 128-column tiles cover badly (160
+// columns: two tiles hold 62 % lattice, three narrow ones 83 %): 160x160x200 18.7 -> 16.1 us
+// per sweep, 192^3 22.7 -> 19.0.
+template <bool TR, int NST, int TXI = 128>
+__global__ void __launch_bounds__(TBDGeom<TXI>::THREADS, TXI == 64 ? 2 : 1)
 sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constant__ CUtensorMap tm_r,
                   const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_v,
                   const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_t,
                   TBDArgs A) {
     extern __shared__ unsigned char smem_raw[];
     grid_release();
-    TBDRing<NST> R = tbd_ring_init<NST>(smem_raw, A.err);
+    TBDRing<NST, TXI> R = tbd_ring_init<NST, TXI>(smem_raw, A.err);
     const TBDField F{&tm_d, &tm_r, &tm_u, &tm_v, &tm_w, &tm_t, A.nx, A.ny, A.nz,
                      A.d_in, A.d_out, A.omc, A.Dh};
-    const int gx = (A.nx + TB_TXI - 1) / TB_TXI;
+    const int gx = (A.nx + TXI - 1) / TXI;
     const int tiles = gx * ((A.ny + TB_TYI - 1) / TB_TYI);
     const int64_t q1 = min((int64_t)(blockIdx.x + 1) * A.per, A.total);
     bool ok = true, first = true;
@@ -406,10 +410,10 @@ sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constan
         if (kb >= A.nz) { q = item_end; continue; }   // padding of a short last chunk
         const int ke = (int)min((int64_t)A.nz, kb + (min(q1, item_end) - q));
         q = min(q1, item_end);
-        ok = tbd_segment<TR, NST>(R, F, tile, kb, ke, first);
+        ok = tbd_segment<TR, NST, TXI>(R, F, tile, kb, ke, first);
         first = false;
     }
-    if (!ok) tbd_ring_drain<NST>(R);
+    if (!ok) tbd_ring_drain<NST, TXI>(R);
 }
 
 // ---------------------------------------------------------------------------------

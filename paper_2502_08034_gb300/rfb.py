@@ -402,7 +402,8 @@ class Solver:
         the lattice fits on the chip and nothing was timed)."""
         k, a, b = c_int32(), c_double(), c_double()
         self._check(lib().rfb_soc_tuned_fp32_kernel(self.h, byref(k), byref(a), byref(b)))
-        names = {0: None, 1: "plain", 11: "resident"}
+        names = {0: None, 1: "plain", 11: "resident", 12: "blocked_narrow_persistent",
+                 13: "blocked_narrow_chunked"}
         names.update({v: k for k, v in FP32_KERNEL.items() if v >= 3})
         return names[k.value], a.value, b.value
 
