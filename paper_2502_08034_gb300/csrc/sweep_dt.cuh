@@ -292,7 +292,11 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
 #pragma unroll
     for (int e = 0; e < 4; ++e)
         for (int s = 0; s < 6; ++s) kcB[e].a[s] = 0.f;
-    if (in_dom && kb >= 2) dB = ldg4(F.d_in + i0 + (int64_t)nx * j + nxny * (kb - 2));
+    // (from L2: the pass before may have written it after this launch began, and neither the
+    // read-only path nor a line left in L1 would show that)
+    if (in_dom && kb >= 2)
+        dB = __ldcg(reinterpret_cast<const float4*>(F.d_in + i0 + (int64_t)nx * j +
+                                                    nxny * (kb - 2)));
     bool good = R.wait(0);
     int s0 = 0;                                        // stage holding plane z
 
