@@ -80,6 +80,7 @@ struct rfb_soc_handle {
     OpPoint umt_op;
     double* d_eta = nullptr;      // Nernst model: eta~ on electrode cells (first use)
     int* d_elec = nullptr;        // Nernst model: electrode-cell list (+ count at [N])
+    double* d_ecells = nullptr;   // ... and what their steps need (n_elec x 3 doubles, 1 float)
     bool have_eta = false;
     double* d_lam[2] = {nullptr, nullptr};   // adjoint state (allocated on first use)
     double* d_g = nullptr;
@@ -1304,7 +1305,7 @@ rfb_status guard(rfb_soc_handle* h) {
 void free_all(rfb_soc_handle* h) {
     // the arena holds flags .. partials; the rest are allocated on first use
     void* ptrs[] = {h->d_arena, h->d_m,    h->d_m32,  h->d_lam[0], h->d_lam[1], h->d_g,
-                    h->d_grad,  h->d_L64,  h->d_L2F,  h->d_eta,    h->d_elec,   h->d_sdf[0],
+                    h->d_grad,  h->d_L64,  h->d_L2F,  h->d_eta,    h->d_elec,   h->d_ecells, h->d_sdf[0],
                     h->d_sdf[1], h->d_gdf,  h->d_stage,  h->d_bv,     h->d_bvpart,
                     h->res.inbox, h->res64.inbox, h->res_cg.inbox,
                     h->res_bv.inbox, h->cg_rows, h->cg_out};
@@ -1680,7 +1681,22 @@ rfb_status rfb_soc_solve_nernst(rfb_soc_handle* h, double s_in, double eta, doub
                               h->stream));
         CK(h, cudaStreamSynchronize(h->stream));
         ensure_L64(h, op);
+        NernstCells E{};
+        if (n_elec > 0) {
+            const size_t ne = (size_t)h->n_elec;
+            if (!h->d_ecells) dalloc(h, &h->d_ecells, 4 * ne);
+            E.b = h->d_ecells;
+            E.diag = E.b + ne;
+            E.hk = E.diag + ne;
+            E.ratio = reinterpret_cast<float*>(E.hk + ne);
+            nernst_cells_kernel<<<flat_grid(n_elec), 256, 0, h->stream>>>(
+                lattice(h), h->K, C, h->d_elec, n_elec, kap0, E);
+            LAUNCHED(h);
+        }
         const float* dtc = op.dt_mode == RFB_DT_LOCAL ? h->d_dtc : nullptr;
+        const int n_eb = (n_elec + NE_T - 1) / NE_T;
+        const int64_t n_blocks = n_eb + (int64_t)((h->nx + 31) / 32) * ((h->ny + 1) / 2) *
+                                            ((h->nz + 1) / 2);
         const int64_t every = o.check_every > 0 ? o.check_every : default_check_every(h, RFB_PREC_FP64);
         rfb_solve_result r{};
         rfb_status st = RFB_OK;
@@ -1702,16 +1718,10 @@ rfb_status rfb_soc_solve_nernst(rfb_soc_handle* h, double s_in, double eta, doub
             const int64_t n = std::min(every, o.max_sweeps - done);
             CK(h, cudaEventRecord(h->ev[0], h->stream));
             for (int64_t q = 0; q < n; ++q) {
-                nernst_interior_kernel<<<h->grid, h->block, 0, h->stream>>>(
-                    lattice(h), h->K, C, dtc, op.dt, h->d_s[h->s_cur], h->d_s[h->s_cur ^ 1],
-                    kap0, h->kchunk);
+                nernst_step_kernel<<<(unsigned)n_blocks, NE_T, 0, h->stream>>>(
+                    lattice(h), h->K, h->d_m, dtc, op.dt, h->d_s[h->s_cur],
+                    h->d_s[h->s_cur ^ 1], h->d_elec, n_elec, n_eb, E, h->d_eta, Vt, omega);
                 LAUNCHED(h);
-                if (n_elec > 0) {
-                    nernst_elec_kernel<<<flat_grid(n_elec), 256, 0, h->stream>>>(
-                        lattice(h), h->K, C, h->d_elec, n_elec, h->d_s[h->s_cur],
-                        h->d_s[h->s_cur ^ 1], h->d_eta, kap0, Vt, omega);
-                    LAUNCHED(h);
-                }
                 h->s_cur ^= 1;
             }
             CK(h, cudaEventRecord(h->ev[1], h->stream));

@@ -713,77 +713,112 @@ __global__ void nernst_list_kernel(Lattice L, Coef<double> C, double kap0,
     }
 }
 
-// Interior step: s_out = s + dt RHS(s) on unknown cells that are not electrode cells.
-__global__ void __launch_bounds__(BX * BY)
-nernst_interior_kernel(Lattice L, L64 K, Coef<double> C, const float* __restrict__ dtc,
-                       double dt_global, const double* __restrict__ s,
-                       double* __restrict__ s_out, double kap0, int kchunk) {
-    const int i = blockIdx.x * BX + threadIdx.x;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    if (i >= L.nx || j >= L.ny) return;
-    const int kb = blockIdx.z * kchunk;
-    const int ke = min(kb + kchunk, L.nz);
-    const int nx = L.nx, nxny = L.nxny;
-    const int64_t oxm = i > 0 ? -1 : 0, oxp = i + 1 < nx ? 1 : 0;
-    const int64_t oym = j > 0 ? -nx : 0, oyp = j + 1 < L.ny ? nx : 0;
-    int64_t c = (int64_t)i + (int64_t)nx * j + (int64_t)nxny * kb;
-    double s_prev = kb > 0 ? s[c - nxny] : 0.0;
-    double s_cur = s[c];
-    for (int k = kb; k < ke; ++k, c += nxny) {
-        const double s_next = (k + 1 < L.nz) ? s[c + nxny] : 0.0;
+// What an electrode cell's step needs beside its row's neighbour coefficients, in list order:
+// the transport part of its row (the source taken out), 1 / (2 k_c) and -d_T / k_c (FP32, for
+// the weight). Formed once per solve: the step then does no division by k_c.
+struct NernstCells {
+    double* __restrict__ b;        // source without the reaction
+    double* __restrict__ diag;     // diagonal without the reaction
+    double* __restrict__ hk;       // 1 / (2 k_c)
+    float* __restrict__ ratio;     // -(d_T / k_c)
+};
+
+__global__ void nernst_cells_kernel(Lattice L, L64 K, Coef<double> C,
+                                    const int* __restrict__ list, int n, double kap0,
+                                    NernstCells E) {
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        const int64_t c = list[q];
         const unsigned f = L.flags[c];
-        const bool elec = (f & F_ELEC) && (!C.m || C.m[c] > 0.0) && kap0 > 0.0;
-        if ((f & F_FLUID) && !elec) {
-            const double r = rhs64(K, c, s_cur, s[c + oxm], s[c + oxp], s[c + oym], s[c + oyp],
-                                   s_prev, s_next);
-            const double dt = dtc ? widen(dtc[c]) : dt_global;
-            s_out[c] = fma(dt, r, s_cur);
-        }
-        s_prev = s_cur;
-        s_cur = s_next;
+        const int nw = n_wall_of(f, (int)(c % L.nx), (int)((c / L.nx) % L.ny), (int)(c / L.nxny),
+                                 L.nx, L.ny, L.nz);
+        const double mult = C.m ? C.m[c] : 1.0, kc = mult * kap0 * nw;
+        const double dg = K.diag[c] + mult * C.rB[nw];
+        E.b[q] = K.b[c] - mult * C.rA[nw];
+        E.diag[q] = dg;
+        E.hk[q] = 0.5 / kc;
+        E.ratio[q] = (float)(dg / kc);
     }
 }
 
-// Electrode step over the list: T = RHS_SBV(s) - k_c (A - B s), eta~_I, the relaxed
-// eta~ update and s_out = sigma(V~ - eta~).
-__global__ void nernst_elec_kernel(Lattice L, L64 K, Coef<double> C,
-                                   const int* __restrict__ list, int n,
-                                   const double* __restrict__ s, double* __restrict__ s_out,
-                                   double* __restrict__ eta_t, double kap0, double Vt,
-                                   double omega) {
-    __shared__ double tA[8], tB[8];
-    if (threadIdx.x < 8) { tA[threadIdx.x] = C.rA[threadIdx.x]; tB[threadIdx.x] = C.rB[threadIdx.x]; }
-    __syncthreads();
+// One Nernst step, s -> s_out: blocks 0 .. n_eb-1 take 64 electrode cells of the list each (T,
+// eta~_I, the relaxed eta~ update and s_out = sigma(V~ - eta~)), the others a 32 x 2 tile of
+// two planes of the lattice (s + dt RHS(s) on the other unknown cells). The two read s and
+// write different cells, so one launch does both. Bound by the FP64 pipe: about 130 operations
+// an electrode cell (asinh, exp, two divisions, rsqrt), eight another; the electrode blocks
+// come first and small so that the tiles fill in behind them (us per step with blocks of 64,
+// 128, 256 threads: 48x48x96 14.4, 15, 17). Two launches a step before: 16x16x32 22.6 -> 8.2,
+// 48x48x96 24.6 -> 14.4, 96x80x120 49 -> 33. Overlapping the steps' launches made it 23.8 (the
+// waiting blocks take the places of running ones).
+constexpr int NE_T = 64;
+__global__ void __launch_bounds__(NE_T)
+nernst_step_kernel(Lattice L, L64 K, const double* __restrict__ m, const float* __restrict__ dtc,
+                   double dt_global, const double* __restrict__ s, double* __restrict__ s_out,
+                   const int* __restrict__ list, int n, int n_eb, NernstCells E,
+                   double* __restrict__ eta_t, double Vt, double omega) {
     const int nx = L.nx, ny = L.ny, nz = L.nz;
     const int64_t nxny = L.nxny;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+    if ((int)blockIdx.x < n_eb) {
+        const int q = blockIdx.x * NE_T + threadIdx.x;
+        if (q >= n) return;
         const int64_t c = list[q];
         const int i = (int)(c % nx);
         const int j = (int)((c / nx) % ny);
         const int k = (int)(c / nxny);
-        const double sc0 = s[c];
-        const double r = rhs64(K, c, sc0, s[c - (i > 0)], s[c + (i + 1 < nx)],
-                               s[c - (j > 0 ? nx : 0)], s[c + (j + 1 < ny ? nx : 0)],
-                               s[c - (k > 0 ? nxny : 0)], s[c + (k + 1 < nz ? nxny : 0)]);
-        const unsigned f = L.flags[c];
-        const int nw = n_wall_of(f, i, j, k, nx, ny, nz);
-        const double mult = C.m ? C.m[c] : 1.0;
-        const double kc = mult * kap0 * nw;
-        const double T = r - mult * (tA[nw] - tB[nw] * sc0);
-        const double dT = -K.diag[c] - mult * tB[nw];
-        const double sc = fmin(fmax(sc0, 1e-300), 1.0 - 0x1p-53);
-        const double root = sqrt(sc * (1.0 - sc));
-        const double e = eta_t[c];
-        const double ei = 2.0 * asinh(-T / (2.0 * kc * root));
+        const double dg = E.diag[q], b = E.b[q], hk = E.hk[q];
+        const float ratio = E.ratio[q];
+        double a[6];
+#pragma unroll
+        for (int f = 0; f < 6; ++f) a[f] = K.f[f][c];
+        const double sc0 = s[c], e = eta_t[c];
+        double T = fma(dg, sc0, b);
+        T = fma(a[0], s[c - (i > 0)], T);
+        T = fma(a[1], s[c + (i + 1 < nx)], T);
+        T = fma(a[2], s[c - (j > 0 ? nx : 0)], T);
+        T = fma(a[3], s[c + (j + 1 < ny ? nx : 0)], T);
+        T = fma(a[4], s[c - (k > 0 ? nxny : 0)], T);
+        T = fma(a[5], s[c + (k + 1 < nz ? nxny : 0)], T);
+        // s clamped into [1e-300, 1 - 2^-53], on the integer pipe
+        const long long lo = __double_as_longlong(1e-300), hi = __double_as_longlong(1.0 - 0x1p-53);
+        const long long sb = __double_as_longlong(sc0);
+        const double sc = __longlong_as_double(sb < lo ? lo : sb > hi ? hi : sb);
+        const double x = sc * (1.0 - sc);
+        const double ei = -2.0 * asinh(T * hk * rsqrt(x));
         // the relaxation weight only sets the step (the fixed point does not depend on
         // it): FP32, one exponential for sinh and cosh
+        const float root = sqrtf((float)x);
         const float ex = __expf(0.5f * (float)e), exi = 1.0f / ex;
-        const float G = (-(float)(dT / kc) * (float)root +
-                         (float)(1.0 - 2.0 * sc) * 0.5f * (ex - exi)) / (0.5f * (ex + exi));
-        const double w = omega / (1.0 + (double)fabsf(G));
+        const float G = (ratio * root + (float)(1.0 - 2.0 * sc) * 0.5f * (ex - exi)) /
+                        (0.5f * (ex + exi));
+        const double w = omega / (1.0 + widen(fabsf(G)));
         const double en = fma(w, ei - e, e);
         eta_t[c] = en;
         s_out[c] = sigmoid64(Vt - en);
+        return;
+    }
+    const int tile = blockIdx.x - n_eb, gx = (nx + 31) / 32, gy = (ny + 1) / 2;
+    const int i = tile % gx * 32 + (threadIdx.x & 31);
+    const int j = (tile / gx) % gy * 2 + (threadIdx.x >> 5);
+    if (i >= nx || j >= ny) return;
+    const int kb = tile / gx / gy * 2, ke = min(kb + 2, nz);
+    const int64_t oxm = i > 0 ? -1 : 0, oxp = i + 1 < nx ? 1 : 0;
+    const int64_t oym = j > 0 ? -nx : 0, oyp = j + 1 < ny ? nx : 0;
+    int64_t c = (int64_t)i + (int64_t)nx * j + nxny * kb;
+    unsigned f_next = L.flags[c];
+    double s_prev = kb > 0 ? s[c - nxny] : 0.0;
+    double s_cur = s[c];
+    for (int k = kb; k < ke; ++k, c += nxny) {
+        const double s_next = (k + 1 < nz) ? s[c + nxny] : 0.0;
+        const unsigned f = f_next;
+        if (k + 1 < ke) f_next = L.flags[c + nxny];
+        const bool elec = (f & F_ELEC) && (!m || positive(m[c]));
+        if ((f & F_FLUID) && !elec) {
+            const float dtl = dtc ? dtc[c] : 0.f;
+            const double r = rhs64(K, c, s_cur, s[c + oxm], s[c + oxp], s[c + oym], s[c + oyp],
+                                   s_prev, s_next);
+            s_out[c] = fma(dtc ? widen(dtl) : dt_global, r, s_cur);
+        }
+        s_prev = s_cur;
+        s_cur = s_next;
     }
 }
 
