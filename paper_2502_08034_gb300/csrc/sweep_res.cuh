@@ -15,18 +15,26 @@
 // store-to-load latency and one block barrier instead of a launch, with no fence and no
 // grid-wide barrier.
 //
+// The first warps own the brick's outer columns (the edge group). They alone wait for the side
+// faces, behind a barrier of their own, and send theirs while the other warps work on the
+// inside, which waits for its z words only after the cells that need none. So the time of a
+// word on its way hides behind the inside: with one order for all warps 64^3 took 1.17 us a
+// sweep, 75x61x118 1.90; now 0.94 and 1.62 (the smallest bricks, one warp, 0.78 and 0.82).
+//
 // Inboxes have two slots (sweep parity). A CTA overwrites the slot of sweep v with sweep
 // v + 2 only after it computed v + 2, which needed the neighbour's words of v + 1, and the
-// neighbour sends those after the barrier that follows its reads of v (the z faces pair
-// thread with thread and need no barrier). Tags grow from launch to launch (the handle keeps
-// the count), so a slot is never cleared.
+// neighbour sends those after its edge group's barrier that follows its reads of v (the z faces
+// pair thread with thread and need no barrier). Side faces go to the copy that the sweep
+// reads, into places that the edge group alone uses. Tags grow from launch to launch (the
+// handle keeps the count), so a slot is never cleared.
 //
 // Every update is dt_coef and dt_update with the operands and the order of the one-sweep
 // kernel, so n sweeps here are bitwise n launches of sweep32d_kernel.
 //
-// Measured (us per sweep in cycles of 200; launches before, resident now): 16x16x32 6.2 and
-// 0.83, 64^3 6.2 and 1.28, 80x60x110 6.2 and 1.91. About 0.75 us of it is the word latency
-// (the smallest lattices); the rest is the shared-memory and issue time of a CTA's cells.
+// Measured (us per sweep, 2000 a launch; launches before, resident now): 16x16x32 6.2 and
+// 0.82, 64^3 6.2 and 0.94, 80x60x110 6.2 and 1.70, 88x88x108 6.4 and 2.41. About 0.75 us of it
+// is the word latency (the smallest lattices); the rest is the shared-memory and issue time of
+// a CTA's cells.
 #pragma once
 
 #include "sweep_dt.cuh"
@@ -35,10 +43,9 @@ namespace rfb {
 
 constexpr int RES_T = 512;         // most threads of a CTA, columns of a brick (a launch has
                                    // the whole warps that its bricks need)
-constexpr int RES_RING = 2;        // pairs of x / y halo words polled per thread, at most
+constexpr int RES_RING = 4;        // pairs of x / y halo words polled per edge thread, at most
 // Shared memory of one plane of the brick: its rows without padding, one row below and one
-// above (a column's index is its thread's, so a warp's accesses never share a bank), then as
-// much again for the columns left and right of the brick, each at its neighbour's index (the
+// above (a warp's columns of one row never share a bank), then as much again for the columns left and right of the brick, each at its neighbour's index (the
 // bank that its reader leaves free). With padded rows of bx + 2 every access of a warp that
 // spans two rows took two turns: 528k cells 1.96 us a sweep. The pitch is fixed, so that a
 // column's cells are immediate offsets and take no address registers.
@@ -51,6 +58,7 @@ struct ResArgs {
     int nx, ny, nz;
     int bx, by;                    // columns of a brick (its planes: CPT)
     int gx, gy, gz;                // bricks
+    int edge;                      // threads of the edge group (whole warps, the first ones)
     const float* __restrict__ u;   // FP32 face velocities * beta / h (low faces)
     const float* __restrict__ v;
     const float* __restrict__ w;   // nz + 1 planes
@@ -70,9 +78,10 @@ struct ResArgs {
 __host__ __device__ constexpr int res_stride(int cpt, int bx, int by) {
     return 2 * RES_T + 2 * cpt * (bx + by);
 }
-// From ten cells a column dt r is kept in shared memory (its own words only): the weights of
-// ten or twelve cells and dt r spill at 128 registers a thread (148 bytes at twelve).
-__host__ __device__ constexpr bool res_dtr_shared(int cpt) { return cpt >= 10; }
+// From eight cells a column dt r is kept in shared memory (its own words only): the weights of
+// eight cells and dt r spill at 128 registers a thread (80x60x110 1.77 us a sweep, without the
+// spills 1.70; ten and twelve cells still spill 88 and 204 bytes).
+__host__ __device__ constexpr bool res_dtr_shared(int cpt) { return cpt >= 8; }
 // bytes of the two copies of a brick and its ring of neighbour columns, then dt r
 __host__ __device__ constexpr int res_smem(int cpt) {
     return (2 * cpt * RES_PLANE + (res_dtr_shared(cpt) ? cpt * RES_T : 0)) * (int)sizeof(float);
@@ -103,6 +112,31 @@ __device__ __forceinline__ void res_peek2(const unsigned long long* p,
                  : "memory");
 }
 
+// Column (x, y) of thread t in a brick of bx x by: the rows y = 0 and y = by - 1, then the rest of
+// the columns x = 0 and x = bx - 1, then the inside.
+__device__ __forceinline__ void res_column(int t, int bx, int by, int& x, int& y) {
+    x = y = 0;
+    if (t >= bx * by) return;                          // no column
+    if (t < 2 * bx) {
+        y = t < bx ? 0 : by - 1;
+        x = t < bx ? t : t - bx;
+        return;
+    }
+    t -= 2 * bx;
+    if (t < 2 * (by - 2)) {
+        y = 1 + (t >> 1);
+        x = t & 1 ? bx - 1 : 0;
+        return;
+    }
+    t -= 2 * (by - 2);
+    y = 1 + t / (bx - 2);                              // bx > 2 here
+    x = 1 + t % (bx - 2);
+}
+// barrier of the edge group alone (whole warps)
+__device__ __forceinline__ void res_edge_sync(int threads) {
+    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
 template <int CPT, bool TR>   // CPT even
 __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
     extern __shared__ float res_s[];
@@ -111,8 +145,10 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
     constexpr int plane = RES_PLANE, copy = CPT * RES_PLANE;
     const int b = blockIdx.x;
     const int ix = b % A.gx, iy = (b / A.gx) % A.gy, iz = b / (A.gx * A.gy);
-    const int x = t % bx, y = t / bx;
-    const bool mine = y < by;                          // owns a column
+    int x, y;
+    res_column(t, bx, by, x, y);
+    const bool mine = t < bx * by;                     // owns a column
+    const bool edge = t < A.edge;                      // of the edge group (whole warps)
     const int i = ix * bx + x, j = iy * by + y, k0 = iz * CPT;
     for (int q = t; q < 2 * copy; q += (int)blockDim.x) res_s[q] = 0.f;
 
@@ -143,30 +179,32 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
     }
 
     // halo words of this thread: the two z faces of its column (bits 0 and 1 of `want`, set
-    // where there is a neighbour) and up to RES_RING pairs of the x and y faces (bits 2, ..)
+    // where there is a neighbour) and, in the edge group, up to RES_RING pairs of the x and y
+    // faces (bits 2, ..)
     const int nfx = CPT * by, nfy = CPT * bx;          // words of one x face, one y face (a
                                                        // column's CPT words together)
     uint32_t want = 0;
     if (mine && iz > 0) want |= 1u;
     if (mine && iz + 1 < A.gz) want |= 2u;
-    int dst[RES_RING];
+    uint32_t dst[RES_RING / 2] = {};                   // two 16-bit indices each
 #pragma unroll
     for (int m = 0; m < RES_RING; ++m) {
-        int q = 2 * (t + m * (int)blockDim.x);
-        dst[m] = 0;
-        if (q >= 2 * (nfx + nfy)) continue;
+        int q = 2 * (t + m * A.edge);
+        if (!edge || q >= 2 * (nfx + nfy)) continue;
+        int at;
         if (q < 2 * nfx) {
             const bool hi = q >= nfx;
             if (hi) q -= nfx;
-            dst[m] = (q % CPT) * plane + RES_ROWS + (q / CPT + 1) * bx + (hi ? bx : -1);
+            at = (q % CPT) * plane + RES_ROWS + (q / CPT + 1) * bx + (hi ? bx : -1);
             if (hi ? ix + 1 < A.gx : ix > 0) want |= 4u << m;
         } else {
             q -= 2 * nfx;
             const bool hi = q >= nfy;
             if (hi) q -= nfy;
-            dst[m] = (q % CPT) * plane + (hi ? by + 1 : 0) * bx + q / CPT;
+            at = (q % CPT) * plane + (hi ? by + 1 : 0) * bx + q / CPT;
             if (hi ? iy + 1 < A.gy : iy > 0) want |= 4u << m;
         }
+        dst[m / 2] |= (uint32_t)at << 16 * (m & 1);
     }
     // words this column sends to, from slot 0 (-1: no neighbour there; a brick is at least
     // two columns wide each way, so a column is on one x face and one y face at most)
@@ -181,7 +219,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
         if (y == 0 && iy > 0) to_y = box(b - A.gx) + 2 * RES_T + 2 * nfx + nfy + x * CPT;
         if (y == by - 1 && iy + 1 < A.gy) to_y = box(b + A.gx) + 2 * RES_T + 2 * nfx + x * CPT;
     }
-    const int o = bx + t;                              // this column in a plane, its x neighbours
+    const int o = bx + y * bx + x;                     // this column in a plane, its x neighbours
     const int oxm = x == 0 ? RES_ROWS + o - 1 : o - 1;
     const int oxp = x == bx - 1 ? RES_ROWS + o + 1 : o + 1;
     float zlo = 0.f, zhi = 0.f;                        // values below and above the column
@@ -207,47 +245,12 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
         }
         __syncthreads();
     }
-    for (int ver = 1; ver <= A.n; ++ver) {
-        const float* Sr = res_s + ((ver - 1) & 1) * copy;       // the brick before this sweep
-        float* Sh = res_s + (ver & 1) * copy;                   // and after
-        float* Sw = Sh + o;
-        const uint32_t tag = A.tag + (uint32_t)ver;
-        unsigned long long* const slot = A.inbox + (ver & 1) * A.stride;
-        const bool more = ver < A.n;
-        if (mine) {
-            // every value first (loads and arithmetic of the cells overlap), then the words,
-            // then the brick's copy
-            float prev = zlo;
-#pragma unroll
-            for (int e = 0; e < CPT; ++e) {
-                const int q = e * plane;
-                const float val = dt_update(
-                    kc[e], A.omc, d[e], DTR_S ? dtr_s[e * RES_T] : dtr[DTR_S ? 0 : e], Sr[q + oxm],
-                    Sr[q + oxp], Sr[q + o - bx], Sr[q + o + bx], prev, e + 1 < CPT ? d[e + 1 < CPT ? e + 1 : e] : zhi);
-                prev = d[e];
-                d[e] = val;
-            }
-            if (more) {
-                if (to_zm >= 0) res_send(slot + to_zm, d[0], tag);
-                if (to_zp >= 0) res_send(slot + to_zp, d[CPT - 1], tag);
-                if (to_x >= 0) {
-#pragma unroll
-                    for (int e = 0; e < CPT; e += 2) res_send2(slot + to_x + e, d[e], d[e + 1], tag);
-                }
-                if (to_y >= 0) {
-#pragma unroll
-                    for (int e = 0; e < CPT; e += 2) res_send2(slot + to_y + e, d[e], d[e + 1], tag);
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < CPT; ++e) Sw[e * plane] = d[e];
-        }
-        if (!more) break;
-        // wait for the neighbours' words of this sweep
-        uint32_t pend = good ? want : 0u;
-        __syncwarp();                  // the warp's own words are sent before it starts polling
-        const unsigned long long* in = slot + own;
-        // a warp stays together until all its lanes have their words
+    // the words of sweep ver - 1 this thread waits for (of `which`): z values into zlo and zhi,
+    // side faces into the brick's copy; a warp stays together until all its lanes have theirs
+    auto take = [&](int ver, uint32_t which, float* Sr) {
+        const uint32_t tag = A.tag + (uint32_t)(ver - 1);
+        const unsigned long long* in = A.inbox + ((ver - 1) & 1) * A.stride + own;
+        uint32_t pend = good ? want & which : 0u;
         for (unsigned spin = 0; __any_sync(0xffffffffu, pend != 0u); ++spin) {
             unsigned long long zw[2], word[RES_RING][2];
 #pragma unroll
@@ -255,7 +258,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
                 if (pend & (1u << m)) zw[m] = res_peek(in + t + m * RES_T);
 #pragma unroll
             for (int m = 0; m < RES_RING; ++m)
-                if (pend & (4u << m)) res_peek2(in + 2 * RES_T + 2 * (t + m * (int)blockDim.x), word[m]);
+                if (pend & (4u << m)) res_peek2(in + 2 * RES_T + 2 * (t + m * A.edge), word[m]);
             if ((pend & 1u) && (uint32_t)(zw[0] >> 32) == tag) {
                 zlo = __uint_as_float((uint32_t)zw[0]);
                 pend &= ~1u;
@@ -268,8 +271,9 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
             for (int m = 0; m < RES_RING; ++m)
                 if ((pend & (4u << m)) && (uint32_t)(word[m][0] >> 32) == tag &&
                     (uint32_t)(word[m][1] >> 32) == tag) {
-                    Sh[dst[m]] = __uint_as_float((uint32_t)word[m][0]);
-                    Sh[dst[m] + plane] = __uint_as_float((uint32_t)word[m][1]);
+                    const uint32_t at = dst[m / 2] >> 16 * (m & 1) & 0xffffu;
+                    Sr[at] = __uint_as_float((uint32_t)word[m][0]);
+                    Sr[at + plane] = __uint_as_float((uint32_t)word[m][1]);
                     pend &= ~(4u << m);
                 }
             if (spin >= RES_SPIN_LIMIT && pend) {      // give up, and wait no more
@@ -278,7 +282,54 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
                 pend = 0;
             }
         }
-        __syncthreads();
+    };
+    for (int ver = 1; ver <= A.n; ++ver) {
+        float* Sr = res_s + ((ver - 1) & 1) * copy;             // the brick before this sweep
+        float* Sw = res_s + (ver & 1) * copy + o;               // and after
+        const uint32_t tag = A.tag + (uint32_t)ver;
+        unsigned long long* const slot = A.inbox + (ver & 1) * A.stride;
+        const bool more = ver < A.n;
+        if (edge && ver > 1) {
+            take(ver, ~0u, Sr);
+            res_edge_sync(A.edge);                     // other threads' side words
+        }
+        auto update = [&](int e, float zm, float zp) {
+            const int q = e * plane;
+            return dt_update(kc[e], A.omc, d[e], DTR_S ? dtr_s[e * RES_T] : dtr[DTR_S ? 0 : e],
+                             Sr[q + oxm], Sr[q + oxp], Sr[q + o - bx], Sr[q + o + bx], zm, zp);
+        };
+        // the inside of the column, then (its z words may have come meanwhile) its ends
+        const float second = d[1], second_last = d[CPT - 2];
+        float prev = d[0];
+#pragma unroll
+        for (int e = 1; e < CPT - 1; ++e) {
+            const float val = update(e, prev, d[e + 1]);
+            prev = d[e];
+            d[e] = val;
+        }
+        if (!edge && ver > 1) take(ver, 3u, Sr);
+        const float lo = update(0, zlo, second), hi = update(CPT - 1, second_last, zhi);
+        d[0] = lo;
+        d[CPT - 1] = hi;
+        if (more) {
+            if (to_zm >= 0) res_send(slot + to_zm, lo, tag);
+            if (to_zp >= 0) res_send(slot + to_zp, hi, tag);
+            if (edge) {
+                if (to_x >= 0) {
+#pragma unroll
+                    for (int e = 0; e < CPT; e += 2) res_send2(slot + to_x + e, d[e], d[e + 1], tag);
+                }
+                if (to_y >= 0) {
+#pragma unroll
+                    for (int e = 0; e < CPT; e += 2) res_send2(slot + to_y + e, d[e], d[e + 1], tag);
+                }
+            }
+            if (mine) {
+#pragma unroll
+                for (int e = 0; e < CPT; ++e) Sw[e * plane] = d[e];
+            }
+            __syncthreads();
+        }
     }
     if (in_xy) {
 #pragma unroll
@@ -295,13 +346,15 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
 // so the whole warps a cut takes decide its time and shared memory costs nothing beside it.
 // Operands and order are those of sweep64c_kernel and adjoint64c_kernel: bitwise the same.
 //
-// Measured (us per sweep, launches before and resident now): 16x16x32 8.2 and 1.6, 32x32x64 8.2
-// and 2.0, 48x48x96 10.3 and 4.6, 64^3 10.2 and 5.7, 60x60x110 12.3 and 7.9.
+// Measured (us per sweep, launches before and resident now): 16x16x32 8.2 and 1.6, 48^3 8.2 and
+// 2.3, 48x48x96 10.3 and 3.7, 64^3 10.2 and 4.6, 60x60x110 12.3 and 6.5 (one order for all warps,
+// as above: 1.5, 2.5, 4.6, 5.6, 7.9).
 // ---------------------------------------------------------------------------------
-constexpr int RES64_RING = 3;      // x / y halo values polled per thread, at most
+constexpr int RES64_RING = 4;      // x / y halo values polled per edge thread, at most
 // coefficients of a cell kept in shared memory (the last ones; registers hold the others):
-// eight doubles for five or six cells do not fit beside the values at 128 registers
-__host__ __device__ constexpr int res64_shared(int cpt) { return cpt >= 6 ? 3 : cpt >= 5 ? 2 : 0; }
+// eight doubles for three to six cells do not fit beside the values at 128 registers (48x48x96
+// 3.79 us a sweep with none of four cells' in shared memory, 3.65 with two a cell)
+__host__ __device__ constexpr int res64_shared(int cpt) { return cpt >= 6 ? 4 : cpt >= 5 ? 3 : cpt >= 4 ? 2 : cpt >= 3 ? 1 : 0; }
 __host__ __device__ constexpr int res64_smem(int cpt) {
     return (2 * cpt * RES_PLANE + cpt * res64_shared(cpt) * RES_T) * (int)sizeof(double);
 }
@@ -312,7 +365,7 @@ __host__ __device__ constexpr int res64_stride(int cpt, int bx, int by) {
 
 struct Res64Args {
     Lattice L;
-    int bx, by, gx, gy, gz;        // as in ResArgs
+    int bx, by, gx, gy, gz, edge;  // as in ResArgs
     L64 K;
     const float* __restrict__ dtc; // per-cell step, nullptr: dt
     double dt;
@@ -349,13 +402,13 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
     const int bx = A.bx, by = A.by;
     const int b = blockIdx.x;
     const int ix = b % A.gx, iy = (b / A.gx) % A.gy, iz = b / (A.gx * A.gy);
-    const int x = t % bx, y = t / bx;
+    int x, y;
+    res_column(t, bx, by, x, y);
+    const bool edge = t < A.edge;
     const int i = ix * bx + x, j = iy * by + y, k0 = iz * CPT;
     const int64_t nxny = A.L.nxny, N = nxny * nz;
     const int64_t c0 = i + (int64_t)nx * j + nxny * k0;
-    // every column of the brick runs (one outside the lattice holds 0 and is not updated),
-    // except whole warps of threads without one
-    const bool mine = y < by;
+    const bool mine = t < bx * by;
     const bool in_xy = mine && i < nx && j < ny;
 
     // coefficients in the order of use: diagonal, source, then the six neighbours
@@ -414,24 +467,25 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
     uint32_t want = 0;
     if (mine && iz > 0) want |= 1u;
     if (mine && iz + 1 < A.gz) want |= 2u;
-    int dst[RES64_RING];
+    uint32_t dst[RES64_RING / 2] = {};                   // two 16-bit indices each
 #pragma unroll
     for (int m = 0; m < RES64_RING; ++m) {
-        int q = t + m * (int)blockDim.x;
-        dst[m] = 0;
-        if (q >= 2 * (nfx + nfy)) continue;
+        int q = t + m * A.edge;
+        if (!edge || q >= 2 * (nfx + nfy)) continue;
+        int at;
         if (q < 2 * nfx) {
             const bool hi = q >= nfx;
             if (hi) q -= nfx;
-            dst[m] = (q % CPT) * plane + RES_ROWS + (q / CPT + 1) * bx + (hi ? bx : -1);
+            at = (q % CPT) * plane + RES_ROWS + (q / CPT + 1) * bx + (hi ? bx : -1);
             if (hi ? ix + 1 < A.gx : ix > 0) want |= 4u << m;
         } else {
             q -= 2 * nfx;
             const bool hi = q >= nfy;
             if (hi) q -= nfy;
-            dst[m] = (q % CPT) * plane + (hi ? by + 1 : 0) * bx + q / CPT;
+            at = (q % CPT) * plane + (hi ? by + 1 : 0) * bx + q / CPT;
             if (hi ? iy + 1 < A.gy : iy > 0) want |= 4u << m;
         }
+        dst[m / 2] |= (uint32_t)at << 16 * (m & 1);
     }
     auto box = [&](int c) { return c * 2 * A.stride; };
     const int own = box(b);
@@ -444,70 +498,21 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
         if (y == 0 && iy > 0) to_y = box(b - A.gx) + 2 * RES_T + 2 * nfx + nfy + x * CPT;
         if (y == by - 1 && iy + 1 < A.gy) to_y = box(b + A.gx) + 2 * RES_T + 2 * nfx + x * CPT;
     }
-    const int o = bx + t;
+    const int o = bx + y * bx + x;
     const int oxm = x == 0 ? RES_ROWS + o - 1 : o - 1;
     const int oxp = x == bx - 1 ? RES_ROWS + o + 1 : o + 1;
     bool good = true;
     __syncthreads();
-    for (int ver = 1; ver <= A.n; ++ver) {
-        const double* Sr = res_s64 + ((ver - 1) & 1) * copy;
-        double* Sh = res_s64 + (ver & 1) * copy;
-        const uint32_t tag = A.tag + (uint32_t)ver;
-        unsigned long long* const slot = A.inbox + 2 * ((ver & 1) * A.stride);
-        const bool more = ver < A.n;
-        if (mine) {
-            auto coef = [&](int e, int m) {
-                return m < NR ? kr[e][m < NR ? m : 0] : ks[(e * NS + m - NR) * RES_T];
-            };
-            auto update = [&](int e, double zm, double zp) {
-                const double* P = Sr + e * plane;
-                double r = fma(coef(e, 0), d[e], coef(e, 1));
-                r = fma(coef(e, 2), P[oxm], r);
-                r = fma(coef(e, 3), P[oxp], r);
-                r = fma(coef(e, 4), P[o - bx], r);
-                r = fma(coef(e, 5), P[o + bx], r);
-                r = fma(coef(e, 6), zm, r);
-                r = fma(coef(e, 7), zp, r);
-                const double val = fma(dt[e], r, d[e]);
-                return (upd >> e) & 1u ? val : d[e];
-            };
-            // the z faces first: their words travel while the other cells are computed
-            const double lo = update(0, zlo, d[1]);
-            if (more && to_zm >= 0) res_send64(slot + 2 * to_zm, lo, tag);
-            const double hi = update(CPT - 1, d[CPT - 2], zhi);
-            if (more && to_zp >= 0) res_send64(slot + 2 * to_zp, hi, tag);
-            double prev = d[0];
-            d[0] = lo;
-#pragma unroll
-            for (int e = 1; e < CPT - 1; ++e) {
-                const double val = update(e, prev, d[e + 1]);
-                prev = d[e];
-                d[e] = val;
-            }
-            d[CPT - 1] = hi;
-            if (more && to_x >= 0) {
-#pragma unroll
-                for (int e = 0; e < CPT; ++e) res_send64(slot + 2 * (to_x + e), d[e], tag);
-            }
-            if (more && to_y >= 0) {
-#pragma unroll
-                for (int e = 0; e < CPT; ++e) res_send64(slot + 2 * (to_y + e), d[e], tag);
-            }
-#pragma unroll
-            for (int e = 0; e < CPT; ++e) Sh[e * plane + o] = d[e];
-        }
-        if (!more) break;
-        uint32_t pend = good ? want : 0u;
-        __syncwarp();                  // the warp's own words are sent before it starts polling
-        const unsigned long long* in = slot + 2 * own;
-        // a warp stays together until all its lanes have their words
+    auto take = [&](int ver, uint32_t which, double* Sr) {
+        const uint32_t tag = A.tag + (uint32_t)(ver - 1);
+        const unsigned long long* in = A.inbox + 2 * (((ver - 1) & 1) * A.stride + own);
+        uint32_t pend = good ? want & which : 0u;
         for (unsigned spin = 0; __any_sync(0xffffffffu, pend != 0u); ++spin) {
             unsigned long long word[2 + RES64_RING][2];
 #pragma unroll
             for (int m = 0; m < 2 + RES64_RING; ++m)
                 if (pend & (1u << m))
-                    res_peek2(in + 2 * (m < 2 ? t + m * RES_T
-                                              : 2 * RES_T + t + (m - 2) * (int)blockDim.x),
+                    res_peek2(in + 2 * (m < 2 ? t + m * RES_T : 2 * RES_T + t + (m - 2) * A.edge),
                               word[m]);
 #pragma unroll
             for (int m = 0; m < 2 + RES64_RING; ++m) {
@@ -515,7 +520,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
                 if ((pend & (1u << m)) && res_take64(word[m], tag, &val)) {
                     if (m == 0) zlo = val;
                     else if (m == 1) zhi = val;
-                    else Sh[dst[m >= 2 ? m - 2 : 0]] = val;
+                    else Sr[dst[m >= 2 ? (m - 2) / 2 : 0] >> 16 * (m & 1) & 0xffffu] = val;
                     pend &= ~(1u << m);
                 }
             }
@@ -525,7 +530,68 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
                 pend = 0;
             }
         }
-        __syncthreads();
+    };
+    for (int ver = 1; ver <= A.n; ++ver) {
+        double* Sr = res_s64 + ((ver - 1) & 1) * copy;
+        double* Sw = res_s64 + (ver & 1) * copy + o;
+        const uint32_t tag = A.tag + (uint32_t)ver;
+        unsigned long long* const slot = A.inbox + 2 * ((ver & 1) * A.stride);
+        const bool more = ver < A.n;
+        if (edge && ver > 1) {
+            take(ver, ~0u, Sr);
+            res_edge_sync(A.edge);
+        }
+        auto coef = [&](int e, int m) {
+            return m < NR ? kr[e][m < NR ? m : 0] : ks[(e * NS + m - NR) * RES_T];
+        };
+        auto update = [&](int e, double zm, double zp) {
+            const double* P = Sr + e * plane;
+            double r = fma(coef(e, 0), d[e], coef(e, 1));
+            r = fma(coef(e, 2), P[oxm], r);
+            r = fma(coef(e, 3), P[oxp], r);
+            r = fma(coef(e, 4), P[o - bx], r);
+            r = fma(coef(e, 5), P[o + bx], r);
+            r = fma(coef(e, 6), zm, r);
+            r = fma(coef(e, 7), zp, r);
+            const double val = fma(dt[e], r, d[e]);
+            return (upd >> e) & 1u ? val : d[e];
+        };
+        const bool work = (t & ~31) < bx * by;         // a warp without columns does no FP64
+        const double second = d[1], second_last = d[CPT - 2];
+        if (work) {
+            double prev = d[0];
+#pragma unroll
+            for (int e = 1; e < CPT - 1; ++e) {
+                const double val = update(e, prev, d[e + 1]);
+                prev = d[e];
+                d[e] = val;
+            }
+        }
+        if (!edge && ver > 1) take(ver, 3u, Sr);
+        if (work) {
+            const double lo = update(0, zlo, second), hi = update(CPT - 1, second_last, zhi);
+            d[0] = lo;
+            d[CPT - 1] = hi;
+        }
+        if (more) {
+            if (to_zm >= 0) res_send64(slot + 2 * to_zm, d[0], tag);
+            if (to_zp >= 0) res_send64(slot + 2 * to_zp, d[CPT - 1], tag);
+            if (edge) {
+                if (to_x >= 0) {
+#pragma unroll
+                    for (int e = 0; e < CPT; ++e) res_send64(slot + 2 * (to_x + e), d[e], tag);
+                }
+                if (to_y >= 0) {
+#pragma unroll
+                    for (int e = 0; e < CPT; ++e) res_send64(slot + 2 * (to_y + e), d[e], tag);
+                }
+            }
+            if (mine) {
+#pragma unroll
+                for (int e = 0; e < CPT; ++e) Sw[e * plane] = d[e];
+            }
+            __syncthreads();
+        }
     }
     if (in_xy) {
 #pragma unroll
