@@ -48,7 +48,7 @@ def pass_kernel(kname):
                        shape, 5 if kname.startswith("three_sweep5") else 4))
     return 2, ("sweep32tbd_kernel (two-sweep TMA-staged pass, %s launch, %d TMA stages%s)" % (
         shape, 4 if kname.startswith("blocked4") else 3,
-        ", 64-column tiles" if "narrow" in kname else ""))
+        ", narrow tiles" if "narrow" in kname else ""))
 FALLBACK_HBM_GBS = 6800.0
 
 
@@ -408,8 +408,9 @@ def run_batch(args):
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak, "traffic": None,
                         "kernel": ("batch_tbd_kernel (two-sweep pass over all 48 lattices, "
-                                   "%d-column tiles, %d TMA stages)" % (
-                                       info["pass_tile_cols"], info["pass_stages"])
+                                   "%s tiles, %d TMA stages)" % (
+                                       "narrow" if info["pass_tile_cols"] == 64
+                                       else "128-column", info["pass_stages"])
                                    if passes else
                                    "batch_sweep_kernel (one sweep of all 48 lattices)"),
                         "note": "per sweep: algorithmic bytes of a launch / launches per sweep",

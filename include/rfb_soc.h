@@ -361,10 +361,11 @@ typedef struct rfb_batch_info {
                                   converged); with a timeout, one cycle per launch */
     int32_t pass_stages;       /* 0: the one-sweep kernel ran; 3 / 4: the batched two-sweep
                                   pass with that many TMA stages */
-    int32_t pass_chunk;        /* z planes per work item of the two-sweep pass */
-    int32_t pass_tile_cols;    /* interior columns of a tile of the two-sweep pass: 128 (one
-                                  CTA per SM), or 64 (two CTAs per SM; narrow lattices waste
-                                  less of a tile); 0 with the one-sweep kernel */
+    int32_t pass_chunk;        /* z planes of a chunk of the two-sweep pass (its CTAs take
+                                  equal runs of the lattices' chunks) */
+    int32_t pass_tile_cols;    /* tiles of the two-sweep pass: 128 (interior columns; one CTA
+                                  per SM), or 64 (narrow tiles cut to each lattice, two CTAs
+                                  per SM); 0 with the one-sweep kernel */
     int32_t df_cycles;         /* cycles whose defects were formed in double-float (FP32
                                   pairs, as in a single mixed solve), before the states
                                   were joined and checked in FP64; the rest of the cycles
@@ -381,9 +382,9 @@ rfb_status rfb_soc_batch_create(rfb_soc_handle* const* hs, int n, rfb_batch** ou
  * dt_mode, inlet_bc, max_sweeps (per lattice) and check_every (0 = autotuned) apply to
  * all. opts.fp32_kernel: 0 = the faster of the one-sweep kernel over every lattice and
  * the batched two-sweep TMA pass (local steps only; timed once per batch), 1 = the
- * one-sweep kernel, 2 = the two-sweep pass with the tile width (128 or 64 columns), TMA
+ * one-sweep kernel, 2 = the two-sweep pass with the tile width (128 columns or narrow), TMA
  * stage count and z chunk timed, 3..6 = the two-sweep pass with 128-column tiles, 7 / 8 =
- * with 64-column tiles (two CTAs per SM); 2..8 give RFB_ERR_INVALID_ARG with the global
+ * with narrow tiles (two CTAs per SM); 2..8 give RFB_ERR_INVALID_ARG with the global
  * step, larger values always. With the two-sweep pass the sweeps per cycle are a multiple
  * of 4. The defects of the cycles are formed in double-float until every lattice has
  * reached its tol or, where tol lies below what double-float defects resolve (10 x tau
@@ -528,7 +529,7 @@ rfb_status rfb_selftest_bounded_wait(int64_t spin_limit, int32_t* gave_up);
  * chosen yet, 1 = one sweep per launch, 3 / 4 = two-sweep passes in the persistent /
  * chunked launch shape, 5 / 6 the same with four TMA stages, 7 .. 10 three-sweep passes,
  * 11 = resident sweeps (fp32_kernel = 0 on a lattice that fits on the chip), 12 / 13 =
- * two-sweep passes with 64-column tiles, persistent / chunked (chosen by timing only);
+ * two-sweep passes with narrow tiles, persistent / chunked (chosen by timing only);
  * and the timed device milliseconds per sweep of the one-sweep kernel and of the fastest
  * pass variant (0 if not timed). Any output pointer may be NULL. */
 rfb_status rfb_soc_tuned_fp32_kernel(const rfb_soc_handle* h, int32_t* kernel,

@@ -132,15 +132,16 @@ struct rfb_soc_handle {
         int64_t per = 0;      // positions per CTA
         dim3 grid;
     } tb_launch[6];           // 2, 3: the same shapes for the three-sweep pass; 4, 5: for the
-                              // two-sweep pass with 64-column tiles (two CTAs per SM)
+                              // two-sweep pass with narrow tiles (two CTAs per SM)
     int tb_variant = -1;      // -1 not chosen yet; bit 0 the launch shape; step-field
                               // passes only: bit 1 one more TMA stage of delta (two-sweep:
                               // four instead of three; three-sweep: five instead of four),
                               // bit 2 three sweeps per pass instead of two; 8, 9: two
-                              // sweeps, 64-column tiles
+                              // sweeps, narrow tiles
     bool tm_ready = false;
     CUtensorMap tm_delta[2], tm_r, tm_u, tm_v, tm_w, tm_f, tm_t;
-    CUtensorMap tmn_delta[2], tmn_r, tmn_u, tmn_v, tmn_w, tmn_t;   // 72-column boxes
+    CUtensorMap tmn_delta[2], tmn_r, tmn_u, tmn_v, tmn_w, tmn_t;   // narrow tiles
+    TBDCut cut{64, TB_TYI};                 // their size
     float* tm_delta_ptr[2] = {nullptr, nullptr};
     double tb_tuned_plain_ms = 0, tb_tuned_tb_ms = 0;
     // resident sweeps (sweep_res.cuh), FP32 and FP64: bricks of the lattice, inboxes (first
@@ -619,7 +620,7 @@ bool tb_eligible(const rfb_soc_handle* h, bool local) {
 }
 
 void tb_encode(rfb_soc_handle* h, CUtensorMap* m, CUtensorMapDataType t, size_t esize, void* ptr,
-               int planes, int box_w) {
+               int planes, int box_w, int box_h = TB_BH) {
     static EncodeTiledFn fn = nullptr;
     if (!fn) {
         void* p = nullptr;
@@ -634,7 +635,7 @@ void tb_encode(rfb_soc_handle* h, CUtensorMap* m, CUtensorMapDataType t, size_t 
     }
     const cuuint64_t dims[3] = {(cuuint64_t)h->nx, (cuuint64_t)h->ny, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)h->nx * esize, (cuuint64_t)h->nxny * esize};
-    const cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)TB_BH, 1};
+    const cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)box_h, 1};
     // no L2 promotion: a box row is fetched at sector granularity (a 256-byte promotion
     // would pull whole 256-byte chunks for the halo columns at both ends of every row)
     const cuuint32_t es[3] = {1, 1, 1};
@@ -666,12 +667,12 @@ void tb_prepare(rfb_soc_handle* h) {
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, tbd_smem<4>()));
         CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<true, 4>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, tbd_smem<4>()));
-        CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<false, 3, 64>,
+        CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<false, 3, 0>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   tbd_smem<3, 64>()));
-        CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<true, 3, 64>,
+                                   tbd_smem<3, 0>()));
+        CK(h, cudaFuncSetAttribute(sweep32tbd_kernel<true, 3, 0>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   tbd_smem<3, 64>()));
+                                   tbd_smem<3, 0>()));
         CK(h, cudaFuncSetAttribute(sweep32t3_kernel<false, 4>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, t3_smem<4>()));
         CK(h, cudaFuncSetAttribute(sweep32t3_kernel<true, 4>,
@@ -694,17 +695,19 @@ void tb_prepare(rfb_soc_handle* h) {
         tb_encode(h, &h->tm_f, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, h->d_mask32, h->nz, TB_BWM);
     tb_encode(h, &h->tm_t, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_dtc, h->nz, TB_BW);
     {
-        constexpr int bw = TBDGeom<64>::BW;
-        for (int q = 0; q < 2; ++q)
-            tb_encode(h, &h->tmn_delta[q], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_delta[q],
-                      h->nz, bw);
-        tb_encode(h, &h->tmn_r, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_r32, h->nz, bw);
-        tb_encode(h, &h->tmn_u, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_u32, h->nz, bw);
-        tb_encode(h, &h->tmn_v, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_v32, h->nz, bw);
-        tb_encode(h, &h->tmn_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_w32, h->nz + 1, bw);
-        tb_encode(h, &h->tmn_t, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_dtc, h->nz, bw);
+        h->cut = tbd_cut(h->nx, h->ny);
+        auto narrow = [&](CUtensorMap* m, float* p, int planes) {
+            tb_encode(h, m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, p, planes, h->cut.txi + 8,
+                      h->cut.tyi + 4);
+        };
+        for (int q = 0; q < 2; ++q) narrow(&h->tmn_delta[q], h->d_delta[q], h->nz);
+        narrow(&h->tmn_r, h->d_r32, h->nz);
+        narrow(&h->tmn_u, h->d_u32, h->nz);
+        narrow(&h->tmn_v, h->d_v32, h->nz);
+        narrow(&h->tmn_w, h->d_w32, h->nz + 1);
+        narrow(&h->tmn_t, h->d_dtc, h->nz);
     }
-    // One CTA per SM fits (152 to 227 KB of shared memory each), two with 64-column tiles.
+    // One CTA per SM fits (152 to 227 KB of shared memory each), two with narrow tiles.
     // Shape 0, persistent: the tile-major (tile, plane) space in equal shares of at least
     // 16 planes (every z segment pays a prologue of k planes, k the sweeps of a pass): no
     // partial last wave, but CTAs on neighbouring tiles run at different planes and do not
@@ -714,8 +717,8 @@ void tb_prepare(rfb_soc_handle* h) {
     int sms = 152;
     CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     for (int g = 0; g < 3; ++g) {                      // pairs of tb_launch
-        const int k = g == 1 ? 3 : 2, rows = g == 1 ? T3_TYI : TB_TYI;
-        const int txi = g == 2 ? 64 : TB_TXI, slots = g == 2 ? 2 * sms : sms;
+        const int k = g == 1 ? 3 : 2, rows = g == 2 ? h->cut.tyi : g == 1 ? T3_TYI : TB_TYI;
+        const int txi = g == 2 ? h->cut.txi : TB_TXI, slots = g == 2 ? 2 * sms : sms;
         const int64_t tiles = (int64_t)((h->nx + txi - 1) / txi) * ((h->ny + rows - 1) / rows);
         auto& P = h->tb_launch[2 * g];
         P.lc = h->nz;
@@ -752,6 +755,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
     if (local) {
         TBDArgs A{};
         A.nx = h->nx; A.ny = h->ny; A.nz = h->nz;
+        A.cut = h->cut;
         const int v = std::max(h->tb_variant, 0);
         const bool narrow = v >= 8;
         const auto& S = h->tb_launch[(narrow ? 4 : v >= 4 ? 2 : 0) + (v & 1)];
@@ -779,7 +783,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
             return;
         }
         const auto k =
-            narrow ? (tr ? sweep32tbd_kernel<true, 3, 64> : sweep32tbd_kernel<false, 3, 64>)
+            narrow ? (tr ? sweep32tbd_kernel<true, 3, 0> : sweep32tbd_kernel<false, 3, 0>)
             : tr   ? (four ? sweep32tbd_kernel<true, 4> : sweep32tbd_kernel<true, 3>)
                    : (four ? sweep32tbd_kernel<false, 4> : sweep32tbd_kernel<false, 3>);
         // a pass may start its blocks while the pass before it runs out (sweep_dt.cuh)
@@ -788,8 +792,8 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
         at1.val.programmaticStreamSerializationAllowed = 1;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = S.grid;
-        cfg.blockDim = dim3(narrow ? TBDGeom<64>::THREADS : TB_THREADS);
-        cfg.dynamicSmemBytes = narrow ? tbd_smem<3, 64>() : four ? tbd_smem<4>() : tbd_smem<3>();
+        cfg.blockDim = dim3(narrow ? TBDGeom<0>::THREADS : TB_THREADS);
+        cfg.dynamicSmemBytes = narrow ? tbd_smem<3, 0>() : four ? tbd_smem<4>() : tbd_smem<3>();
         cfg.stream = h->stream;
         cfg.attrs = &at1;
         cfg.numAttrs = 1;
@@ -1006,7 +1010,7 @@ std::mutex g_tune_mu;
 
 // Project-written autotuner for one lattice: time (twice, keeping the faster) 12 plain
 // sweeps and 12 sweeps of each launch shape of the two-sweep pass (with local steps: with
-// three and with four TMA stages, and with 64-column tiles) by CUDA events on the current
+// three and with four TMA stages, and with narrow tiles) by CUDA events on the current
 // forcing and keep the fastest (tb_only: choose between the pass variants only).
 void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false) {
     if (!tb_eligible(h, op.dt_mode == RFB_DT_LOCAL)) { h->tb_mode = 0; return; }
@@ -2775,14 +2779,14 @@ struct rfb_batch {
     BatchLoop* d_loop = nullptr;
     BatchLoop* h_loop = nullptr;         // pinned
     // two-sweep passes over every lattice (local steps, every lattice nz >= 2): per-lattice
-    // tensor maps (boxes for 128- and for 64-column tiles), (lattice, tile, z chunk) items,
-    // tile width, chunk length and stage count (autotuned)
+    // tensor maps (boxes for 128-column and for narrow tiles), the list's plan, tile width,
+    // chunk length of the list's order and stage count (autotuned)
     BatchTBD* d_tbd = nullptr;           // 136-column boxes
-    BatchTBD* d_tbdn = nullptr;          // 72-column boxes
-    BatchTBItem* d_tbitems = nullptr;
-    int n_tbitems = 0;
-    int tb_lc = 0;                       // chunk length of the built item list
-    int tb_txi = 128;                    // interior columns of a tile (128 or 64)
+    BatchTBD* d_tbdn = nullptr;          // boxes of narrow tiles
+    int* d_plan = nullptr;               // tile planes before each lattice, and in all
+    int tb_lc = 0;                       // planes of a chunk
+    int tb_txi = 128;                    // 128 interior columns of a tile, or 64: narrow tiles
+                                         // (each lattice's own cut)
     int tb_nst = 0;                      // 0: one-sweep kernel; 3 / 4: passes, stages
     int sms = 152;
     int tuned_mode = -1;                 // kernel choice the tuning was made for
@@ -2857,43 +2861,27 @@ void build_items(rfb_batch* b, int kchunk) {
     if (b->loop_exec) { cudaGraphExecDestroy(b->loop_exec); b->loop_exec = nullptr; }
 }
 
-// Items of the batched two-sweep pass for a z-chunk length and tile width: per lattice,
-// chunk-major with the tiles of a chunk consecutive.
-void build_tb_items(rfb_batch* b, int lc, int txi) {
-    if (b->tb_lc == lc && b->tb_txi == txi) return;
-    std::vector<BatchTBItem> items;
-    for (size_t q = 0; q < b->hs.size(); ++q) {
-        const rfb_soc_handle* h = b->hs[q];
-        const int tiles = ((h->nx + txi - 1) / txi) * ((h->ny + TB_TYI - 1) / TB_TYI);
-        for (int kb = 0; kb < h->nz; kb += lc)
-            for (int t = 0; t < tiles; ++t)
-                items.push_back(BatchTBItem{(int)q, t, kb, std::min(kb + lc, h->nz)});
-    }
-    if (b->d_tbitems) cudaFree(b->d_tbitems);
-    b->d_tbitems = nullptr;
-    BCK(b, cudaMalloc((void**)&b->d_tbitems, items.size() * sizeof(BatchTBItem)));
-    BCK(b, cudaMemcpy(b->d_tbitems, items.data(), items.size() * sizeof(BatchTBItem),
-                      cudaMemcpyHostToDevice));
-    b->n_tbitems = (int)items.size();
-    b->tb_lc = lc;
-    b->tb_txi = txi;
-    if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
-    if (b->loop_exec) { cudaGraphExecDestroy(b->loop_exec); b->loop_exec = nullptr; }
+// the lists of a pass: counted from the lattices that are still active
+void batch_plan(rfb_batch* b) {
+    batch_plan_kernel<<<1, 32, 0, b->stream>>>(b->tb_txi == 64 ? b->d_tbdn : b->d_tbd, b->d_insts,
+                                               (int)b->hs.size(), b->tb_lc, b->d_plan);
+    BLAUNCHED(b);
 }
 
 void batch_sweeps(rfb_batch* b, int n, bool local) {
     if (b->tb_nst) {   // two-sweep passes (n even); pass p reads delta[p & 1]
         for (int q = 0; q < n / 2; ++q) {
+            const int n_inst = (int)b->hs.size();
             if (b->tb_txi == 64)   // two CTAs per SM
-                batch_tbd_kernel<3, 64><<<2 * b->sms, TBDGeom<64>::THREADS, tbd_smem<3, 64>(),
-                                          b->stream>>>(b->d_tbdn, b->d_insts, b->d_tbitems,
-                                                       b->n_tbitems, q & 1, b->d_tberr);
+                batch_tbd_kernel<3, 0><<<2 * b->sms, TBDGeom<0>::THREADS, tbd_smem<3, 0>(),
+                                         b->stream>>>(b->d_tbdn, b->d_insts, b->d_plan, n_inst,
+                                                      b->tb_lc, q & 1, b->d_tberr);
             else if (b->tb_nst == 4)
                 batch_tbd_kernel<4, 128><<<b->sms, TB_THREADS, tbd_smem<4>(), b->stream>>>(
-                    b->d_tbd, b->d_insts, b->d_tbitems, b->n_tbitems, q & 1, b->d_tberr);
+                    b->d_tbd, b->d_insts, b->d_plan, n_inst, b->tb_lc, q & 1, b->d_tberr);
             else
                 batch_tbd_kernel<3, 128><<<b->sms, TB_THREADS, tbd_smem<3>(), b->stream>>>(
-                    b->d_tbd, b->d_insts, b->d_tbitems, b->n_tbitems, q & 1, b->d_tberr);
+                    b->d_tbd, b->d_insts, b->d_plan, n_inst, b->tb_lc, q & 1, b->d_tberr);
             BLAUNCHED(b);
         }
         return;
@@ -2939,6 +2927,7 @@ void batch_check(rfb_batch* b, bool fused, int sweeps_done) {
 void batch_cycle(rfb_batch* b, int every, bool local, bool to_host = true) {
     batch_zero_kernel<<<152 * 4, 256, 0, b->stream>>>(b->d_insts, (int)b->hs.size());
     BLAUNCHED(b);
+    if (b->tb_nst) batch_plan(b);
     batch_sweeps(b, every, local);
     batch_check(b, true, every);
     if (to_host)
@@ -2996,6 +2985,9 @@ void build_loop_graph(rfb_batch* b, int every, bool local) {
 // sweeps per cycle so that the FP64 check costs about 3% of a cycle.
 // mode: 0 fastest of both kernels, 1 one-sweep kernel only, 2 two-sweep passes only
 void autotune(rfb_batch* b, bool local, std::vector<BatchInst>& insts0, int mode) {
+    // the graphs hold the kernels chosen before
+    if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
+    if (b->loop_exec) { cudaGraphExecDestroy(b->loop_exec); b->loop_exec = nullptr; }
     // candidates: z-chunk of the items x grid size (1x / 2x the resident blocks, walking
     // the item list persistently, or one block per item)
     const int cands[] = {8, 16, 32, 64};
@@ -3023,19 +3015,22 @@ void autotune(rfb_batch* b, bool local, std::vector<BatchInst>& insts0, int mode
     b->tuned_kchunk = best_k;
     b->tuned_sweep_ms = best / 4.0;
     // two-sweep passes (local steps and tensor maps in place): chunk length x (tile width,
-    // stages): 128-column tiles with three or four stages (one CTA per SM), 64-column tiles
-    // with three (two CTAs per SM; lattices narrower than 128 columns waste less of a tile)
+    // stages): 128-column tiles with three or four stages (one CTA per SM), narrow tiles
+    // with three (two CTAs per SM; lattices narrower than 128 columns waste less of a tile);
+    // the longest chunk: whole columns of a tile, one run per CTA
     b->tb_nst = 0;
     if (mode >= 2) best = 1e30f;
     if (b->d_tbd && mode != 1) {
         float best_tb = 1e30f;
         int bl = 0, bn = 0, bw = 128;
         const int shapes[3][2] = {{128, 3}, {128, 4}, {64, 3}};
-        for (int lc : {16, 32, 64}) {
+        for (int lc : {16, 32, 64, 1 << 30}) {
             for (const auto& sh : shapes) {
                 if ((mode == 3 && sh[0] != 128) || (mode == 4 && sh[0] != 64)) continue;
-                build_tb_items(b, lc, sh[0]);
+                b->tb_lc = lc;
+                b->tb_txi = sh[0];
                 b->tb_nst = sh[1];
+                batch_plan(b);
                 batch_sweeps(b, 2, local);   // warm-up
                 BCK(b, cudaEventRecord(b->ev[0], b->stream));
                 batch_sweeps(b, 4, local);
@@ -3048,7 +3043,8 @@ void autotune(rfb_batch* b, bool local, std::vector<BatchInst>& insts0, int mode
         }
         b->tb_nst = 0;
         if (best_tb < best || mode >= 2) {
-            build_tb_items(b, bl, bw);
+            b->tb_lc = bl;
+            b->tb_txi = bw;
             b->tb_nst = bn;
             b->tuned_sweep_ms = best_tb / 4.0;
         }
@@ -3101,6 +3097,7 @@ rfb_status rfb_soc_batch_create(rfb_soc_handle* const* hs, int n, rfb_batch** ou
         BCK(b, cudaMalloc((void**)&b->d_loop, sizeof(BatchLoop)));
         BCK(b, cudaMallocHost((void**)&b->h_loop, sizeof(BatchLoop)));
         BCK(b, cudaMalloc((void**)&b->d_tberr, sizeof(unsigned int)));
+        BCK(b, cudaMalloc((void**)&b->d_plan, (n + 1) * sizeof(int)));
         BCK(b, cudaEventCreate(&b->ev[0]));
         BCK(b, cudaEventCreate(&b->ev[1]));
         int sms = 152, per = 4;
@@ -3124,7 +3121,7 @@ rfb_status rfb_soc_batch_destroy(rfb_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->loop_exec) cudaGraphExecDestroy(b->loop_exec);
     void* ptrs[] = {b->d_insts, b->d_ctl,  b->d_items,  b->d_item_begin, b->d_partials,
-                    b->d_loop,  b->d_tbd,  b->d_tbdn, b->d_tbitems, b->d_tberr};
+                    b->d_loop,  b->d_tbd,  b->d_tbdn, b->d_plan, b->d_tberr};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (b->h_ctl) cudaFreeHost(b->h_ctl);
@@ -3249,27 +3246,28 @@ rfb_status rfb_soc_batch_solve(rfb_batch* b, const double* s_in, const double* e
                 BCK(b, cudaFuncSetAttribute(batch_tbd_kernel<4, 128>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             tbd_smem<4>()));
-                BCK(b, cudaFuncSetAttribute(batch_tbd_kernel<3, 64>,
+                BCK(b, cudaFuncSetAttribute(batch_tbd_kernel<3, 0>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            tbd_smem<3, 64>()));
+                                            tbd_smem<3, 0>()));
             }
-            for (int wide = 0; wide < 2; ++wide) {   // 72- then 136-column boxes
-                const int bw = wide ? TB_BW : TBDGeom<64>::BW;
+            for (int wide = 0; wide < 2; ++wide) {   // narrow, then 128-column tiles
                 std::vector<BatchTBD> tbd(n);
                 for (int q = 0; q < n; ++q) {
                     rfb_soc_handle* h = b->hs[q];
                     BatchTBD& T = tbd[q];
                     std::memset(&T, 0, sizeof T);
+                    T.cut = wide ? TBDCut{TB_TXI, TB_TYI} : tbd_cut(h->nx, h->ny);
+                    auto encode = [&](CUtensorMap* m, float* p, int planes) {
+                        tb_encode(h, m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, p, planes,
+                                  T.cut.txi + 8, T.cut.tyi + 4);
+                    };
                     try {
-                        for (int p = 0; p < 2; ++p)
-                            tb_encode(h, &T.td[p], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
-                                      insts[q].delta[p], h->nz, bw);
-                        tb_encode(h, &T.tr, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_r32, h->nz, bw);
-                        tb_encode(h, &T.tu, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_u32, h->nz, bw);
-                        tb_encode(h, &T.tv, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_v32, h->nz, bw);
-                        tb_encode(h, &T.tw, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_w32,
-                                  h->nz + 1, bw);
-                        tb_encode(h, &T.tt, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->d_dtc, h->nz, bw);
+                        for (int p = 0; p < 2; ++p) encode(&T.td[p], insts[q].delta[p], h->nz);
+                        encode(&T.tr, h->d_r32, h->nz);
+                        encode(&T.tu, h->d_u32, h->nz);
+                        encode(&T.tv, h->d_v32, h->nz);
+                        encode(&T.tw, h->d_w32, h->nz + 1);
+                        encode(&T.tt, h->d_dtc, h->nz);
                     } catch (Fail f) {
                         bset_err(b, "lattice %d: %s", q, h->err.c_str());
                         throw;
@@ -3291,7 +3289,7 @@ rfb_status rfb_soc_batch_solve(rfb_batch* b, const double* s_in, const double* e
         BCK(b, cudaMemsetAsync(b->d_tberr, 0, sizeof(unsigned int), b->stream));
         // opts.fp32_kernel: 0 the faster, 1 the one-sweep kernel, 2 two-sweep passes (tile
         // width, stages and chunk timed), 3 .. 6 passes with 128-column tiles, 7 / 8 passes
-        // with 64-column tiles (mode 3 and 4 below)
+        // with narrow tiles (mode 3 and 4 below)
         if (o.fp32_kernel > 8) {
             bset_err(b, "opts.fp32_kernel of a batch must be 0 .. 8");
             return RFB_ERR_INVALID_ARG;
@@ -3443,6 +3441,8 @@ rfb_status rfb_soc_batch_solve(rfb_batch* b, const double* s_in, const double* e
             }
         }
         if (info) {
+            int max_nz = 0;
+            for (const rfb_soc_handle* h : b->hs) max_nz = std::max(max_nz, h->nz);
             info->kchunk = b->tuned_kchunk;
             info->sweeps_per_cycle = every;
             info->n_items = b->n_items;
@@ -3452,7 +3452,7 @@ rfb_status rfb_soc_batch_solve(rfb_batch* b, const double* s_in, const double* e
             info->cycles = done / every;
             info->graph_launches = graph_launches;
             info->pass_stages = b->tb_nst;
-            info->pass_chunk = b->tb_nst ? b->tb_lc : 0;
+            info->pass_chunk = b->tb_nst ? std::min(b->tb_lc, max_nz) : 0;
             info->pass_tile_cols = b->tb_nst ? b->tb_txi : 0;
             info->df_cycles = (int32_t)df_cycles;
             info->time_ms = ms;

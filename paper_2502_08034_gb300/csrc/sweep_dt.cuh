@@ -131,19 +131,32 @@ sweep32d_kernel(DArgs A, const float* __restrict__ s, float* __restrict__ s_out,
 // mbarrier waits are those of sweep32tb_kernel (sweep_tb.cuh); a stage holds six FP32
 // planes (delta, forcing, u, v, w, step).
 // ---------------------------------------------------------------------------------
-// Tile geometry: TXI interior columns (128, or 64 for narrow lattices in batches), the 12
-// interior rows of sweep_tb.cuh, boxes of TXI + 8 columns and 16 rows, one thread per 4
-// cells of the box columns on 14 rows.
+// Tile geometry: TXI = 128 interior columns and the 12 interior rows of sweep_tb.cuh, boxes of
+// 136 columns and 16 rows, one thread per 4 cells of the box columns on 14 rows; or (TXI = 0)
+// narrow tiles cut to the lattice (tbd_cut), two CTAs per SM.
 template <int TXI>
 struct TBDGeom {
     static_assert(TXI % 4 == 0, "4-cell groups");
     static constexpr int BW = TXI + 8;           // staged columns
     static constexpr int GX = BW / 4;            // thread columns
-    static constexpr int THREADS = GX * TB_GY;   // 476 (TXI = 128) or 252 (TXI = 64)
+    static constexpr int THREADS = GX * TB_GY;   // 476
     static constexpr int PLANE = BW * TB_BH;
     static constexpr int F32 = PLANE * 4;        // bytes of one staged FP32 plane
     static constexpr int STAGE = 6 * F32;        // delta, forcing, u, v, w, step
     static_assert(F32 % 128 == 0, "stage buffers stay 128-B aligned");
+};
+// Narrow tiles: any txi x tyi whose threads ((txi + 8) / 4 on tyi + 2 rows) and box (txi + 8
+// columns, tyi + 4 rows) fit; the pitch of a staged plane is fixed. A row of the box is as long
+// as its threads' cells, so a warp's accesses are consecutive whatever the cut.
+template <>
+struct TBDGeom<0> {
+    static constexpr int THREADS = 256;
+    static constexpr int PLANE = 1408;
+    static constexpr int F32 = PLANE * 4;
+    static constexpr int STAGE = 6 * F32;
+};
+struct TBDCut {
+    int txi, tyi;                                // interior columns (4-cell groups) and rows
 };
 static_assert(TBDGeom<128>::F32 == TB_F32 && TBDGeom<128>::THREADS == TB_THREADS, "geometry");
 constexpr int TBD_STAGE = TBDGeom<128>::STAGE;
@@ -154,10 +167,39 @@ __host__ __device__ constexpr int tbd_bar() { return tbd_l1<NST, TXI>() + 2 * TB
 template <int NST, int TXI = 128>
 __host__ __device__ constexpr int tbd_smem() { return tbd_bar<NST, TXI>() + 64 + 128; }   // + slack
 static_assert(tbd_smem<4>() <= 232448, "four stages fit the 227 KB a CTA may use");
-static_assert(2 * tbd_smem<3, 64>() <= 233472, "two narrow three-stage CTAs fit an SM");
+static_assert(2 * (tbd_smem<3, 0>() + 1024) <= 233472, "two narrow three-stage CTAs fit an SM");
+
+// The narrow cut of an nx x ny plane with the least work per pass: a CTA's threads run for every
+// tile, whether or not their cells lie in the lattice, and every row of a box costs its cells
+// and about a 128-byte line more. Tiles of 64 x 12 throughout covered lattices of 68, 72 or 80
+// columns twice over. us per sweep with those and now: 160x160x200 16.1 and 15.0 (42 tiles, now
+// 36 of 80 x 9; 32 x 23 with 35 tiles 15.3), 136x136x200 13.6 and 11.3, 100x100x150 5.86 and
+// 5.65, 192^3 19.4 either way.
+inline TBDCut tbd_cut(int nx, int ny) {
+    using G = TBDGeom<0>;
+    TBDCut best{64, TB_TYI};
+    double least = INFINITY;
+    for (int n = 1; n <= 1 + (nx - 1) / 4; ++n) {          // tiles across
+        const int txi = ((nx + n - 1) / n + 3) / 4 * 4;
+        const int bw = txi + 8;
+        if ((nx + txi - 1) / txi != n || bw > 256) continue;
+        const int rows = std::min(std::min(G::THREADS / (bw / 4) - 2, G::PLANE / bw - 4),
+                                  std::min(ny, 252));
+        if (rows < 2 && rows < ny) continue;
+        const int m = (ny + rows - 1) / rows, tyi = (ny + m - 1) / m;
+        const double cost = (double)n * m * (4 * G::THREADS + (bw + 32) * (tyi + 4));
+        if (cost < least) {
+            least = cost;
+            best = TBDCut{txi, tyi};
+        }
+        if (txi <= 32) break;                              // narrower: mostly halo
+    }
+    return best;
+}
 
 struct TBDArgs {
     int nx, ny, nz;
+    TBDCut cut;                       // narrow tiles
     int lc;                           // planes per z chunk (nz: one chunk)
     int64_t total;                    // tiles x chunks x lc (chunk-major, tile fastest)
     int64_t per;                      // planes of that space per CTA
@@ -177,6 +219,7 @@ struct TBDField {
     const CUtensorMap* w;
     const CUtensorMap* t;
     int nx, ny, nz;
+    TBDCut cut;                       // narrow tiles
     const float* d_in;                // delta read by this pass (prologue plane)
     float* d_out;
     float omc, Dh;
@@ -245,19 +288,22 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
                                             int kb, int ke, bool early = false) {
     using G = TBDGeom<TXI>;
     const int tid = threadIdx.x;
-    const int tx = tid % G::GX, ty = tid / G::GX;
+    const int txi = TXI ? TXI : F.cut.txi, tyi = TXI ? TB_TYI : F.cut.tyi;
+    const int bw = txi + 8, groups = bw / 4;
+    const bool live = TXI != 0 || tid < groups * (tyi + 2);   // has cells in the box
+    const int tx = live ? tid % groups : 0, ty = live ? tid / groups : 0;
     const int bxx = 4 * tx, byy = 1 + ty;              // this thread's cells in the box
     const int nx = F.nx, ny = F.ny, nz = F.nz;
-    const bool interior = tx >= 1 && tx < 1 + TXI / 4 && ty >= 1 && ty <= TB_TYI;
+    const bool interior = live && tx >= 1 && tx < 1 + txi / 4 && ty >= 1 && ty <= tyi;
     const int64_t nxny = (int64_t)nx * ny;
-    const int o = byy * G::BW + bxx;                   // offset in a staged plane
-    const int gx = (nx + TXI - 1) / TXI;
+    const int o = byy * bw + bxx;                      // offset in a staged plane
+    const int gx = (nx + txi - 1) / txi;
     const float omc = F.omc, Dh = F.Dh;
     unsigned char* smem = R.smem;
-    const int x0 = TXI * (tile % gx) - 4;           // box origin (4-cell aligned)
-    const int y0 = TB_TYI * (tile / gx) - 2;
+    const int x0 = txi * (tile % gx) - 4;           // box origin (4-cell aligned)
+    const int y0 = tyi * (tile / gx) - 2;
     const int i0 = x0 + bxx, j = y0 + byy;
-    const bool in_dom = i0 >= 0 && i0 < nx && j >= 0 && j < ny;
+    const bool in_dom = live && i0 >= 0 && i0 < nx && j >= 0 && j < ny;
     auto issue_delta = [&](int p, int s) {
         if (tid == 0) tma_load_3d(R.stage(s), F.d, x0, y0, p, &R.bar[s]);
     };
@@ -266,7 +312,7 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
         if (tid != 0) return;                          // one thread issues the copies
         unsigned char* S = R.stage(s);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(&R.bar[s], G::STAGE);
+        mbar_expect_tx(&R.bar[s], TXI ? G::STAGE : 24 * bw * (tyi + 4));
         tma_load_3d(S + G::F32, F.r, x0, y0, p, &R.bar[s]);
         tma_load_3d(S + 2 * G::F32, F.u, x0, y0, p, &R.bar[s]);
         tma_load_3d(S + 3 * G::F32, F.v, x0, y0, p, &R.bar[s]);
@@ -318,7 +364,7 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
         const float4 u4 = lds4(U0 + o);
         const float un = U0[o + 4];
         const float4 v4 = lds4(V0 + o);
-        const float4 vh4 = lds4(V0 + o + G::BW);
+        const float4 vh4 = lds4(V0 + o + bw);
         const float4 wl4 = lds4(W0 + o);
         const float4 wh4 = lds4(W1 + o);
         const float4 t4 = lds4(T0 + o);
@@ -331,7 +377,7 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
         float4 l1 = dc;
         if (in_dom && z >= 0 && z < nz) {
             const float dxm = D0[o - 1], dxp = D0[o + 4];
-            const float4 dym = lds4(D0 + o - G::BW), dyp = lds4(D0 + o + G::BW);
+            const float4 dym = lds4(D0 + o - bw), dyp = lds4(D0 + o + bw);
             float out[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -341,14 +387,14 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
             l1 = make_float4(out[0], out[1], out[2], out[3]);
         }
         float* L1w = reinterpret_cast<float*>(smem + tbd_l1<NST, TXI>()) + (z & 1) * G::PLANE;
-        *reinterpret_cast<float4*>(L1w + o) = l1;
+        if (live) *reinterpret_cast<float4*>(L1w + o) = l1;
         // ---- level 2 at plane z-1 (its level-1 neighbours were stored last step)
         const int zz = z - 1;
         if (zz >= kb && interior && in_dom) {
             const float* L1r =
                 reinterpret_cast<const float*>(smem + tbd_l1<NST, TXI>()) + (zz & 1) * G::PLANE;
             const float lxm = L1r[o - 1], lxp = L1r[o + 4];
-            const float4 lym = lds4(L1r + o - G::BW), lyp = lds4(L1r + o + G::BW);
+            const float4 lym = lds4(L1r + o - bw), lyp = lds4(L1r + o + bw);
             float out[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -387,11 +433,11 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
 // to 41.0 on 256^3: a block's barriers, tensor maps and first five fields are in place when
 // the pass before it ends, and the last partial wave overlaps them.
 //
-// TXI = 64 (three stages, two CTAs per SM): lattices that 128-column tiles cover badly (160
-// columns: two tiles hold 62 % lattice, three narrow ones 83 %): 160x160x200 18.7 -> 16.1 us
-// per sweep, 192^3 22.7 -> 19.0.
+// TXI = 0 (narrow tiles, three stages, two CTAs per SM): lattices that 128-column tiles cover
+// badly (160 columns: two tiles hold 62 % lattice): 160x160x200 18.7 -> 15.0 us per sweep,
+// 192^3 22.7 -> 19.4.
 template <bool TR, int NST, int TXI = 128>
-__global__ void __launch_bounds__(TBDGeom<TXI>::THREADS, TXI == 64 ? 2 : 1)
+__global__ void __launch_bounds__(TBDGeom<TXI>::THREADS, TXI == 0 ? 2 : 1)
 sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constant__ CUtensorMap tm_r,
                   const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_v,
                   const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_t,
@@ -399,10 +445,10 @@ sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constan
     extern __shared__ unsigned char smem_raw[];
     grid_release();
     TBDRing<NST, TXI> R = tbd_ring_init<NST, TXI>(smem_raw, A.err);
-    const TBDField F{&tm_d, &tm_r, &tm_u, &tm_v, &tm_w, &tm_t, A.nx, A.ny, A.nz,
+    const TBDField F{&tm_d, &tm_r, &tm_u, &tm_v, &tm_w, &tm_t, A.nx, A.ny, A.nz, A.cut,
                      A.d_in, A.d_out, A.omc, A.Dh};
-    const int gx = (A.nx + TXI - 1) / TXI;
-    const int tiles = gx * ((A.ny + TB_TYI - 1) / TB_TYI);
+    const int txi = TXI ? TXI : A.cut.txi, tyi = TXI ? TB_TYI : A.cut.tyi;
+    const int tiles = ((A.nx + txi - 1) / txi) * ((A.ny + tyi - 1) / tyi);
     const int64_t q1 = min((int64_t)(blockIdx.x + 1) * A.per, A.total);
     bool ok = true, first = true;
     for (int64_t q = (int64_t)blockIdx.x * A.per; q < q1 && ok;) {
@@ -421,42 +467,99 @@ sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constan
 }
 
 // ---------------------------------------------------------------------------------
-// Batched two-sweep pass: many lattices in one launch. Work items are (lattice, tile, z
-// chunk), lattice-major with neighbouring tiles of a chunk next to each other; one CTA per
-// SM walks the item list in a fixed round-robin order. Each lattice's tensor maps live
-// in global memory (written by the host before the launch); lattices that have converged
-// are skipped (their flag is read from the batch's descriptors, which the check kernels
-// update), so a captured graph keeps working as lattices drop out.
+// Batched two-sweep pass: many lattices in one launch. The planes of every tile of every lattice
+// that has not converged form one list (lattice by lattice; within one, chunks of lc planes, in
+// each the tiles one after the other, the last chunk padded to lc). CTAs (one per SM, two with
+// narrow tiles) take equal runs of it, of lc planes at most: chunk by chunk in turn while there
+// is more than a chunk each, so that neighbouring tiles run together, and one shorter run each
+// once there is less. batch_plan_kernel counts the list once per cycle from the lattices'
+// flags, so as lattices drop out the others spread over the whole chip, also in a captured
+// graph. Each lattice's tensor maps live in global memory (written by the host before the
+// launch).
+//
+// What bounds a small batch is the CTA with the most planes. Fixed items of 16 planes handed out
+// in turn gave 16 lattices of 36^2x37 to 92^2x132 up to 57 steps per CTA and pass, with 37 planes
+// on average; equal runs of narrow tiles take 30 for 27:
+// a solve of them 34.2 -> 24.5 ms (tiles cut to each lattice and fixed items: 27.6). 48 lattices
+// of 64^3 to 192^2x384, bound by HBM, 1430 -> 1324 ms; one run per CTA of whole columns, whose
+// neighbours run at other times, took 1517 there.
 // ---------------------------------------------------------------------------------
 struct BatchTBD {
     CUtensorMap td[2];                // delta buffer 0 and 1
     CUtensorMap tr, tu, tv, tw, tt;   // forcing, u, v, w, step
     int nx, ny, nz, pad_;
+    TBDCut cut;                       // narrow tiles
     float omc, Dh;
 };
 
-struct BatchTBItem {
-    int inst, tile, kb, ke;           // planes kb .. ke-1 of one tile of one lattice
-};
+// planes a CTA takes at least (each run starts with two planes that only feed it)
+constexpr int BATCH_RUN_MIN = 4;
+
+__device__ __forceinline__ int batch_tiles(const BatchTBD& L) {
+    return ((L.nx + L.cut.txi - 1) / L.cut.txi) * ((L.ny + L.cut.tyi - 1) / L.cut.tyi);
+}
+
+// plan[q]: list positions of the active lattices before lattice q; plan[n]: all of them. One warp.
+__global__ void __launch_bounds__(32)
+batch_plan_kernel(const BatchTBD* __restrict__ lat, const BatchInst* __restrict__ insts, int n,
+                  int lc, int* __restrict__ plan) {
+    int base = 0;
+    for (int q0 = 0; q0 < n; q0 += 32) {
+        const int q = q0 + threadIdx.x;
+        int own = 0;
+        if (q < n && insts[q].active) {
+            const int nz = lat[q].nz, len = min(lc, nz);
+            own = batch_tiles(lat[q]) * ((nz + len - 1) / len * len);
+        }
+        int sum = own;
+        for (int w = 1; w < 32; w *= 2) {
+            const int below = __shfl_up_sync(0xffffffffu, sum, w);
+            if ((int)threadIdx.x >= w) sum += below;
+        }
+        if (q < n) plan[q] = base + sum - own;
+        base += __shfl_sync(0xffffffffu, sum, 31);
+    }
+    if (threadIdx.x == 0) plan[n] = base;
+}
 
 template <int NST, int TXI>
-__global__ void __launch_bounds__(TBDGeom<TXI>::THREADS, TXI == 64 ? 2 : 1)
+__global__ void __launch_bounds__(TBDGeom<TXI>::THREADS, TXI == 0 ? 2 : 1)
 batch_tbd_kernel(const BatchTBD* __restrict__ lat, const BatchInst* __restrict__ insts,
-                 const BatchTBItem* __restrict__ items, int n_items, int parity,
-                 unsigned int* err) {
+                 const int* __restrict__ plan, int n, int lc, int parity, unsigned int* err) {
     extern __shared__ unsigned char smem_raw[];
+    const int total = plan[n];
+    const int run = min(max((total + (int)gridDim.x - 1) / (int)gridDim.x, BATCH_RUN_MIN), lc);
+    if ((int64_t)blockIdx.x * run >= total) return;
     TBDRing<NST, TXI> R = tbd_ring_init<NST, TXI>(smem_raw, err);
-    bool ok = true;
-    for (int w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
-        const BatchTBItem it = items[w];
-        const BatchInst* I = insts + it.inst;
-        if (!I->active) continue;   // uniform over the CTA
-        const BatchTBD* L = lat + it.inst;
-        const TBDField F{&L->td[parity], &L->tr, &L->tu, &L->tv, &L->tw, &L->tt, L->nx, L->ny,
-                         L->nz, I->delta[parity], I->delta[parity ^ 1], L->omc, L->Dh};
-        ok = tbd_segment<false, NST, TXI>(R, F, it.tile, it.kb, it.ke);
+    for (int64_t first = (int64_t)blockIdx.x * run; first < total; first += (int64_t)gridDim.x * run) {
+        int pos = (int)first;
+        const int end = min(pos + run, total);
+        int q = 0;                                     // the lattice that holds position pos
+        for (int hi = n; hi - q > 1;) {                // plan[q] <= pos < plan[hi]
+            const int mid = (q + hi) / 2;
+            if (plan[mid] <= pos) q = mid;
+            else hi = mid;
+        }
+        while (pos < end) {
+            while (plan[q + 1] <= pos) ++q;            // converged ones have no planes
+            const BatchTBD* L = lat + q;
+            const BatchInst* I = insts + q;
+            const TBDField F{&L->td[parity], &L->tr, &L->tu, &L->tv, &L->tw, &L->tt, L->nx,
+                             L->ny, L->nz, L->cut, I->delta[parity], I->delta[parity ^ 1],
+                             L->omc, L->Dh};
+            const int tiles = batch_tiles(*L), len = min(lc, L->nz);
+            const int item = (pos - plan[q]) / len, z = (pos - plan[q]) % len;
+            const int kc = item / tiles * len, kb = kc + z;
+            const int left = min(len - z, end - pos);  // of this item, in this run
+            pos += left;
+            const int ke = min(kb + left, L->nz);
+            if (kb >= ke) continue;                    // padding of the last chunk
+            if (!tbd_segment<false, NST, TXI>(R, F, item % tiles, kb, ke)) {
+                tbd_ring_drain<NST>(R);
+                return;
+            }
+        }
     }
-    if (!ok) tbd_ring_drain<NST>(R);
 }
 
 }  // namespace rfb

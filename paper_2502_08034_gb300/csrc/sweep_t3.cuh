@@ -372,7 +372,7 @@ sweep32t3_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constant
     const uint32_t tmem = tbase + ((uint32_t)(32 * (warp & 3)) << 16) +
                           (uint32_t)((warp >> 2) * 3 * T3_SLOT_COLS);
     const TBDField F{&tm_d, &tm_r, &tm_u, &tm_v, &tm_w, &tm_t, A.nx, A.ny, A.nz,
-                     A.d_in, A.d_out, A.omc, A.Dh};
+                     A.cut, A.d_in, A.d_out, A.omc, A.Dh};
     const int gx = (A.nx + TB_TXI - 1) / TB_TXI;
     const int tiles = gx * ((A.ny + T3_TYI - 1) / T3_TYI);
     const int64_t q1 = min((int64_t)(blockIdx.x + 1) * A.per, A.total);
