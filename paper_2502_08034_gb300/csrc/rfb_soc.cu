@@ -2871,17 +2871,26 @@ void batch_plan(rfb_batch* b) {
 void batch_sweeps(rfb_batch* b, int n, bool local) {
     if (b->tb_nst) {   // two-sweep passes (n even); pass p reads delta[p & 1]
         for (int q = 0; q < n / 2; ++q) {
-            const int n_inst = (int)b->hs.size();
-            if (b->tb_txi == 64)   // two CTAs per SM
-                batch_tbd_kernel<3, 0><<<2 * b->sms, TBDGeom<0>::THREADS, tbd_smem<3, 0>(),
-                                         b->stream>>>(b->d_tbdn, b->d_insts, b->d_plan, n_inst,
-                                                      b->tb_lc, q & 1, b->d_tberr);
-            else if (b->tb_nst == 4)
-                batch_tbd_kernel<4, 128><<<b->sms, TB_THREADS, tbd_smem<4>(), b->stream>>>(
-                    b->d_tbd, b->d_insts, b->d_plan, n_inst, b->tb_lc, q & 1, b->d_tberr);
-            else
-                batch_tbd_kernel<3, 128><<<b->sms, TB_THREADS, tbd_smem<3>(), b->stream>>>(
-                    b->d_tbd, b->d_insts, b->d_plan, n_inst, b->tb_lc, q & 1, b->d_tberr);
+            // a pass after a pass may start its blocks while that one runs out (the plan and
+            // the forcing were complete before the first)
+            const bool narrow = b->tb_txi == 64;         // two CTAs per SM
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at.val.programmaticStreamSerializationAllowed = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(narrow ? 2 * b->sms : b->sms);
+            cfg.blockDim = dim3(narrow ? TBDGeom<0>::THREADS : TB_THREADS);
+            cfg.dynamicSmemBytes =
+                narrow ? tbd_smem<3, 0>() : b->tb_nst == 4 ? tbd_smem<4>() : tbd_smem<3>();
+            cfg.stream = b->stream;
+            cfg.attrs = &at;
+            cfg.numAttrs = q > 0 ? 1 : 0;
+            const auto k = narrow           ? batch_tbd_kernel<3, 0>
+                           : b->tb_nst == 4 ? batch_tbd_kernel<4, 128>
+                                            : batch_tbd_kernel<3, 128>;
+            BCK(b, cudaLaunchKernelEx(&cfg, k, (const BatchTBD*)(narrow ? b->d_tbdn : b->d_tbd),
+                                      (const BatchInst*)b->d_insts, (const int*)b->d_plan,
+                                      (int)b->hs.size(), b->tb_lc, q & 1, b->d_tberr));
             BLAUNCHED(b);
         }
         return;

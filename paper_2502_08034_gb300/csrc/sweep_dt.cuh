@@ -480,7 +480,9 @@ sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constan
 // What bounds a small batch is the CTA with the most planes. Fixed items of 16 planes handed out
 // in turn gave 16 lattices of 36^2x37 to 92^2x132 up to 57 steps per CTA and pass, with 37 planes
 // on average; equal runs of narrow tiles take 30 for 27:
-// a solve of them 34.2 -> 24.5 ms (tiles cut to each lattice and fixed items: 27.6). 48 lattices
+// a solve of them 34.2 -> 24.5 ms (tiles cut to each lattice and fixed items: 27.6), and 22.4 with
+// programmatic dependent launches from a cycle's second pass on (the plan, read before the wait,
+// is complete before the first). 48 lattices
 // of 64^3 to 192^2x384, bound by HBM, 1430 -> 1324 ms; one run per CTA of whole columns, whose
 // neighbours run at other times, took 1517 there.
 // ---------------------------------------------------------------------------------
@@ -527,10 +529,12 @@ __global__ void __launch_bounds__(TBDGeom<TXI>::THREADS, TXI == 0 ? 2 : 1)
 batch_tbd_kernel(const BatchTBD* __restrict__ lat, const BatchInst* __restrict__ insts,
                  const int* __restrict__ plan, int n, int lc, int parity, unsigned int* err) {
     extern __shared__ unsigned char smem_raw[];
+    grid_release();
     const int total = plan[n];
     const int run = min(max((total + (int)gridDim.x - 1) / (int)gridDim.x, BATCH_RUN_MIN), lc);
     if ((int64_t)blockIdx.x * run >= total) return;
     TBDRing<NST, TXI> R = tbd_ring_init<NST, TXI>(smem_raw, err);
+    bool early = true;                                 // before the launch's first segment
     for (int64_t first = (int64_t)blockIdx.x * run; first < total; first += (int64_t)gridDim.x * run) {
         int pos = (int)first;
         const int end = min(pos + run, total);
@@ -554,10 +558,11 @@ batch_tbd_kernel(const BatchTBD* __restrict__ lat, const BatchInst* __restrict__
             pos += left;
             const int ke = min(kb + left, L->nz);
             if (kb >= ke) continue;                    // padding of the last chunk
-            if (!tbd_segment<false, NST, TXI>(R, F, item % tiles, kb, ke)) {
+            if (!tbd_segment<false, NST, TXI>(R, F, item % tiles, kb, ke, early)) {
                 tbd_ring_drain<NST>(R);
                 return;
             }
+            early = false;
         }
     }
 }
