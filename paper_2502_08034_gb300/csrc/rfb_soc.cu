@@ -876,7 +876,7 @@ ResKernel res_kernel(int cpt) {
 }
 
 // The resident FP32 sweeps are the faster ones wherever the lattice fits (up to about 0.9 M
-// cells): 1.9 us a sweep at 528k cells, where launches and passes take 6.2 us.
+// cells): 1.7 us a sweep at 528k cells, where launches and passes take 6.2 us.
 bool res_fits(rfb_soc_handle* h) {
     if (h->res.cpt < 0) res_plan(h, h->res, {2, 4, 6, 8, 10, 12}, 2 * RES_RING);
     return h->res.cpt > 0;

@@ -352,8 +352,9 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
 // ---------------------------------------------------------------------------------
 constexpr int RES64_RING = 4;      // x / y halo values polled per edge thread, at most
 // coefficients of a cell kept in shared memory (the last ones; registers hold the others):
-// eight doubles for three to six cells do not fit beside the values at 128 registers (48x48x96
-// 3.79 us a sweep with none of four cells' in shared memory, 3.65 with two a cell)
+// eight doubles for three to six cells do not fit beside the values at 128 registers (four
+// cells: 264 bytes of spills with none of them in shared memory, 40 with two a cell; 64^3 4.7
+// and 4.5 us a sweep)
 __host__ __device__ constexpr int res64_shared(int cpt) { return cpt >= 6 ? 4 : cpt >= 5 ? 3 : cpt >= 4 ? 2 : cpt >= 3 ? 1 : 0; }
 __host__ __device__ constexpr int res64_smem(int cpt) {
     return (2 * cpt * RES_PLANE + cpt * res64_shared(cpt) * RES_T) * (int)sizeof(double);
