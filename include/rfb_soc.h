@@ -205,7 +205,8 @@ rfb_status rfb_soc_set_stream(rfb_soc_handle* h, void* cuda_stream);
  *   res    nullable; filled on return (also on NOT_CONVERGED / NONFINITE)
  * Starts from the current state if one is set (previous solve, rfb_soc_set_state or
  * rfb_soc_upsample), otherwise from s = s_in on every fluid cell.
- * RFB_PREC_MIXED: cycles of opts.check_every (default 200) FP32 correction sweeps
+ * RFB_PREC_MIXED: cycles of opts.check_every (default: up to 200, a whole multiple of one, two
+ * or three by the lattice or by the kernel asked for) FP32 correction sweeps
  * delta <- delta + dt (L delta + r) followed by a defect check that adds delta to the
  * state and refreshes r; res->residual and the outputs come from an FP64 check of the
  * returned state. Kinetics mode 1 requires RFB_PREC_FP64.

@@ -143,6 +143,9 @@ struct rfb_soc_handle {
     CUtensorMap tmn_delta[2], tmn_r, tmn_u, tmn_v, tmn_w, tmn_t;   // narrow tiles
     TBDCut cut{64, TB_TYI};                 // their size
     float* tm_delta_ptr[2] = {nullptr, nullptr};
+    bool tb_forced = false;   // the variant is one that a call asked for
+    int auto_depth = 1;       // sweeps whose multiples the check intervals are: fp32_kernel 0,
+    int pass_depth = 0;       // fp32_kernel 2 (0: the variant's own)
     double tb_tuned_plain_ms = 0, tb_tuned_tb_ms = 0;
     // resident sweeps (sweep_res.cuh), FP32 and FP64: bricks of the lattice, inboxes (first
     // use), the tag of the next launch's words
@@ -648,6 +651,18 @@ void tb_encode(rfb_soc_handle* h, CUtensorMap* m, CUtensorMapDataType t, size_t 
     }
 }
 
+// The chunk count of a pass of k sweeps (tiles x chunks work items on `slots` CTAs) with the
+// fewest plane steps, waves x (chunk + k); those steps.
+double best_chunks(int64_t tiles, int nz, int slots, int k, int* chunks) {
+    double best = INFINITY;
+    for (int c = 1; c <= std::max(1, nz / 8); ++c) {
+        const int lc = (nz + c - 1) / c, cc = (nz + lc - 1) / lc;
+        const double cost = std::ceil((double)(tiles * cc) / slots) * (lc + k);
+        if (cost < best) { best = cost; *chunks = cc; }
+    }
+    return best;
+}
+
 void tb_prepare(rfb_soc_handle* h) {
     if (h->tm_ready) return;
     // The shared-memory limit is an attribute of the kernel in the current device's
@@ -726,12 +741,7 @@ void tb_prepare(rfb_soc_handle* h) {
         P.per = std::max<int64_t>((P.total + slots - 1) / slots, 16);
         P.grid = dim3((unsigned)((P.total + P.per - 1) / P.per));
         int best_c = 1;
-        double best = INFINITY;
-        for (int c = 1; c <= std::max(1, h->nz / 8); ++c) {
-            const int lc = (h->nz + c - 1) / c, cc = (h->nz + lc - 1) / lc;
-            const double cost = std::ceil((double)(tiles * cc) / slots) * (lc + k);
-            if (cost < best) { best = cost; best_c = cc; }
-        }
+        best_chunks(tiles, h->nz, slots, k, &best_c);
         auto& Q = h->tb_launch[2 * g + 1];
         Q.lc = (h->nz + best_c - 1) / best_c;
         Q.total = tiles * best_c * Q.lc;
@@ -747,9 +757,9 @@ int tb_depth(const rfb_soc_handle* h) {
 }
 
 // one pass (two or three sweeps) from delta[cur] into delta[cur ^ 1] (tr: of the
-// transposed operator; local steps only)
+// transposed operator; local steps only; apart: begins when the pass before it has ended)
 void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur, bool local,
-             bool tr = false) {
+             bool tr = false, bool apart = false) {
     const int at = h->d_delta[cur] == h->tm_delta_ptr[0] ? 0 : 1;
     const CUtensorMap& td = h->tm_delta[at];
     if (local) {
@@ -765,6 +775,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
         A.omc = (float)(1.0 - op.cfl);
         A.Dh = C.Dh;
         A.err = wait_err_word(h);
+        A.early = apart ? 0 : 1;
         const bool four = (v & 2) != 0;
         if (v >= 4 && !narrow) {
             if (tr && four)
@@ -796,7 +807,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
         cfg.dynamicSmemBytes = narrow ? tbd_smem<3, 0>() : four ? tbd_smem<4>() : tbd_smem<3>();
         cfg.stream = h->stream;
         cfg.attrs = &at1;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = apart ? 0 : 1;
         if (narrow)
             CK(h, cudaLaunchKernelEx(&cfg, k, h->tmn_delta[at], h->tmn_r, h->tmn_u, h->tmn_v,
                                      h->tmn_w, h->tmn_t, A));
@@ -882,6 +893,29 @@ bool res_fits(rfb_soc_handle* h) {
     return h->res.cpt > 0;
 }
 
+// Sweeps whose multiples the check intervals of a default solve are where its sweeps run
+// resident: the depth of the launches that the resident sweeps replaced (why: see
+// tune_fp32_kernel), by a rule on their shapes instead of a timing, so that a solve stops at
+// the same sweep every time. One-sweep launches were the fastest where one wave of their
+// blocks fills the chip (three blocks of 256 threads per SM, together up to 10 2/3 planes:
+// 6.7 to 7.7 us a sweep, beyond that 8.8 and more); of the passes the three-sweep ones (7.4 to
+// 7.6 us up to 12 plane steps, from 13 on 8.1 and more) where the two-sweep ones take 11 steps
+// (7.7 to 8.0; with 10 steps 7.0). A timing came to the same on 129 of 147 lattices of up to
+// 1 M cells; of the others 17 take as long either way within 4 %, and the blocks of one
+// (132x44x114) are half empty.
+int res_depth(rfb_soc_handle* h) {
+    if (!tb_eligible(h, true)) return 1;
+    int sms = 152, chunks = 1;
+    CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    const int64_t blocks = (int64_t)h->vgrid.x * h->vgrid.y * h->vgrid.z;
+    if (blocks <= 3 * sms && 3 * blocks * h->vkchunk <= 32 * sms) return 1;
+    auto steps = [&](int rows, int k) {
+        const int64_t tiles = (int64_t)((h->nx + TB_TXI - 1) / TB_TXI) * ((h->ny + rows - 1) / rows);
+        return best_chunks(tiles, h->nz, sms, k, &chunks);
+    };
+    return steps(TB_TYI, 2) > 10 && steps(T3_TYI, 3) <= 12 ? 3 : 2;
+}
+
 // n sweeps (tr: of the transposed operator) from delta = 0; the result is left in d_delta[0].
 // One launch does them all, or 4096 at a time (a launch of some ms).
 void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n, bool tr) {
@@ -918,8 +952,9 @@ void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int6
 }
 
 // How a call's FP32 sweeps run: one launch per sweep, passes of the chosen variant (two or
-// three sweeps each, single sweeps for the remainder), or resident sweeps.
-enum class Sweep32 { plain, pass, resident };
+// three sweeps each, single sweeps for the remainder; apart: one after the other, to time
+// them), or resident sweeps.
+enum class Sweep32 { plain, pass, apart, resident };
 
 // n FP32 correction sweeps delta <- delta + dt (L delta + r), starting from delta = 0.
 // The result is left in d_delta[0].
@@ -928,7 +963,7 @@ void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Swe
         res_sweeps(h, op, make_coef<float>(h, op, true, false), n, false);
         return;
     }
-    const bool use_tb = how == Sweep32::pass;
+    const bool use_tb = how != Sweep32::plain;
     const size_t bytes = (size_t)h->N * sizeof(float);
     CK(h, cudaMemsetAsync(h->d_delta[0], 0, bytes, h->stream));
     CK(h, cudaMemsetAsync(h->d_delta[1], 0, bytes, h->stream));
@@ -942,7 +977,7 @@ void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Swe
         tb_prepare(h);
         const int k = tb_depth(h);
         for (; q + k <= n; q += k) {
-            tb_pass(h, op, C, cur, local);
+            tb_pass(h, op, C, cur, local, false, how == Sweep32::apart);
             cur ^= 1;
         }
     }
@@ -1002,7 +1037,7 @@ struct TuneKey {
     }
 };
 struct TuneVal {
-    int tb_mode, tb_variant;
+    int tb_mode, tb_variant, auto_depth, pass_depth;
     double plain_ms, tb_ms;
 };
 std::map<TuneKey, TuneVal> g_tune_cache;
@@ -1012,8 +1047,24 @@ std::mutex g_tune_mu;
 // sweeps and 12 sweeps of each launch shape of the two-sweep pass (with local steps: with
 // three and with four TMA stages, and with narrow tiles) by CUDA events on the current
 // forcing and keep the fastest (tb_only: choose between the pass variants only).
+//
+// The check intervals follow another choice, made here too: whole multiples of one, two or
+// three sweeps, whichever takes the least time a sweep in launches that begin when the one
+// before has ended. What a solve returns depends on where its checks lie: where a pocket
+// converges slowly, two sweeps more or less move single cells by far more than rounding. So
+// the intervals do not change with the way the sweeps are launched: overlapping passes made
+// two sweeps the faster depth where three was (256^3: 41.0 and 42.3 us a sweep; apart 45.0 and
+// 44.1), and the solves there stopped at other sweeps. Of each depth the shapes that came first
+// anywhere are timed (420 lattices of 1.3 to 16 M cells: in all but 12 the depth that was the
+// fastest of all shapes before passes overlapped; in those two depths lie within the spread of
+// the timing).
 void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false) {
-    if (!tb_eligible(h, op.dt_mode == RFB_DT_LOCAL)) { h->tb_mode = 0; return; }
+    if (!tb_eligible(h, op.dt_mode == RFB_DT_LOCAL)) {
+        h->tb_mode = 0;
+        h->auto_depth = 1;
+        return;
+    }
+    h->tb_forced = false;
     const TuneKey key{h->nx, h->ny, h->nz, h->d_m32 != nullptr,
                       op.dt_mode == RFB_DT_LOCAL, h->device};
     {
@@ -1022,6 +1073,8 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
         if (it != g_tune_cache.end() && (tb_only || it->second.tb_mode >= 0)) {
             h->tb_variant = it->second.tb_variant;
             if (!tb_only) h->tb_mode = it->second.tb_mode;
+            h->auto_depth = it->second.auto_depth;
+            h->pass_depth = it->second.pass_depth;
             h->tb_tuned_plain_ms = it->second.plain_ms;
             h->tb_tuned_tb_ms = it->second.tb_ms;
             return;
@@ -1035,8 +1088,8 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
     if (op.dt_mode == RFB_DT_LOCAL) cands = {0, 1, 2, 3, 8, 9};
     float ms[10], plain_ms = INFINITY;
     for (float& m : ms) m = INFINITY;
-    auto time_one = [&](int v, float& best) {
-        const Sweep32 how = v < 0 ? Sweep32::plain : Sweep32::pass;
+    auto time_one = [&](int v, float& best, bool apart = false) {
+        const Sweep32 how = v < 0 ? Sweep32::plain : apart ? Sweep32::apart : Sweep32::pass;
         if (v >= 0) h->tb_variant = v;
         sweeps32(h, op, 6, how);   // warm-up (and tensor maps)
         for (int rep = 0; rep < 2; ++rep) {   // the faster of two timings
@@ -1051,6 +1104,15 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
     };
     if (!tb_only) time_one(-1, plain_ms);
     for (int v : cands) time_one(v, ms[v]);
+    float two = INFINITY, three = INFINITY;              // launched apart, as above
+    if (op.dt_mode == RFB_DT_LOCAL) {
+        for (int v : {1, 2, 3}) time_one(v, two, true);
+        for (int v : {4, 5}) time_one(v, three, true);
+    } else {
+        two = std::min(ms[0], ms[1]);                    // its passes never overlap
+    }
+    h->pass_depth = two <= three ? 2 : 3;
+    h->auto_depth = plain_ms <= std::min(two, three) ? 1 : h->pass_depth;
     int bestv = 0;
     for (int v : cands)
         if (ms[v] < ms[bestv]) bestv = v;
@@ -1060,8 +1122,8 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
     h->tb_tuned_tb_ms = tb / 12;
     if (!tb_only) h->tb_mode = tb < plain_ms ? 1 : 0;
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune_cache[key] = TuneVal{tb_only ? -1 : h->tb_mode, h->tb_variant, h->tb_tuned_plain_ms,
-                                h->tb_tuned_tb_ms};
+    g_tune_cache[key] = TuneVal{tb_only ? -1 : h->tb_mode, h->tb_variant, h->auto_depth,
+                                h->pass_depth, h->tb_tuned_plain_ms, h->tb_tuned_tb_ms};
 }
 
 void init_state(rfb_soc_handle* h, bool umt, double s_in) {
@@ -1199,14 +1261,22 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
                             : o.fp32_kernel <= 6 ? (o.fp32_kernel - 5) | 2
                             : o.fp32_kernel <= 8 ? (o.fp32_kernel - 7) | 4
                                                   : (o.fp32_kernel - 9) | 6;
+            h->tb_forced = true;
             use_tb = true;
         } else if (o.fp32_kernel == 0) {
             if (h->tb_mode < 0) tune_fp32_kernel(h, op);
             use_tb = h->tb_mode == 1;
         }
     }
-    // sweeps per pass: the default interval and the shortened ones are whole passes
-    const int depth = use_tb ? tb_depth(h) : 1;
+    // the default check interval and the shortened ones are whole multiples of `depth` sweeps
+    // (a variant that a call asked for keeps its own)
+    int depth = 1;
+    if (use_res) depth = res_depth(h);
+    else if (use_tb && (o.fp32_kernel >= 2 && (h->tb_forced || h->pass_depth == 0)))
+        depth = tb_depth(h);
+    else if (mixed && o.fp32_kernel == 2) depth = h->pass_depth;
+    else if (mixed && o.fp32_kernel == 0 && h->auto_depth > 1)
+        depth = h->tb_forced ? tb_depth(h) : h->auto_depth;
     const Sweep32 how = use_res ? Sweep32::resident : use_tb ? Sweep32::pass : Sweep32::plain;
     if (o.check_every == 0) every = std::max<int64_t>(depth, every / depth * depth);
     // Check interval: `every` sweeps, shortened near the end. The residual of these
@@ -1214,9 +1284,8 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
     // inlet state is carried through the lattice, then falls faster), so a crossing
     // extrapolated from the last two checks lies too late there and the interval stays at
     // `every`; in the geometric tail the extrapolation is accurate, and the next check is
-    // placed just past the predicted crossing of tol (at least 16 sweeps, whole passes) instead of
-    // up to `every` sweeps beyond it; intervals are whole passes of the FP32 kernel. One
-    // check costs about 9 to 13 FP32 sweeps.
+    // placed just past the predicted crossing of tol (at least 16 sweeps) instead of up to
+    // `every` sweeps beyond it. One check costs about 9 to 13 FP32 sweeps.
     int64_t next_every = every;
     while (true) {
         if (r.nonfinite > 0) { st = RFB_ERR_NONFINITE; break; }

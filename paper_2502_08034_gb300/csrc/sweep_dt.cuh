@@ -203,6 +203,7 @@ struct TBDArgs {
     int lc;                           // planes per z chunk (nz: one chunk)
     int64_t total;                    // tiles x chunks x lc (chunk-major, tile fastest)
     int64_t per;                      // planes of that space per CTA
+    int early;                        // the launch may start before the pass before it has ended
     const float* __restrict__ d_in;   // delta read by this pass (prologue plane)
     float* __restrict__ d_out;
     float omc, Dh;
@@ -324,9 +325,13 @@ __device__ __forceinline__ bool tbd_segment(TBDRing<NST, TXI>& R, const TBDField
         issue_delta(p, s);
     };
     __syncthreads();   // the previous segment's readers are done with every stage
-    for (int s = 0; s < NST; ++s) issue_rest(kb - 1 + s, s);            // kb-1, kb, ...
-    if (early) grid_wait();
-    for (int s = 0; s < NST; ++s) issue_delta(kb - 1 + s, s);
+    if (early) {                                                        // kb-1, kb, ...
+        for (int s = 0; s < NST; ++s) issue_rest(kb - 1 + s, s);
+        grid_wait();
+        for (int s = 0; s < NST; ++s) issue_delta(kb - 1 + s, s);
+    } else {
+        for (int s = 0; s < NST; ++s) issue(kb - 1 + s, s);
+    }
 
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 l1_m2 = zero4, l1_m1 = zero4;               // own level 1 at z-2, z-1
@@ -450,7 +455,7 @@ sweep32tbd_kernel(const __grid_constant__ CUtensorMap tm_d, const __grid_constan
     const int txi = TXI ? TXI : A.cut.txi, tyi = TXI ? TB_TYI : A.cut.tyi;
     const int tiles = ((A.nx + txi - 1) / txi) * ((A.ny + tyi - 1) / tyi);
     const int64_t q1 = min((int64_t)(blockIdx.x + 1) * A.per, A.total);
-    bool ok = true, first = true;
+    bool ok = true, first = A.early != 0;
     for (int64_t q = (int64_t)blockIdx.x * A.per; q < q1 && ok;) {
         const int64_t item = q / A.lc;
         const int zl = (int)(q % A.lc);
