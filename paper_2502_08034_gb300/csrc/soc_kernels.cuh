@@ -1439,6 +1439,7 @@ batch_check_df_kernel(const BatchInst* __restrict__ insts, const BatchItem* __re
         const BatchInst* I = insts + it.inst;
         float sum2 = 0.f, vmax = 0.f;
         int bad = 0;
+        __syncthreads();   // the sums of the item before have been read
         if (I->active) {   // uniform over the block
             const Lattice L = I->L;
             const L2F K = I->K2;
