@@ -121,8 +121,7 @@ struct rfb_soc_handle {
     dim3 sgrid;
     int vkchunk = 8;          // vectorised FP32 sweep (nx % 4 == 0)
     dim3 vgrid, vblock;
-    // temporally blocked FP32 sweep (nx % 16 == 0, no area multiplier)
-    int tb_mode = -1;         // -1 not chosen yet, 0 one-sweep kernel, 1 two-sweep passes
+    // temporally blocked FP32 sweeps (tb_eligible)
     // two launch shapes of the two-sweep pass (sweep_tb.cuh): 0 persistent (one CTA per
     // SM, equal shares of the tile-major plane space), 1 one (tile, z chunk) item per CTA
     // with the chunk count that wastes least of the last wave; the autotuner picks one
@@ -133,20 +132,26 @@ struct rfb_soc_handle {
         dim3 grid;
     } tb_launch[6];           // 2, 3: the same shapes for the three-sweep pass; 4, 5: for the
                               // two-sweep pass with narrow tiles (two CTAs per SM)
-    int tb_variant = -1;      // -1 not chosen yet; bit 0 the launch shape; step-field
+    // The choice among one-sweep launches and passes, for each pseudo-time step by itself: its
+    // passes take other lattices (tb_eligible), maps and sweeps a pass.
+    struct TBChoice {
+        int mode = -1;        // -1 not chosen yet, 0 one-sweep kernel, 1 passes
+        int variant = -1;     // -1 not chosen yet; bit 0 the launch shape; step-field
                               // passes only: bit 1 one more TMA stage of delta (two-sweep:
                               // four instead of three; three-sweep: five instead of four),
                               // bit 2 three sweeps per pass instead of two; 8, 9: two
                               // sweeps, narrow tiles
+        bool forced = false;  // the variant is one that a call asked for
+        int auto_depth = 1;   // sweeps whose multiples the check intervals are: fp32_kernel 0,
+        int pass_depth = 0;   // fp32_kernel 2 (0: the variant's own)
+        double plain_ms = 0, pass_ms = 0;   // timed, per sweep
+    } tb[2];                  // the global step's, the local steps'
+    int tb_last = 1;          // the one of the last mixed solve
     bool tm_ready = false;
     CUtensorMap tm_delta[2], tm_r, tm_u, tm_v, tm_w, tm_f, tm_t;
     CUtensorMap tmn_delta[2], tmn_r, tmn_u, tmn_v, tmn_w, tmn_t;   // narrow tiles
     TBDCut cut{64, TB_TYI};                 // their size
     float* tm_delta_ptr[2] = {nullptr, nullptr};
-    bool tb_forced = false;   // the variant is one that a call asked for
-    int auto_depth = 1;       // sweeps whose multiples the check intervals are: fp32_kernel 0,
-    int pass_depth = 0;       // fp32_kernel 2 (0: the variant's own)
-    double tb_tuned_plain_ms = 0, tb_tuned_tb_ms = 0;
     // resident sweeps (sweep_res.cuh), FP32 and FP64: bricks of the lattice, inboxes (first
     // use), the tag of the next launch's words
     struct ResPlan {
@@ -752,8 +757,9 @@ void tb_prepare(rfb_soc_handle* h) {
 }
 
 // sweeps of one pass of the chosen variant
-int tb_depth(const rfb_soc_handle* h) {
-    return h->tb_variant >= 4 && h->tb_variant < 8 ? 3 : 2;
+int tb_depth(const rfb_soc_handle* h, bool local) {
+    const int v = h->tb[local].variant;
+    return local && v >= 4 && v < 8 ? 3 : 2;
 }
 
 // one pass (two or three sweeps) from delta[cur] into delta[cur ^ 1] (tr: of the
@@ -766,7 +772,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
         TBDArgs A{};
         A.nx = h->nx; A.ny = h->ny; A.nz = h->nz;
         A.cut = h->cut;
-        const int v = std::max(h->tb_variant, 0);
+        const int v = std::max(h->tb[1].variant, 0);
         const bool narrow = v >= 8;
         const auto& S = h->tb_launch[(narrow ? 4 : v >= 4 ? 2 : 0) + (v & 1)];
         A.lc = S.lc; A.total = S.total; A.per = S.per;
@@ -818,7 +824,7 @@ void tb_pass(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int cur
     }
     TBArgs A{};
     A.nx = h->nx; A.ny = h->ny; A.nz = h->nz;
-    const auto& S = h->tb_launch[std::max(h->tb_variant, 0) & 1];
+    const auto& S = h->tb_launch[std::max(h->tb[0].variant, 0) & 1];
     A.lc = S.lc; A.total = S.total; A.per = S.per;
     A.d_in = h->d_delta[cur];
     A.d_out = h->d_delta[cur ^ 1];
@@ -975,7 +981,7 @@ void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Swe
     int64_t q = 0;
     if (use_tb) {
         tb_prepare(h);
-        const int k = tb_depth(h);
+        const int k = tb_depth(h, local);
         for (; q + k <= n; q += k) {
             tb_pass(h, op, C, cur, local, false, how == Sweep32::apart);
             cur ^= 1;
@@ -994,7 +1000,7 @@ void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Swe
 // before, else passes of the step-field kernels (two or three sweeps each, the variant the
 // autotuner chose), plain sweeps for the remainder.
 void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n) {
-    if (op.dt_mode == RFB_DT_LOCAL && h->tb_variant < 0 && res_fits(h)) {
+    if (op.dt_mode == RFB_DT_LOCAL && h->tb[1].variant < 0 && res_fits(h)) {
         res_sweeps(h, op, C, n, true);
         return;
     }
@@ -1007,8 +1013,8 @@ void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C
     int64_t q = 0;
     if (local && tb_eligible(h, true)) {
         tb_prepare(h);
-        if (h->tb_variant < 0) h->tb_variant = 1;   // chunked shape unless tuned
-        const int k = tb_depth(h);
+        if (h->tb[1].variant < 0) h->tb[1].variant = 1;   // chunked shape unless tuned
+        const int k = tb_depth(h, true);
         for (; q + k <= n; q += k) {
             tb_pass(h, op, C, cur, true, true);
             cur ^= 1;
@@ -1036,11 +1042,7 @@ struct TuneKey {
                std::tie(o.nx, o.ny, o.nz, o.mult, o.local, o.device);
     }
 };
-struct TuneVal {
-    int tb_mode, tb_variant, auto_depth, pass_depth;
-    double plain_ms, tb_ms;
-};
-std::map<TuneKey, TuneVal> g_tune_cache;
+std::map<TuneKey, rfb_soc_handle::TBChoice> g_tune_cache;
 std::mutex g_tune_mu;
 
 // Project-written autotuner for one lattice: time (twice, keeping the faster) 12 plain
@@ -1059,24 +1061,21 @@ std::mutex g_tune_mu;
 // fastest of all shapes before passes overlapped; in those two depths lie within the spread of
 // the timing).
 void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false) {
-    if (!tb_eligible(h, op.dt_mode == RFB_DT_LOCAL)) {
-        h->tb_mode = 0;
-        h->auto_depth = 1;
+    const bool local = op.dt_mode == RFB_DT_LOCAL;
+    auto& T = h->tb[local];
+    if (!tb_eligible(h, local)) {
+        T.mode = 0;
+        T.auto_depth = 1;
         return;
     }
-    h->tb_forced = false;
-    const TuneKey key{h->nx, h->ny, h->nz, h->d_m32 != nullptr,
-                      op.dt_mode == RFB_DT_LOCAL, h->device};
+    const TuneKey key{h->nx, h->ny, h->nz, h->d_m32 != nullptr, local, h->device};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
-        if (it != g_tune_cache.end() && (tb_only || it->second.tb_mode >= 0)) {
-            h->tb_variant = it->second.tb_variant;
-            if (!tb_only) h->tb_mode = it->second.tb_mode;
-            h->auto_depth = it->second.auto_depth;
-            h->pass_depth = it->second.pass_depth;
-            h->tb_tuned_plain_ms = it->second.plain_ms;
-            h->tb_tuned_tb_ms = it->second.tb_ms;
+        if (it != g_tune_cache.end() && (tb_only || it->second.mode >= 0)) {
+            const int mode = tb_only ? T.mode : it->second.mode;
+            T = it->second;
+            T.mode = mode;
             return;
         }
     }
@@ -1085,12 +1084,12 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
     // lattice measured (us per sweep of the best of each: 128x128x256 10.6 and 13.7, 160x160x200
     // 18.8 and 23.2, 192^3 22.7 and 26.6, 256^3 41.0 and 42.3, 256x256x512 75 and 87).
     std::vector<int> cands = {0, 1};
-    if (op.dt_mode == RFB_DT_LOCAL) cands = {0, 1, 2, 3, 8, 9};
+    if (local) cands = {0, 1, 2, 3, 8, 9};
     float ms[10], plain_ms = INFINITY;
     for (float& m : ms) m = INFINITY;
     auto time_one = [&](int v, float& best, bool apart = false) {
         const Sweep32 how = v < 0 ? Sweep32::plain : apart ? Sweep32::apart : Sweep32::pass;
-        if (v >= 0) h->tb_variant = v;
+        if (v >= 0) T.variant = v;
         sweeps32(h, op, 6, how);   // warm-up (and tensor maps)
         for (int rep = 0; rep < 2; ++rep) {   // the faster of two timings
             float t = 0.f;
@@ -1105,25 +1104,26 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
     if (!tb_only) time_one(-1, plain_ms);
     for (int v : cands) time_one(v, ms[v]);
     float two = INFINITY, three = INFINITY;              // launched apart, as above
-    if (op.dt_mode == RFB_DT_LOCAL) {
+    if (local) {
         for (int v : {1, 2, 3}) time_one(v, two, true);
         for (int v : {4, 5}) time_one(v, three, true);
     } else {
         two = std::min(ms[0], ms[1]);                    // its passes never overlap
     }
-    h->pass_depth = two <= three ? 2 : 3;
-    h->auto_depth = plain_ms <= std::min(two, three) ? 1 : h->pass_depth;
+    T.pass_depth = two <= three ? 2 : 3;
+    T.auto_depth = plain_ms <= std::min(two, three) ? 1 : T.pass_depth;
     int bestv = 0;
     for (int v : cands)
         if (ms[v] < ms[bestv]) bestv = v;
-    h->tb_variant = bestv;
-    const float tb = ms[bestv];
-    h->tb_tuned_plain_ms = tb_only ? INFINITY : plain_ms / 12;
-    h->tb_tuned_tb_ms = tb / 12;
-    if (!tb_only) h->tb_mode = tb < plain_ms ? 1 : 0;
+    T.variant = bestv;
+    T.forced = false;
+    T.plain_ms = plain_ms / 12;
+    T.pass_ms = ms[bestv] / 12;
+    if (!tb_only) T.mode = ms[bestv] < plain_ms ? 1 : 0;
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune_cache[key] = TuneVal{tb_only ? -1 : h->tb_mode, h->tb_variant, h->auto_depth,
-                                h->pass_depth, h->tb_tuned_plain_ms, h->tb_tuned_tb_ms};
+    auto& kept = g_tune_cache[key];
+    kept = T;
+    if (tb_only) kept.mode = -1;
 }
 
 void init_state(rfb_soc_handle* h, bool umt, double s_in) {
@@ -1246,37 +1246,40 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
     };
     // FP32 kernel: resident sweeps where the lattice fits on the chip (local steps), else
     // one-sweep launches or passes (forced by opts or autotuned once)
+    const bool local = op.dt_mode == RFB_DT_LOCAL;
+    auto& T = h->tb[local];
     bool use_tb = false, use_res = false;
     if (mixed) {
-        use_res = o.fp32_kernel == 0 && op.dt_mode == RFB_DT_LOCAL && res_fits(h);
+        h->tb_last = local;
+        use_res = o.fp32_kernel == 0 && local && res_fits(h);
         h->res_used = use_res;
         if (use_res) {
         } else if (o.fp32_kernel == 2) {
-            if (h->tb_variant < 0) tune_fp32_kernel(h, op, true);
+            if (T.variant < 0) tune_fp32_kernel(h, op, true);
             use_tb = true;
         } else if (o.fp32_kernel >= 3) {
             // a forced variant (kept for later calls): 3 / 4 and 5 / 6 two-sweep passes with
             // three / four TMA stages, 7 / 8 and 9 / 10 three-sweep passes with four / five
-            h->tb_variant = o.fp32_kernel <= 4 ? o.fp32_kernel - 3
-                            : o.fp32_kernel <= 6 ? (o.fp32_kernel - 5) | 2
-                            : o.fp32_kernel <= 8 ? (o.fp32_kernel - 7) | 4
-                                                  : (o.fp32_kernel - 9) | 6;
-            h->tb_forced = true;
+            T.variant = o.fp32_kernel <= 4   ? o.fp32_kernel - 3
+                        : o.fp32_kernel <= 6 ? (o.fp32_kernel - 5) | 2
+                        : o.fp32_kernel <= 8 ? (o.fp32_kernel - 7) | 4
+                                             : (o.fp32_kernel - 9) | 6;
+            T.forced = true;
             use_tb = true;
         } else if (o.fp32_kernel == 0) {
-            if (h->tb_mode < 0) tune_fp32_kernel(h, op);
-            use_tb = h->tb_mode == 1;
+            if (T.mode < 0) tune_fp32_kernel(h, op);
+            // (area multipliers may have come since)
+            use_tb = T.mode == 1 && tb_eligible(h, local);
         }
     }
     // the default check interval and the shortened ones are whole multiples of `depth` sweeps
     // (a variant that a call asked for keeps its own)
     int depth = 1;
     if (use_res) depth = res_depth(h);
-    else if (use_tb && (o.fp32_kernel >= 2 && (h->tb_forced || h->pass_depth == 0)))
-        depth = tb_depth(h);
-    else if (mixed && o.fp32_kernel == 2) depth = h->pass_depth;
-    else if (mixed && o.fp32_kernel == 0 && h->auto_depth > 1)
-        depth = h->tb_forced ? tb_depth(h) : h->auto_depth;
+    else if (use_tb && o.fp32_kernel >= 2 && (T.forced || T.pass_depth == 0)) depth = tb_depth(h, local);
+    else if (mixed && o.fp32_kernel == 2) depth = T.pass_depth;
+    else if (mixed && o.fp32_kernel == 0 && T.auto_depth > 1 && tb_eligible(h, local))
+        depth = T.forced ? tb_depth(h, local) : T.auto_depth;
     const Sweep32 how = use_res ? Sweep32::resident : use_tb ? Sweep32::pass : Sweep32::plain;
     if (o.check_every == 0) every = std::max<int64_t>(depth, every / depth * depth);
     // Check interval: `every` sweeps, shortened near the end. The residual of these
@@ -2660,15 +2663,16 @@ rfb_status rfb_soc_tuned_fp32_kernel(const rfb_soc_handle* h, int32_t* kernel,
                                      double* blocked_ms_per_sweep) {
     if (!h) return RFB_ERR_INVALID_ARG;
     int32_t k = 0;
+    const auto& T = h->tb[h->tb_last];
     if (h->res_used) k = 11;
-    else if (h->tb_mode == 0) k = 1;
-    else if (h->tb_mode == 1 || h->tb_variant >= 0) {
-        const int v = std::max(h->tb_variant, 0);
+    else if (T.mode == 0) k = 1;
+    else if (T.mode == 1 || T.variant >= 0) {
+        const int v = std::max(T.variant, 0);
         k = (v >= 8 ? 12 : v & 4 ? (v & 2 ? 9 : 7) : (v & 2 ? 5 : 3)) + (v & 1);
     }
     if (kernel) *kernel = k;
-    if (plain_ms_per_sweep) *plain_ms_per_sweep = h->tb_tuned_plain_ms;
-    if (blocked_ms_per_sweep) *blocked_ms_per_sweep = h->tb_tuned_tb_ms;
+    if (plain_ms_per_sweep) *plain_ms_per_sweep = T.plain_ms;
+    if (blocked_ms_per_sweep) *blocked_ms_per_sweep = T.pass_ms;
     return RFB_OK;
 }
 
