@@ -525,6 +525,12 @@ rfb_status rfb_soc_get_bv_state(rfb_soc_handle* h, double* c_o, double* c_r, dou
  * argument, RFB_ERR_CUDA if a CUDA call failed (detail in rfb_soc_last_error(NULL)). */
 rfb_status rfb_selftest_bounded_wait(int64_t spin_limit, int32_t* gave_up);
 
+/* Self-test of the resident kernels' waits (a CTA polls for its neighbours' values): from now on
+ * each wait of this handle's launches gives up after `polls` polls, 1 .. 2^26 (0: the default,
+ * about a second). With a few polls the words are still on their way when a wait gives up: the
+ * call ends with RFB_ERR_CUDA, the states hold no result, and the next call runs as usual. */
+rfb_status rfb_selftest_wait_limit(rfb_soc_handle* h, int64_t polls);
+
 /* The FP32 correction kernel the handle's autotuner chose for RFB_PREC_MIXED solves with
  * fp32_kernel = 0 or 2 (or the one a solve forced), as an opts.fp32_kernel value: 0 = not
  * chosen yet, 1 = one sweep per launch, 3 / 4 = two-sweep passes in the persistent /

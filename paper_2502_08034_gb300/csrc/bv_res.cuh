@@ -110,7 +110,7 @@ struct ResBrick {
     __device__ __forceinline__ void poll(const unsigned long long* slot, int stride, uint32_t tag,
                                          double (&zlo)[NV], double (&zhi)[NV],
                                          double (&ring)[RING], unsigned int* err,
-                                         bool& good) const {
+                                         unsigned polls, bool& good) const {
         constexpr int NZ = 2 * NV, NI = NZ + RING;     // z words of value v: bits 2 v, 2 v + 1
         const unsigned long long* in = slot + 2 * own;
         uint32_t pend = (want >> 2) << NZ;
@@ -136,7 +136,7 @@ struct ResBrick {
                     pend &= ~(1u << m);
                 }
             }
-            if (spin >= RES_SPIN_LIMIT && pend) {
+            if (spin + 1 >= polls && pend) {
                 atomicExch(err, 1u);
                 good = false;
                 pend = 0;
@@ -158,6 +158,7 @@ struct ResReduce {
     double* sh;                    // 32 + 2 doubles of shared memory
     uint32_t tag;                  // of the next reduction
     unsigned int* err;
+    unsigned polls;                // of one wait, at most
     bool good;                     // this thread may wait (none of its waits gave up)
     bool dead;                     // a wait of this CTA gave up (the same in all its threads)
 
@@ -195,7 +196,7 @@ struct ResReduce {
 #pragma unroll
                 for (int m = 0; m < RES_LANE; ++m)
                     if ((pend & (1u << m)) && res_take64(word[m], tag, &v[m])) pend &= ~(1u << m);
-                if (spin >= RES_SPIN_LIMIT && pend) {
+                if (spin + 1 >= polls && pend) {
                     atomicExch(err, 1u);
                     good = false;
                     pend = 0;
@@ -235,6 +236,7 @@ struct BVCgArgs {
     unsigned long long* rows;
     double* out;                   // its, stalled, BV_STATS values, exchanges, reductions
     unsigned int* err;
+    unsigned polls;
 };
 constexpr int BV_CG_OUT = BV_STATS + 4;
 constexpr int BV_RING = 2;
@@ -258,7 +260,7 @@ __global__ void __launch_bounds__(T, 1) bv_cgr_kernel(const BVCgArgs A) {
     ResBrick<CPT, BV_RING, 1> G;
     G.init(A.cut, A.stride);
     double* const S = res_sd;
-    ResReduce R{A.rows, res_sd + CPT * RES_PLANE, A.rtag + 1, A.err, true, false};
+    ResReduce R{A.rows, res_sd + CPT * RES_PLANE, A.rtag + 1, A.err, A.polls, true, false};
     auto plus = [](double a, double b) { return a + b; };
     const int64_t nxny = B.nxny;
     const int64_t c0 = G.i + (int64_t)B.nx * G.j + nxny * G.k0;
@@ -304,7 +306,7 @@ __global__ void __launch_bounds__(T, 1) bv_cgr_kernel(const BVCgArgs A) {
         zlo[0] = zhi[0] = 0.0;
         for (int m = 0; m < BV_RING; ++m) ring[m] = 0.0;
         __syncwarp();                  // the warp's own words are sent before it starts polling
-        G.poll(slot(), A.stride, tag, zlo, zhi, ring, A.err, R.good);
+        G.poll(slot(), A.stride, tag, zlo, zhi, ring, A.err, A.polls, R.good);
     };
     // A v for the column e, v in S with its neighbours
     auto apply = [&](int e, const double (&v)[CPT], double lo, double hi) {
@@ -479,6 +481,7 @@ struct BVSweepArgs {
     unsigned long long* inbox;
     int stride;
     unsigned int* err;
+    unsigned polls;
 };
 constexpr int BVS_CPT = 2;         // cells of a column: 22 doubles each
 __host__ __device__ constexpr int bv_sweep_smem() {
@@ -620,7 +623,7 @@ __global__ void __launch_bounds__(T, 1) bv_sweepr_kernel(const BVSweepArgs A) {
         }
         if (!more) break;
         __syncwarp();                  // the warp's own words are sent before it starts polling
-        G.poll(slot, A.stride, tag, zlo, zhi, ring, A.err, good);
+        G.poll(slot, A.stride, tag, zlo, zhi, ring, A.err, A.polls, good);
 #pragma unroll
         for (int m = 0; m < BV_RING; ++m)
             if (G.want & (4u << m)) Sw[G.dst[m]] = ring[m];

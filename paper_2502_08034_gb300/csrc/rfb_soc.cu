@@ -166,6 +166,7 @@ struct rfb_soc_handle {
     double* cg_out = nullptr;                // its result
     uint32_t cg_rtag = 0;
     bool res_used = false;        // the last FP32 correction sweeps were resident ones
+    unsigned wait_polls = RES_SPIN_LIMIT;    // of a resident kernel's wait, at most
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 };
 
@@ -566,6 +567,7 @@ void res64_sweeps(rfb_soc_handle* h, const OpPoint& op, double** buf, int& cur, 
     A.g = g;
     A.umt = op.umt;
     A.err = wait_err_word(h);
+    A.polls = h->wait_polls;
     A.stride = res64_stride(P.cpt, P.bx, P.by);
     const int ctas = P.gx * P.gy * P.gz;
     if (!P.inbox) dalloc(h, &P.inbox, (size_t)ctas * 4 * A.stride);
@@ -936,6 +938,7 @@ void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int6
     A.omc = (float)(1.0 - op.cfl);
     A.Dh = C.Dh;
     A.err = wait_err_word(h);
+    A.polls = h->wait_polls;
     A.stride = res_stride(P.cpt, P.bx, P.by);
     const int ctas = P.gx * P.gy * P.gz;
     if (!P.inbox) dalloc(h, &P.inbox, (size_t)ctas * 2 * A.stride);
@@ -1869,6 +1872,7 @@ void bv_res_sweeps(rfb_soc_handle* h, const BVArgs& B, const double* phi, double
     A.phi = phi;
     A.stride = res64_stride(P.cpt, P.bx, P.by);
     A.err = wait_err_word(h);
+    A.polls = h->wait_polls;
     const int ctas = P.gx * P.gy * P.gz, smem = bv_sweep_smem();
     if (!P.inbox) dalloc(h, &P.inbox, (size_t)ctas * 12 * A.stride);
     A.inbox = P.inbox;
@@ -1904,6 +1908,7 @@ void bv_res_potential(rfb_soc_handle* h, const BVArgs& B, const double* kcell, c
     A.max_it = max_it;
     A.stride = res64_stride(P.cpt, P.bx, P.by);
     A.err = wait_err_word(h);
+    A.polls = h->wait_polls;
     const int ctas = P.gx * P.gy * P.gz, smem = bv_cg_smem(P.cpt);
     if (!P.inbox) {
         dalloc(h, &P.inbox, (size_t)ctas * 4 * A.stride);
@@ -2553,8 +2558,9 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
                 df_check(true);
                 joined = false;
                 done += n;
+                if (wait_gave_up(h)) { st = RFB_ERR_CUDA; break; }
             }
-            if (!joined) {
+            if (!joined && st != RFB_ERR_CUDA) {
                 const bool bad = st == RFB_ERR_NONFINITE;
                 join_and_check();
                 if (!bad && h->h_red[6] > 0) st = RFB_ERR_NONFINITE;
@@ -2568,6 +2574,7 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
             reduce_readback(h, 0);
             ++r.checks;
             rel = h->h_red[1] > 0 ? std::sqrt(h->h_red[0] / h->h_red[1]) : 0.0;
+            if (wait_gave_up(h)) { st = RFB_ERR_CUDA; break; }
             if (h->h_red[6] > 0) { st = RFB_ERR_NONFINITE; break; }
             if (rel <= tol) break;
             if (done >= o.max_sweeps) { st = RFB_ERR_NOT_CONVERGED; break; }
@@ -2590,6 +2597,12 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
             }
             done += n;
         }
+        if (st == RFB_ERR_CUDA) {   // the cycle's values mean nothing: no gradient
+            r.sweeps = done;
+            r.residual = rel;
+            if (res) *res = r;
+            return st;
+        }
         // gradients
         const double kap0A = umt ? 0.0 : h->kin.k0 / h->h * (C.nl ? op.K1 : op.A);
         const double kap0B = umt ? 0.0 : h->kin.k0 / h->h * op.B;
@@ -2598,7 +2611,6 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
             umt ? nullptr : h->d_grad, h->d_partials, h->kchunk);
         LAUNCHED(h);
         reduce_readback(h, 0);
-        if (wait_gave_up(h)) st = RFB_ERR_CUDA;
         double dbeta = jscale * h->h_red[0] / op.beta;
         if (obj == RFB_OBJ_U) dbeta -= fwd.U / op.beta;
         if (umt) CK(h, cudaMemsetAsync(h->d_grad, 0, N * 8, h->stream));
@@ -2655,6 +2667,16 @@ rfb_status rfb_selftest_bounded_wait(int64_t spin_limit, int32_t* gave_up) {
         return RFB_ERR_CUDA;
     }
     *gave_up = (hv[0] == 1u && hv[1] == 1u) ? 1 : 0;
+    return RFB_OK;
+}
+
+rfb_status rfb_selftest_wait_limit(rfb_soc_handle* h, int64_t polls) {
+    if (!h) return RFB_ERR_INVALID_ARG;
+    if (polls < 0 || polls > ((int64_t)1 << 26)) {
+        set_err(h, "polls must be in [0, 2^26]");
+        return RFB_ERR_INVALID_ARG;
+    }
+    h->wait_polls = polls ? (unsigned)polls : RES_SPIN_LIMIT;
     return RFB_OK;
 }
 

@@ -51,7 +51,8 @@ constexpr int RES_RING = 4;        // pairs of x / y halo words polled per edge 
 // column's cells are immediate offsets and take no address registers.
 constexpr int RES_ROWS = 640;      // bx * (by + 2) at most
 constexpr int RES_PLANE = 2 * RES_ROWS;
-// polls of one wait before it gives up (each a round trip to L2: about a second)
+// polls of one wait before it gives up (each a round trip to L2: about a second), unless the
+// handle says otherwise
 constexpr unsigned RES_SPIN_LIMIT = 1u << 20;
 
 struct ResArgs {
@@ -72,6 +73,7 @@ struct ResArgs {
     unsigned long long* inbox;     // CTAs x 2 slots x stride words
     int stride;
     unsigned int* err;             // set if a neighbour's word never arrives
+    unsigned polls;                // of one wait, at most
 };
 
 // words of one inbox slot: the z faces, then the x and y faces
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep32r_kernel(const ResArgs A) {
                     Sr[at + plane] = __uint_as_float((uint32_t)word[m][1]);
                     pend &= ~(4u << m);
                 }
-            if (spin >= RES_SPIN_LIMIT && pend) {      // give up, and wait no more
+            if (spin + 1 >= A.polls && pend) {         // give up, and wait no more
                 atomicExch(A.err, 1u);
                 good = false;
                 pend = 0;
@@ -378,6 +380,7 @@ struct Res64Args {
     unsigned long long* inbox;     // CTAs x 2 slots x stride entries of two words
     int stride;
     unsigned int* err;
+    unsigned polls;
 };
 
 __device__ __forceinline__ void res_send64(unsigned long long* p, double x, uint32_t tag) {
@@ -525,7 +528,7 @@ __global__ void __launch_bounds__(RES_T, 1) sweep64r_kernel(const Res64Args A) {
                     pend &= ~(1u << m);
                 }
             }
-            if (spin >= RES_SPIN_LIMIT && pend) {
+            if (spin + 1 >= A.polls && pend) {
                 atomicExch(A.err, 1u);
                 good = false;
                 pend = 0;

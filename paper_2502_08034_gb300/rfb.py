@@ -123,6 +123,7 @@ def lib():
         L.rfb_soc_tuned_fp32_kernel.argtypes = [H, POINTER(c_int32), POINTER(c_double),
                                                 POINTER(c_double)]
         L.rfb_selftest_bounded_wait.argtypes = [c_int64, POINTER(c_int32)]
+        L.rfb_selftest_wait_limit.argtypes = [H, c_int64]
         L.rfb_soc_solve_nernst.argtypes = [H, c_double, c_double, c_double, c_double,
                                            POINTER(SolveOpts), POINTER(SolveResult)]
         L.rfb_soc_get_overpotential.argtypes = [H, c_void_p, c_int]
@@ -135,7 +136,8 @@ def lib():
                      "rfb_soc_current_noalloc", "rfb_soc_upsample", "rfb_soc_set_area_mult",
                      "rfb_soc_adjoint", "rfb_soc_batch_create", "rfb_soc_batch_solve",
                      "rfb_soc_batch_destroy", "rfb_soc_tuned_fp32_kernel",
-                     "rfb_selftest_bounded_wait", "rfb_soc_solve_nernst",
+                     "rfb_selftest_bounded_wait", "rfb_selftest_wait_limit",
+                     "rfb_soc_solve_nernst",
                      "rfb_soc_get_overpotential", "rfb_soc_solve_bv", "rfb_soc_get_bv_state"):
             getattr(L, name).restype = c_int
         _LIB = L
@@ -396,6 +398,11 @@ class Solver:
     @property
     def kernel_launches(self) -> int:
         return int(lib().rfb_soc_kernel_launches(self.h))
+
+    def selftest_wait_limit(self, polls=0):
+        """rfb_selftest_wait_limit: waits of the resident kernels give up after ``polls`` polls
+        (0: the default)."""
+        self._check(lib().rfb_selftest_wait_limit(self.h, int(polls)))
 
     def tuned_fp32_kernel(self):
         """(name, plain ms/sweep, blocked ms/sweep) chosen by the autotuner ("resident":
