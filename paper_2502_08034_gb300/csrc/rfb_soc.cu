@@ -160,6 +160,7 @@ struct rfb_soc_handle {
         int threads = 0;          // whole warps for a brick's columns and its polled side faces
         int edge = 0;             // whole warps for its outer columns and those faces alone
         unsigned long long* inbox = nullptr;
+        size_t words = 0;         // of the inbox
         uint32_t tag = 0;
     } res, res64, res_cg, res_bv;
     unsigned long long* cg_rows = nullptr;   // reduction rows of the resident potential solve
@@ -313,9 +314,17 @@ void reduce_readback(rfb_soc_handle* h, int min_slot0) {
 
 // After a reduction: whether a bounded wait of the sweeps before it gave up (a TMA stage of a
 // pass, or a neighbour's word of the resident sweeps); the word is cleared for the next call.
+// The tags of a potential solve go on from CTA 0's counts, and where it gave up, other CTAs may
+// have sent words beyond those: they are wiped, or the next solve would take them for its own.
+// (The sweeps' tags go on by the sweeps of a launch, however it ended.)
 bool wait_gave_up(rfb_soc_handle* h) {
     if (h->h_red[NRED] == 0.0) return false;
     CK(h, cudaMemsetAsync(wait_err_word(h), 0, sizeof(unsigned int), h->stream));
+    if (h->cg_rows) {
+        const int ctas = h->res_cg.gx * h->res_cg.gy * h->res_cg.gz;
+        CK(h, cudaMemsetAsync(h->res_cg.inbox, 0, h->res_cg.words * 8, h->stream));
+        CK(h, cudaMemsetAsync(h->cg_rows, 0, (size_t)ctas * 4 * 8, h->stream));
+    }
     set_err(h, "the sweep kernel waited too long for a TMA stage or for a neighbour's values");
     return true;
 }
@@ -1911,7 +1920,8 @@ void bv_res_potential(rfb_soc_handle* h, const BVArgs& B, const double* kcell, c
     A.polls = h->wait_polls;
     const int ctas = P.gx * P.gy * P.gz, smem = bv_cg_smem(P.cpt);
     if (!P.inbox) {
-        dalloc(h, &P.inbox, (size_t)ctas * 4 * A.stride);
+        P.words = (size_t)ctas * 4 * A.stride;
+        dalloc(h, &P.inbox, P.words);
         dalloc(h, &h->cg_rows, (size_t)ctas * 4);
         dalloc(h, &h->cg_out, BV_CG_OUT);
     }

@@ -1,6 +1,7 @@
 """Failure detection of the resident kernels, without a fault: a wait that gives up (after one
 poll, when its words are still on their way) ends the call with an error at that cycle, whichever
 call it is, and the calls after it return what a fresh handle returns."""
+import dataclasses
 import functools
 import time
 
@@ -68,6 +69,32 @@ def test_solves_stop_at_the_cycle(precision):
             u, _ = sv.umt(1e-10, precision=precision)
             out.append((r["I_tot"], u, r["sweeps"], sv.get_state()))
     assert out[0][:3] == out[1][:3] and np.array_equal(out[0][3], out[1][3])
+
+
+def test_potential_solves_after_one_that_gave_up():
+    """Blocks that went on after the first one had given up leave words with tags that the next
+    solve uses: it must not take them (solves cut off at many points, then one to its end)."""
+    from paper_2502_08034_gb300 import rfb, synth
+    case = dataclasses.replace(synth.build_case("waitbv", (13, 11, 15), 0.82, 4.0, 5, 0.002, -0.10,
+                                                0.2, 1e-12, flow_device="cuda"), k0=2e-5)
+    out = []
+    for fail in (True, False):
+        with rfb.Solver.from_case(case) as sv:
+            sv.solve(case.s_in, case.eta, 1e-12)
+            kw = dict(start="sbv", cycle=50, max_sweeps=100, allow_not_converged=True)
+            for polls in range(1, 13) if fail else ():
+                sv.selftest_wait_limit(polls)
+                try:
+                    sv.solve_bv(case.s_in, case.eta, 1e-30, **kw)
+                    assert polls > 1
+                except rfb.RfbError as e:
+                    assert e.status == rfb.RFB_ERR_CUDA
+                sv.selftest_wait_limit(0)
+            r = sv.solve_bv(case.s_in, case.eta, 1e-30, **kw)
+            out.append((r["I_tot"], r["cg_iterations"], r["phi_min"], sv.get_bv_state()))
+    assert out[0][:3] == out[1][:3]
+    for k, x in out[0][3].items():
+        assert np.array_equal(x, out[1][3][k])
 
 
 def test_wait_limit_arguments():
