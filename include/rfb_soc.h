@@ -531,6 +531,12 @@ rfb_status rfb_selftest_bounded_wait(int64_t spin_limit, int32_t* gave_up);
  * call ends with RFB_ERR_CUDA, the states hold no result, and the next call runs as usual. */
 rfb_status rfb_selftest_wait_limit(rfb_soc_handle* h, int64_t polls);
 
+/* Self-test of the way round a refused launch: from now on (on != 0) this handle's launches of
+ * resident kernels, which need all their blocks on the chip at once, are treated as refused
+ * (as in a context that has a part of the SMs). The call then runs on the launches that need no
+ * such thing, and so do the handle's later calls (after on = 0, until rfb_soc_set_stream). */
+rfb_status rfb_selftest_refuse_resident(rfb_soc_handle* h, int32_t on);
+
 /* The FP32 correction kernel the handle's autotuner chose for RFB_PREC_MIXED solves with
  * fp32_kernel = 0 or 2 (or the one a solve forced), as an opts.fp32_kernel value: 0 = not
  * chosen yet, 1 = one sweep per launch, 3 / 4 = two-sweep passes in the persistent /

@@ -161,6 +161,7 @@ struct rfb_soc_handle {
         int edge = 0;             // whole warps for its outer columns and those faces alone
         unsigned long long* inbox = nullptr;
         size_t words = 0;         // of the inbox
+        bool refused = false;     // the launch was: see res_launch
         uint32_t tag = 0;
     } res, res64, res_cg, res_bv;
     unsigned long long* cg_rows = nullptr;   // reduction rows of the resident potential solve
@@ -168,6 +169,7 @@ struct rfb_soc_handle {
     uint32_t cg_rtag = 0;
     bool res_used = false;        // the last FP32 correction sweeps were resident ones
     unsigned wait_polls = RES_SPIN_LIMIT;    // of a resident kernel's wait, at most
+    bool refuse_resident = false;            // self-test: as if every such launch were refused
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 };
 
@@ -542,6 +544,29 @@ void res_plan(rfb_soc_handle* h, rfb_soc_handle::ResPlan& P, const std::vector<i
     }
 }
 
+// The launch of a resident kernel: every CTA at once (measured: with part of the SMs held for
+// 3 s by another stream's kernel none starts before all can, so no wait runs out meanwhile).
+// False where that is refused (a context or stream with a part of the SMs, no cooperative
+// launches): nothing has run, the plan is given up, and the launches that need no such thing
+// serve this call and those after it on this stream.
+bool res_launch(rfb_soc_handle* h, rfb_soc_handle::ResPlan& P, const void* k, void* args, int smem) {
+    if (P.refused) return false;
+    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    void* list[] = {args};
+    const cudaError_t e =
+        h->refuse_resident ? cudaErrorCooperativeLaunchTooLarge
+                           : cudaLaunchCooperativeKernel(k, dim3(P.gx * P.gy * P.gz),
+                                                         dim3(P.threads), list, smem, h->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        (void)cudaGetLastError();
+        P.refused = true;
+        return false;
+    }
+    CK(h, e);
+    ++h->launches;
+    return true;
+}
+
 template <bool ADJ>
 void (*res64_kernel(int cpt))(Res64Args) {
     switch (cpt) {
@@ -557,13 +582,13 @@ void (*res64_kernel(int cpt))(Res64Args) {
 // cells): 6.5 us a sweep at 396k cells, where launches take 12.3.
 bool res64_fits(rfb_soc_handle* h) {
     if (h->res64.cpt < 0) res_plan(h, h->res64, {2, 3, 4, 5, 6}, RES64_RING);
-    return h->res64.cpt > 0;
+    return h->res64.cpt > 0 && !h->res64.refused;
 }
 
 // n FP64 sweeps from buf[cur] (adjoint: transposed steps with source g), 2048 a launch; the
-// result is left in buf[cur]
-void res64_sweeps(rfb_soc_handle* h, const OpPoint& op, double** buf, int& cur, int64_t n,
-                  const double* g) {
+// result is left in buf[cur]. Returns the sweeps that were not run (n: the launch was refused).
+int64_t res64_sweeps(rfb_soc_handle* h, const OpPoint& op, double** buf, int& cur, int64_t n,
+                     const double* g) {
     auto& P = h->res64;
     Res64Args A{};
     A.L = lattice(h);
@@ -583,19 +608,16 @@ void res64_sweeps(rfb_soc_handle* h, const OpPoint& op, double** buf, int& cur, 
     A.inbox = P.inbox;
     const auto k = g ? res64_kernel<true>(P.cpt) : res64_kernel<false>(P.cpt);
     const int smem = res64_smem(P.cpt);
-    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     for (int64_t q = 0; q < n; q += A.n) {
         A.n = (int)std::min<int64_t>(n - q, 2048);
         A.in = buf[cur];
         A.out = buf[cur ^ 1];
         A.tag = P.tag;
+        if (!res_launch(h, P, (const void*)k, &A, smem)) return n - q;
         P.tag += (uint32_t)A.n;
-        void* args[] = {&A};
-        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads), args, smem,
-                                          h->stream));
-        ++h->launches;
         cur ^= 1;
     }
+    return 0;
 }
 
 // n FP64 sweeps on s (or t for U_mt), ping-pong, with the assembled operator
@@ -606,10 +628,7 @@ void sweeps64(rfb_soc_handle* h, const OpPoint& op, bool umt, int64_t n) {
     const float* dtc = op.dt_mode == RFB_DT_LOCAL ? h->d_dtc : nullptr;
     Lattice L = lattice(h);
     const Coef<double> C = make_coef<double>(h, op, false, false);
-    if (!C.nl && n > 1 && res64_fits(h)) {
-        res64_sweeps(h, op, buf, cur, n, nullptr);
-        return;
-    }
+    if (!C.nl && n > 1 && res64_fits(h)) n = res64_sweeps(h, op, buf, cur, n, nullptr);
     for (int64_t q = 0; q < n; ++q) {
         const auto k = C.nl ? (dtc ? sweep64c_kernel<true, true> : sweep64c_kernel<true, false>)
                             : (dtc ? sweep64c_kernel<false, true> : sweep64c_kernel<false, false>);
@@ -907,7 +926,7 @@ ResKernel res_kernel(int cpt) {
 // cells): 1.7 us a sweep at 528k cells, where launches and passes take 6.2 us.
 bool res_fits(rfb_soc_handle* h) {
     if (h->res.cpt < 0) res_plan(h, h->res, {2, 4, 6, 8, 10, 12}, 2 * RES_RING);
-    return h->res.cpt > 0;
+    return h->res.cpt > 0 && !h->res.refused;
 }
 
 // Sweeps whose multiples the check intervals of a default solve are where its sweeps run
@@ -934,8 +953,9 @@ int res_depth(rfb_soc_handle* h) {
 }
 
 // n sweeps (tr: of the transposed operator) from delta = 0; the result is left in d_delta[0].
-// One launch does them all, or 4096 at a time (a launch of some ms).
-void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n, bool tr) {
+// One launch does them all, or 4096 at a time (a launch of some ms). False: the launch was
+// refused, nothing has run.
+bool res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n, bool tr) {
     auto& P = h->res;
     ResArgs A{};
     A.nx = h->nx; A.ny = h->ny; A.nz = h->nz;
@@ -954,19 +974,20 @@ void res_sweeps(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int6
     A.inbox = P.inbox;
     const ResKernel k = tr ? res_kernel<true>(P.cpt) : res_kernel<false>(P.cpt);
     const int smem = res_smem(P.cpt);
-    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     for (int64_t q = 0; q < n; q += A.n) {
         A.n = (int)std::min<int64_t>(n - q, 4096);
         A.in = q ? h->d_delta[0] : nullptr;
         A.out = h->d_delta[q ? 1 : 0];
         A.tag = P.tag;
+        if (!res_launch(h, P, (const void*)k, &A, smem)) {
+            if (q == 0) return false;
+            set_err(h, "resident sweeps: a launch was refused after one that was not");
+            throw Fail{RFB_ERR_CUDA};
+        }
         P.tag += (uint32_t)A.n;
-        void* args[] = {&A};
-        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads), args, smem,
-                                          h->stream));
-        ++h->launches;
         if (q) swap_delta(h);
     }
+    return true;
 }
 
 // How a call's FP32 sweeps run: one launch per sweep, passes of the chosen variant (two or
@@ -978,8 +999,9 @@ enum class Sweep32 { plain, pass, apart, resident };
 // The result is left in d_delta[0].
 void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Sweep32::plain) {
     if (how == Sweep32::resident) {
-        res_sweeps(h, op, make_coef<float>(h, op, true, false), n, false);
-        return;
+        if (res_sweeps(h, op, make_coef<float>(h, op, true, false), n, false)) return;
+        h->res_used = false;
+        how = Sweep32::plain;
     }
     const bool use_tb = how != Sweep32::plain;
     const size_t bytes = (size_t)h->N * sizeof(float);
@@ -1012,10 +1034,9 @@ void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Swe
 // before, else passes of the step-field kernels (two or three sweeps each, the variant the
 // autotuner chose), plain sweeps for the remainder.
 void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n) {
-    if (op.dt_mode == RFB_DT_LOCAL && h->tb[1].variant < 0 && res_fits(h)) {
-        res_sweeps(h, op, C, n, true);
+    if (op.dt_mode == RFB_DT_LOCAL && h->tb[1].variant < 0 && res_fits(h) &&
+        res_sweeps(h, op, C, n, true))
         return;
-    }
     const size_t bytes = (size_t)h->N * sizeof(float);
     CK(h, cudaMemsetAsync(h->d_delta[0], 0, bytes, h->stream));
     CK(h, cudaMemsetAsync(h->d_delta[1], 0, bytes, h->stream));
@@ -1643,6 +1664,7 @@ rfb_status rfb_soc_set_stream(rfb_soc_handle* h, void* s) {
     rfb_status g = guard(h);
     if (g) return g;
     h->stream = (cudaStream_t)s;
+    for (auto* P : {&h->res, &h->res64, &h->res_cg, &h->res_bv}) P->refused = false;
     return RFB_OK;
 }
 
@@ -1861,18 +1883,18 @@ bool bv_cg_fits(rfb_soc_handle* h) {
     auto& P = h->res_cg;
     if (P.cpt < 0) res_plan(h, P, {2, 3, 4}, BV_RING, 1, 256);
     if (P.cpt == 0) res_plan(h, P, {2, 3, 4}, BV_RING);
-    return P.cpt > 0;
+    return P.cpt > 0 && !P.refused;
 }
 bool bv_sweep_fits(rfb_soc_handle* h) {
     auto& P = h->res_bv;
     if (P.cpt < 0) res_plan(h, P, {BVS_CPT}, BV_RING, 3, 256);
     if (P.cpt == 0) res_plan(h, P, {BVS_CPT}, BV_RING, 3);
-    return P.cpt > 0;
+    return P.cpt > 0 && !P.refused;
 }
 
 // n species sweeps at the potential phi from buf[v][cur] into buf[v][cur ^ 1] and on, 2048 a
-// launch
-void bv_res_sweeps(rfb_soc_handle* h, const BVArgs& B, const double* phi, double* (&buf)[3][2],
+// launch. Returns the sweeps that were not run (the launch was refused).
+int64_t bv_res_sweeps(rfb_soc_handle* h, const BVArgs& B, const double* phi, double* (&buf)[3][2],
                    int& cur, int64_t n) {
     auto& P = h->res_bv;
     BVSweepArgs A{};
@@ -1886,7 +1908,6 @@ void bv_res_sweeps(rfb_soc_handle* h, const BVArgs& B, const double* phi, double
     if (!P.inbox) dalloc(h, &P.inbox, (size_t)ctas * 12 * A.stride);
     A.inbox = P.inbox;
     const auto k = P.threads <= 256 ? bv_sweepr_kernel<256> : bv_sweepr_kernel<RES_T>;
-    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     for (int64_t q = 0; q < n; q += A.n) {
         A.n = (int)std::min<int64_t>(n - q, 2048);
         for (int v = 0; v < 3; ++v) {
@@ -1894,18 +1915,16 @@ void bv_res_sweeps(rfb_soc_handle* h, const BVArgs& B, const double* phi, double
             A.C2[v] = buf[v][cur ^ 1];
         }
         A.tag = P.tag;
+        if (!res_launch(h, P, (const void*)k, &A, smem)) return n - q;
         P.tag += (uint32_t)A.n;
-        void* args[] = {&A};
-        CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads),
-                                          args, smem, h->stream));
-        ++h->launches;
         cur ^= 1;
     }
+    return 0;
 }
 
 // One potential solve: out receives the iterations, the looks without progress and the
-// BV_STATS values of the last look.
-void bv_res_potential(rfb_soc_handle* h, const BVArgs& B, const double* kcell, const double* kmem,
+// BV_STATS values of the last look. False: the launch was refused.
+bool bv_res_potential(rfb_soc_handle* h, const BVArgs& B, const double* kcell, const double* kmem,
                       const double* bphi, double* phi, double tol, int max_it,
                       double (&out)[BV_CG_OUT]) {
     auto& P = h->res_cg;
@@ -1931,16 +1950,13 @@ void bv_res_potential(rfb_soc_handle* h, const BVArgs& B, const double* kcell, c
     A.tag = P.tag;
     A.rtag = h->cg_rtag;
     const auto k = bv_cgr(P.cpt, P.threads);
-    CK(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    void* args[] = {&A};
-    CK(h, cudaLaunchCooperativeKernel((const void*)k, dim3(ctas), dim3(P.threads), args, smem,
-                                      h->stream));
-    ++h->launches;
+    if (!res_launch(h, P, (const void*)k, &A, smem)) return false;
     CK(h, cudaMemcpyAsync(out, h->cg_out, sizeof out, cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     // the next launch's words follow this one's
     P.tag += (uint32_t)out[2 + BV_STATS];
     h->cg_rtag += (uint32_t)out[3 + BV_STATS];
+    return true;
 }
 
 // N-double fields of the Butler-Volmer state in h->d_bv: 0-1 O, 2-3 R, 4-5 H
@@ -2051,7 +2067,6 @@ rfb_status rfb_soc_solve_bv(rfb_soc_handle* h, double s_in, double eta, double t
         const double scale[3] = {c0, c0, P.c_H_in};
         std::vector<double> hp((size_t)BV_NB * BV_STATS);
         const int nb = (int)std::min<int64_t>(BV_NB, (N + BV_TPB - 1) / BV_TPB);
-        const bool res_cg = bv_cg_fits(h), res_sweep = bv_sweep_fits(h);
         double hred[NRED + 1];
         rfb_bv_result r{};
         rfb_status st = RFB_OK;
@@ -2083,10 +2098,10 @@ rfb_status rfb_soc_solve_bv(rfb_soc_handle* h, double s_in, double eta, double t
         bool cg_ok = false;
         auto potential = [&](double bmax) -> double {
             double* phi = bv_field(h, 6);
-            if (res_cg) {
-                double o[BV_CG_OUT];
+            double o[BV_CG_OUT];
+            if (bv_cg_fits(h) &&
                 bv_res_potential(h, A, bv_field(h, 9), bv_field(h, 10), bv_field(h, 8), phi,
-                                 P.cg_rtol * bmax, P.max_cg, o);
+                                 P.cg_rtol * bmax, P.max_cg, o)) {
                 const double* st6 = o + 2;
                 r.cg_iterations += (int64_t)o[0];
                 r.phi_mean = st6[2] / (double)h->n_fluid;
@@ -2197,13 +2212,14 @@ rfb_status rfb_soc_solve_bv(rfb_soc_handle* h, double s_in, double eta, double t
                 break;
             }
             const int64_t n = std::min<int64_t>(P.cycle, o.max_sweeps - done);
-            if (res_sweep) {
+            int64_t left = n;
+            if (bv_sweep_fits(h)) {
                 double* buf[3][2];
                 for (int v = 0; v < 3; ++v)
                     for (int c = 0; c < 2; ++c) buf[v][c] = bv_field(h, 2 * v + c);
-                bv_res_sweeps(h, A, bv_field(h, 6), buf, h->bv_cur, n);
+                left = bv_res_sweeps(h, A, bv_field(h, 6), buf, h->bv_cur, n);
             }
-            for (int64_t q = 0; q < n && !res_sweep; ++q) {
+            for (int64_t q = 0; q < left; ++q) {
                 const int cur = h->bv_cur;
                 bv_sweep_kernel<<<flat_grid(N), BV_TPB, 0, h->stream>>>(
                     A, bv_field(h, 0 + cur), bv_field(h, 2 + cur), bv_field(h, 4 + cur),
@@ -2596,9 +2612,9 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
                 break;
             }
             const int64_t n = std::min(every, o.max_sweeps - done);
-            const bool resident = res64_fits(h);
-            if (resident) res64_sweeps(h, op, h->d_lam, cur, n, h->d_g);
-            for (int64_t q = 0; q < n && !resident; ++q) {
+            int64_t left = n;
+            if (res64_fits(h)) left = res64_sweeps(h, op, h->d_lam, cur, n, h->d_g);
+            for (int64_t q = 0; q < left; ++q) {
                 adjoint64c_kernel<0><<<h->sgrid, h->block, 0, h->stream>>>(
                     lattice(h), h->K, C.dtc, op.dt, h->d_lam[cur], h->d_lam[cur ^ 1], h->d_g,
                     nullptr, op.umt, h->skchunk);
@@ -2687,6 +2703,12 @@ rfb_status rfb_selftest_wait_limit(rfb_soc_handle* h, int64_t polls) {
         return RFB_ERR_INVALID_ARG;
     }
     h->wait_polls = polls ? (unsigned)polls : RES_SPIN_LIMIT;
+    return RFB_OK;
+}
+
+rfb_status rfb_selftest_refuse_resident(rfb_soc_handle* h, int32_t on) {
+    if (!h) return RFB_ERR_INVALID_ARG;
+    h->refuse_resident = on != 0;
     return RFB_OK;
 }
 

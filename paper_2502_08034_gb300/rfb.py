@@ -124,6 +124,7 @@ def lib():
                                                 POINTER(c_double)]
         L.rfb_selftest_bounded_wait.argtypes = [c_int64, POINTER(c_int32)]
         L.rfb_selftest_wait_limit.argtypes = [H, c_int64]
+        L.rfb_selftest_refuse_resident.argtypes = [H, c_int32]
         L.rfb_soc_solve_nernst.argtypes = [H, c_double, c_double, c_double, c_double,
                                            POINTER(SolveOpts), POINTER(SolveResult)]
         L.rfb_soc_get_overpotential.argtypes = [H, c_void_p, c_int]
@@ -137,6 +138,7 @@ def lib():
                      "rfb_soc_adjoint", "rfb_soc_batch_create", "rfb_soc_batch_solve",
                      "rfb_soc_batch_destroy", "rfb_soc_tuned_fp32_kernel",
                      "rfb_selftest_bounded_wait", "rfb_selftest_wait_limit",
+                     "rfb_selftest_refuse_resident",
                      "rfb_soc_solve_nernst",
                      "rfb_soc_get_overpotential", "rfb_soc_solve_bv", "rfb_soc_get_bv_state"):
             getattr(L, name).restype = c_int
@@ -403,6 +405,10 @@ class Solver:
         """rfb_selftest_wait_limit: waits of the resident kernels give up after ``polls`` polls
         (0: the default)."""
         self._check(lib().rfb_selftest_wait_limit(self.h, int(polls)))
+
+    def selftest_refuse_resident(self, on=True):
+        """rfb_selftest_refuse_resident: launches of resident kernels are treated as refused."""
+        self._check(lib().rfb_selftest_refuse_resident(self.h, int(on)))
 
     def tuned_fp32_kernel(self):
         """(name, plain ms/sweep, blocked ms/sweep) chosen by the autotuner ("resident":
