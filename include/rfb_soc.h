@@ -123,9 +123,13 @@ typedef struct rfb_solve_opts {
                                three-sweep passes (128 x 10 tiles, the update
                                coefficients of the two older levels in tensor memory),
                                persistent / chunked; 9 / 10 = as 7 / 8 with five delta
-                               stages instead of four. Every pass is bitwise the same
-                               number of one-sweep launches; check intervals are whole
-                               passes */
+                               stages instead of four; 11 = resident sweeps (a lattice
+                               that fits on the chip, else RFB_ERR_INVALID_ARG); 12 / 13 =
+                               as 3 / 4 with narrow tiles cut to the lattice. Every pass is
+                               bitwise the same number of one-sweep launches; the default
+                               check interval of 3 .. 10, 12 and 13 is whole passes. An
+                               adjoint takes 1; other values leave it what the handle's
+                               forward solves chose */
     int32_t timeout_ms;     /* > 0: stop after the first FP64 check at or past this much
                                wall time since the call began and return
                                RFB_ERR_NOT_CONVERGED (the state is valid); 0 = none */
@@ -309,7 +313,7 @@ typedef enum rfb_objective {
  *                    RFB_PREC_MIXED (FP32 sweeps of the transposed operator correcting lam,
  *                    defects g + L^T lam in double-float arithmetic, the last one confirmed
  *                    in FP64; kinetics mode 0 or U_MT, nx % 4 == 0, else
- *                    RFB_ERR_INVALID_ARG)
+ *                    RFB_ERR_INVALID_ARG; fp32_kernel 1: one sweep per launch)
  *   d_area_mult      nullable; N doubles (host or device per kind) receiving dJ/dm_c
  *                    (zero on solid cells and cells without fiber neighbours)
  *   d_velocity_scale nullable; host double receiving dJ/dbeta
@@ -542,8 +546,7 @@ rfb_status rfb_selftest_refuse_resident(rfb_soc_handle* h, int32_t on);
  * chosen yet, 1 = one sweep per launch, 3 / 4 = two-sweep passes in the persistent /
  * chunked launch shape, 5 / 6 the same with four TMA stages, 7 .. 10 three-sweep passes,
  * 11 = resident sweeps (fp32_kernel = 0 on a lattice that fits on the chip), 12 / 13 =
- * two-sweep passes with narrow tiles, persistent / chunked (chosen by timing only);
- * and the timed device milliseconds per sweep of the one-sweep kernel and of the fastest
+ * two-sweep passes with narrow tiles, persistent / chunked; and the timed device milliseconds per sweep of the one-sweep kernel and of the fastest
  * pass variant (0 if not timed). Any output pointer may be NULL. */
 rfb_status rfb_soc_tuned_fp32_kernel(const rfb_soc_handle* h, int32_t* kernel,
                                      double* plain_ms_per_sweep,

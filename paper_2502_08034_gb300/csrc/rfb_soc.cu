@@ -1032,9 +1032,10 @@ void sweeps32(rfb_soc_handle* h, const OpPoint& op, int64_t n, Sweep32 how = Swe
 // dt (L^T delta + r), from delta = 0; the result is left in d_delta[0] (nx % 4 == 0).
 // With local steps: resident sweeps where the lattice fits and no pass variant was chosen
 // before, else passes of the step-field kernels (two or three sweeps each, the variant the
-// autotuner chose), plain sweeps for the remainder.
-void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n) {
-    if (op.dt_mode == RFB_DT_LOCAL && h->tb[1].variant < 0 && res_fits(h) &&
+// autotuner chose), plain sweeps for the remainder. plain: one-sweep launches alone.
+void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C, int64_t n,
+                      bool plain) {
+    if (op.dt_mode == RFB_DT_LOCAL && !plain && h->tb[1].variant < 0 && res_fits(h) &&
         res_sweeps(h, op, C, n, true))
         return;
     const size_t bytes = (size_t)h->N * sizeof(float);
@@ -1044,7 +1045,7 @@ void sweeps32_adjoint(rfb_soc_handle* h, const OpPoint& op, const Coef<float>& C
     Lattice L = lattice(h);
     int cur = 0;
     int64_t q = 0;
-    if (local && tb_eligible(h, true)) {
+    if (local && !plain && tb_eligible(h, true)) {
         tb_prepare(h);
         if (h->tb[1].variant < 0) h->tb[1].variant = 1;   // chunked shape unless tuned
         const int k = tb_depth(h, true);
@@ -1195,15 +1196,21 @@ bool read_opts(rfb_soc_handle* h, const rfb_solve_opts* in, rfb_solve_opts* o) {
     for (int q = 0; q < 6; ++q)
         if (o->reserved[q] != 0) { set_err(h, "opts.reserved must be zero"); return false; }
     if (o->timeout_ms < 0) { set_err(h, "opts.timeout_ms must be >= 0"); return false; }
-    if (o->fp32_kernel < 0 || o->fp32_kernel > 10 ||
+    if (o->fp32_kernel < 0 || o->fp32_kernel > 13 ||
         (o->fp32_kernel >= 5 && o->dt_mode != RFB_DT_LOCAL)) {
         set_err(h, "opts.fp32_kernel must be 0 (auto), 1 (one sweep), 2 (passes), 3 / 4 "
                    "(two-sweep passes, persistent / chunked launch) or, with local steps, "
-                   "5 / 6 (the same with four TMA stages), 7 / 8 (three-sweep passes) or "
-                   "9 / 10 (three-sweep passes with five delta stages)");
+                   "5 / 6 (the same with four TMA stages), 7 / 8 (three-sweep passes), "
+                   "9 / 10 (three-sweep passes with five delta stages), 11 (resident sweeps) "
+                   "or 12 / 13 (two-sweep passes with narrow tiles)");
         return false;
     }
-    if (o->fp32_kernel >= 2 && !tb_eligible(h, o->dt_mode == RFB_DT_LOCAL)) {
+    if (o->fp32_kernel == 11) {
+        if (!res_fits(h)) {
+            set_err(h, "resident sweeps need a lattice that fits on the chip");
+            return false;
+        }
+    } else if (o->fp32_kernel >= 2 && !tb_eligible(h, o->dt_mode == RFB_DT_LOCAL)) {
         set_err(h, "two-sweep passes need nz >= 2 and nx %% 4 == 0 (local steps), or nx %% 16 "
                    "== 0 and no area multiplier (global step)");
         return false;
@@ -1284,7 +1291,7 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
     bool use_tb = false, use_res = false;
     if (mixed) {
         h->tb_last = local;
-        use_res = o.fp32_kernel == 0 && local && res_fits(h);
+        use_res = o.fp32_kernel == 11 || (o.fp32_kernel == 0 && local && res_fits(h));
         h->res_used = use_res;
         if (use_res) {
         } else if (o.fp32_kernel == 2) {
@@ -1292,11 +1299,13 @@ rfb_status drive(rfb_soc_handle* h, const rfb_solve_opts& o, OpPoint& op, bool u
             use_tb = true;
         } else if (o.fp32_kernel >= 3) {
             // a forced variant (kept for later calls): 3 / 4 and 5 / 6 two-sweep passes with
-            // three / four TMA stages, 7 / 8 and 9 / 10 three-sweep passes with four / five
-            T.variant = o.fp32_kernel <= 4   ? o.fp32_kernel - 3
-                        : o.fp32_kernel <= 6 ? (o.fp32_kernel - 5) | 2
-                        : o.fp32_kernel <= 8 ? (o.fp32_kernel - 7) | 4
-                                             : (o.fp32_kernel - 9) | 6;
+            // three / four TMA stages, 7 / 8 and 9 / 10 three-sweep passes with four / five,
+            // 12 / 13 two-sweep passes with narrow tiles
+            T.variant = o.fp32_kernel <= 4    ? o.fp32_kernel - 3
+                        : o.fp32_kernel <= 6  ? (o.fp32_kernel - 5) | 2
+                        : o.fp32_kernel <= 8  ? (o.fp32_kernel - 7) | 4
+                        : o.fp32_kernel <= 10 ? (o.fp32_kernel - 9) | 6
+                                              : (o.fp32_kernel - 12) | 8;
             T.forced = true;
             use_tb = true;
         } else if (o.fp32_kernel == 0) {
@@ -2580,7 +2589,7 @@ rfb_status rfb_soc_adjoint(rfb_soc_handle* h, rfb_objective obj, double tol,
                     break;
                 }
                 const int64_t n = std::min(every, o.max_sweeps - done);
-                sweeps32_adjoint(h, op, C32, n);
+                sweeps32_adjoint(h, op, C32, n, o.fp32_kernel == 1);
                 df_check(true);
                 joined = false;
                 done += n;

@@ -155,7 +155,8 @@ class RfbError(RuntimeError):
 FP32_KERNEL = {"auto": 0, "plain": 1, "blocked": 2, "blocked_persistent": 3,
                "blocked_chunked": 4, "blocked4_persistent": 5, "blocked4_chunked": 6,
                "three_sweep_persistent": 7, "three_sweep_chunked": 8,
-               "three_sweep5_persistent": 9, "three_sweep5_chunked": 10}
+               "three_sweep5_persistent": 9, "three_sweep5_chunked": 10, "resident": 11,
+               "blocked_narrow_persistent": 12, "blocked_narrow_chunked": 13}
 
 
 def make_opts(precision="fp64", inlet_bc="face", dt_mode="local", check_every=0, cfl=0.4,
@@ -415,8 +416,7 @@ class Solver:
         the lattice fits on the chip and nothing was timed)."""
         k, a, b = c_int32(), c_double(), c_double()
         self._check(lib().rfb_soc_tuned_fp32_kernel(self.h, byref(k), byref(a), byref(b)))
-        names = {0: None, 1: "plain", 11: "resident", 12: "blocked_narrow_persistent",
-                 13: "blocked_narrow_chunked"}
+        names = {0: None, 1: "plain"}
         names.update({v: k for k, v in FP32_KERNEL.items() if v >= 3})
         return names[k.value], a.value, b.value
 
