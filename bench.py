@@ -36,11 +36,13 @@ DT_SWEEP_BYTES_PER_CELL = 4 + 4 + 4 + 12 + 4
 
 
 def pass_kernel(kname):
-    """(sweeps per launch, kernel description) of an FP32 kernel name of the binding."""
+    """(sweeps per launch, kernel description) of an FP32 kernel name of the binding; None for
+    the resident kernel, whose launch does the sweeps of a whole correction cycle, as many as
+    the check interval has there."""
     if not kname or kname == "plain":
         return 1, "sweep32d_kernel (one sweep)"
     if kname == "resident":
-        return 200, "sweep32r_kernel (resident: the sweeps of a correction cycle in one launch)"
+        return None, "sweep32r_kernel (resident: the sweeps of a correction cycle in one launch)"
     shape = kname.rsplit("_", 1)[1]
     if kname.startswith("three_sweep"):
         return 3, ("sweep32t3_kernel (three-sweep TMA-staged pass, coefficients of the older "
@@ -49,6 +51,29 @@ def pass_kernel(kname):
     return 2, ("sweep32tbd_kernel (two-sweep TMA-staged pass, %s launch, %d TMA stages%s)" % (
         shape, 4 if kname.startswith("blocked4") else 3,
         ", narrow tiles" if "narrow" in kname else ""))
+
+
+def sweep_roofline(kname, n_cells, sweeps, sweep_ms, peak):
+    """The roofline entry of `sweeps` FP32 sweeps over n_cells cells in sweep_ms of kernel time:
+    algorithmic bytes per launch (each cell's correction, forcing, three face velocities and
+    step read once, the correction written once, whether the launch applies one sweep or a
+    pass), and the captured DRAM bytes, over the time of a launch. The resident kernel keeps the
+    fields on the chip: it has no bytes per sweep, and its entry no figures."""
+    depth, kdesc = pass_kernel(kname)
+    out = {"bound": "hbm", "achieved": None, "peak": peak, "unit": "GB/s", "frac": None,
+           "traffic": None, "kernel": kdesc, "sweeps_per_launch": depth, "dram_frac": None}
+    if depth is None:
+        out["bound"] = "on-chip: words between blocks, shared memory"
+        return out
+    launches = (sweeps + depth - 1) // depth
+    out["achieved"] = DT_SWEEP_BYTES_PER_CELL * n_cells * launches / (sweep_ms / 1e3) / 1e9
+    out["frac"] = out["achieved"] / peak
+    out["traffic"] = kernel_traffic(n_cells, kname)
+    if out["traffic"]:
+        out["dram_frac"] = out["traffic"] * launches / (sweep_ms / 1e3) / 1e9 / peak
+    return out
+
+
 FALLBACK_HBM_GBS = 6800.0
 
 
@@ -75,7 +100,8 @@ def parse():
                     choices=["auto", "plain", "blocked", "blocked_persistent", "blocked_chunked",
                              "blocked4_persistent", "blocked4_chunked",
                              "three_sweep_persistent", "three_sweep_chunked",
-                             "three_sweep5_persistent", "three_sweep5_chunked"],
+                             "three_sweep5_persistent", "three_sweep5_chunked", "resident",
+                             "blocked_narrow_persistent", "blocked_narrow_chunked"],
                     help="FP32 correction kernel: chosen by the autotuner (default), one sweep "
                          "per launch, or TMA-staged passes (variant autotuned; two-sweep "
                          "passes persistent, or one (tile, z chunk) item per CTA; blocked4: "
@@ -493,10 +519,7 @@ def run_upsample(args):
     N = cases[-1].n
     fr = levels[-1]
     kname, _, _ = fine.tuned_fp32_kernel()
-    depth, kdesc = pass_kernel(kname)
-    launches_fine = (fr["sweeps"] + depth - 1) // depth
-    # algorithmic bytes per launch (a pass reads and writes each cell once)
-    achieved = DT_SWEEP_BYTES_PER_CELL * N * launches_fine / (fr["sweep_ms"] / 1e3) / 1e9
+    roof = sweep_roofline(kname, N, fr["sweeps"], fr["sweep_ms"], peak)
     effective = DT_SWEEP_BYTES_PER_CELL * N * fr["sweeps"] / (fr["sweep_ms"] / 1e3) / 1e9
     out = {"metric": METRIC, "value": cells / (elapsed / 1e3) / 1e9, "unit": UNIT,
            "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
@@ -511,12 +534,9 @@ def run_upsample(args):
                       "U_mt_sweeps": ru["sweeps"]},
            "cold_start_finest": {"sweeps": cold["sweeps"], "time_ms": cold["time_ms"]},
            "upsample_gain": upsample_gain,
-           "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                        "frac": achieved / peak,
-                        "traffic": kernel_traffic(N, kname) if depth > 1 else None,
-                        "kernel": "%s on the finest level" % kdesc,
-                        "bytes_per_cell_per_launch": DT_SWEEP_BYTES_PER_CELL,
-                        "peak_kind": peak_kind},
+           "roofline": dict(roof, kernel="%s on the finest level" % roof["kernel"],
+                            bytes_per_cell_per_launch=DT_SWEEP_BYTES_PER_CELL,
+                            peak_kind=peak_kind),
            "effective_bandwidth": {"value": effective, "unit": "GB/s", "frac": effective / peak,
                                    "note": "28 B per cell per sweep x sweeps/s, finest level"},
            "clocks": clk.summary(), "setup_s": setup_s}
@@ -818,20 +838,11 @@ def main():
     value = units / (elapsed_ms / 1e3) / 1e9
     sweep_ms = sum(r["sweep_ms"] for r in results)
     peak, peak_kind = peak_hbm()
-    # algorithmic bytes per launch: a launch reads each cell's correction, forcing, three
-    # face velocities and step once and writes the correction once, whether it applies
-    # one sweep or a two-sweep pass
     kname, tuned_plain_ms, tuned_blocked_ms = sv.tuned_fp32_kernel()
     if args.fp32_kernel not in ("auto", "blocked"):
         kname = args.fp32_kernel
-    depth, kdesc = pass_kernel(kname)   # one launch per `depth` sweeps
-    kernel_launches = (sweeps + depth - 1) // depth
-    achieved = DT_SWEEP_BYTES_PER_CELL * N * kernel_launches / (sweep_ms / 1e3) / 1e9
+    roof = sweep_roofline(kname, N, sweeps, sweep_ms, peak)
     effective = DT_SWEEP_BYTES_PER_CELL * N * sweeps / (sweep_ms / 1e3) / 1e9
-    traffic = kernel_traffic(N, kname)
-    # measured DRAM bytes per launch over the launch time: the kernel's % of HBM peak
-    launch_s = (sweep_ms / 1e3) / max(1, kernel_launches)
-    dram_frac = traffic / launch_s / 1e9 / peak if traffic else None
     last = results[-1]
 
     extras = {}
@@ -940,14 +951,10 @@ def main():
                "sweeps_per_step": sweeps / args.steps,
                "residual": last["residual"], "I_tot_A": last["I_tot"], "U": last["U"],
                "mass_balance_rel": last["mass_balance_rel"],
-               "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak,
-                            "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
-                            "kernel": kdesc, "sweeps_per_launch": depth,
-                            "autotuner_ms_per_sweep": {"plain": tuned_plain_ms,
-                                                       "blocked": tuned_blocked_ms},
-                            "bytes_per_cell_per_launch": DT_SWEEP_BYTES_PER_CELL,
-                            "dram_frac": dram_frac, "nominal_peak_gbs": 7900.0,
-                            "peak_kind": peak_kind},
+               "roofline": dict(roof, autotuner_ms_per_sweep={"plain": tuned_plain_ms,
+                                                              "blocked": tuned_blocked_ms},
+                                bytes_per_cell_per_launch=DT_SWEEP_BYTES_PER_CELL,
+                                nominal_peak_gbs=7900.0, peak_kind=peak_kind),
                "effective_bandwidth": {"value": effective, "unit": "GB/s",
                                        "frac": effective / peak,
                                        "note": "28 B per cell per sweep x sweeps/s"},

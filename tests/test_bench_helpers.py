@@ -108,3 +108,20 @@ def test_oracle_baselines_on_every_core_and_to_steady_state():
     assert workers == min(os.cpu_count() or 1, 4) and rate > 0 and sec > 0
     t, n = bench.oracle_time_to_steady(case, 1e-8)
     assert t > 0 and 0 < n < 100000
+
+
+def test_roofline_entries_follow_the_launches_of_the_kernel():
+    """Passes: one read of the fields per launch of their sweeps; resident sweeps keep the fields
+    on the chip, so their entry has no bytes (a launch does a check interval's sweeps, whatever
+    that is)."""
+    n, ms, peak = 10 ** 6, 2.0, 6000.0
+    for kernel, depth in (("plain", 1), ("blocked4_chunked", 2), ("blocked_narrow_persistent", 2),
+                          ("three_sweep_chunked", 3)):
+        r = bench.sweep_roofline(kernel, n, 601, ms, peak)
+        launches = -(-601 // depth)
+        assert r["sweeps_per_launch"] == depth and r["bound"] == "hbm"
+        assert r["achieved"] == bench.DT_SWEEP_BYTES_PER_CELL * n * launches / 2e-3 / 1e9
+        assert r["frac"] == r["achieved"] / peak
+    r = bench.sweep_roofline("resident", n, 601, ms, peak)
+    assert r["sweeps_per_launch"] is None and "sweep32r_kernel" in r["kernel"]
+    assert r["achieved"] is r["frac"] is r["traffic"] is r["dram_frac"] is None
