@@ -933,18 +933,21 @@ bool res_fits(rfb_soc_handle* h) {
 // resident: the depth of the launches that the resident sweeps replaced (why: see
 // tune_fp32_kernel), by a rule on their shapes instead of a timing, so that a solve stops at
 // the same sweep every time. One-sweep launches were the fastest where one wave of their
-// blocks fills the chip (three blocks of 256 threads per SM, together up to 10 2/3 planes:
-// 6.7 to 7.7 us a sweep, beyond that 8.8 and more); of the passes the three-sweep ones (7.4 to
-// 7.6 us up to 12 plane steps, from 13 on 8.1 and more) where the two-sweep ones take 11 steps
-// (7.7 to 8.0; with 10 steps 7.0). A timing came to the same on 129 of 147 lattices of up to
-// 1 M cells; of the others 17 take as long either way within 4 %, and the blocks of one
-// (132x44x114) are half empty.
+// blocks fills the chip (three blocks of 256 threads per SM: 6.7 to 7.3 us a sweep with up to
+// three planes a block, 8.6 and more beyond), with four planes a block only up to 8.5 planes
+// per SM (7.2 to 7.4; from there 7.8 to 9.2) or where less than three eighths of a block's
+// threads have cells (7.2 on average). Of the passes the three-sweep ones were (7.4 to 7.6 us up
+// to 12 plane steps, from 13 on 8.0 and more) where the two-sweep ones take 11 steps (7.7 to
+// 8.0; with 10 steps 7.0). A timing came to the same on 463 of 538 lattices of up to 0.95 M
+// cells, two thirds of them near one of these lines; the others take as long either way within
+// a few percent.
 int res_depth(rfb_soc_handle* h) {
     if (!tb_eligible(h, true)) return 1;
     int sms = 152, chunks = 1;
     CK(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     const int64_t blocks = (int64_t)h->vgrid.x * h->vgrid.y * h->vgrid.z;
-    if (blocks <= 3 * sms && 3 * blocks * h->vkchunk <= 32 * sms) return 1;
+    const int vk = h->vkchunk;
+    if (blocks <= 3 * sms && (vk <= 3 || h->nx < 48 || 2 * blocks * vk <= 17 * sms)) return 1;
     auto steps = [&](int rows, int k) {
         const int64_t tiles = (int64_t)((h->nx + TB_TXI - 1) / TB_TXI) * ((h->ny + rows - 1) / rows);
         return best_chunks(tiles, h->nz, sms, k, &chunks);

@@ -43,11 +43,13 @@ def _solves(dims, kernel):
 
 
 # one wave of one-sweep blocks; more, whose two-sweep launches were the faster; three-sweep ones
-@pytest.mark.parametrize("dims,depth", [((64, 64, 64), 1), ((88, 84, 110), 1), ((32, 81, 165), 2),
-                                        ((72, 64, 176), 2), ((136, 76, 69), 3),
+@pytest.mark.parametrize("dims,depth", [((64, 64, 64), 1), ((88, 84, 110), 1), ((24, 203, 63), 1),
+                                        ((32, 81, 165), 2), ((72, 64, 176), 2),
+                                        ((132, 44, 114), 3), ((136, 76, 69), 3),
                                         ((64, 88, 141), 3)])
 def test_resident_solves_stop_like_the_launches_they_replaced(dims, depth):
-    got, want = _solves(dims, "auto"), _solves(dims, DEPTH[depth])
+    got, want = _solves(dims, "resident"), _solves(dims, DEPTH[depth])
+    assert [n for n, _ in _solves(dims, "auto")] == [n for n, _ in got]
     assert [n for n, _ in got] == [n for n, _ in want]
     for (_, s), (_, t) in zip(got, want):
         assert np.array_equal(s, t)
