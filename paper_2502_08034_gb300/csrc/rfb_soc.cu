@@ -1209,7 +1209,13 @@ bool read_opts(rfb_soc_handle* h, const rfb_solve_opts* in, rfb_solve_opts* o) {
         return false;
     }
     if (o->fp32_kernel == 11) {
-        if (!res_fits(h)) {
+        bool fits = false;
+        try {
+            fits = res_fits(h);
+        } catch (Fail) {                     // no C++ exception leaves a C entry point
+            return false;
+        }
+        if (!fits) {
             set_err(h, "resident sweeps need a lattice that fits on the chip");
             return false;
         }
