@@ -1082,7 +1082,7 @@ struct TuneKey {
 std::map<TuneKey, rfb_soc_handle::TBChoice> g_tune_cache;
 std::mutex g_tune_mu;
 
-// Project-written autotuner for one lattice: time (twice, keeping the faster) 12 plain
+// Project-written autotuner for one lattice: time (up to twice, keeping the faster) 12 plain
 // sweeps and 12 sweeps of each launch shape of the two-sweep pass (with local steps: with
 // three and with four TMA stages, and with narrow tiles) by CUDA events on the current
 // forcing and keep the fastest (tb_only: choose between the pass variants only).
@@ -1116,7 +1116,7 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
             return;
         }
     }
-    // candidates: plain (-1), then pass variants (12 sweeps: whole passes of each). Not the
+    // candidates: pass variants (12 sweeps: whole passes of each), then plain (-1). Not the
     // three-sweep passes: since passes overlap their ends the two-sweep ones are faster on every
     // lattice measured (us per sweep of the best of each: 128x128x256 10.6 and 13.7, 160x160x200
     // 18.8 and 23.2, 192^3 22.7 and 26.6, 256^3 41.0 and 42.3, 256x256x512 75 and 87).
@@ -1124,10 +1124,12 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
     if (local) cands = {0, 1, 2, 3, 8, 9};
     float ms[10], plain_ms = INFINITY;
     for (float& m : ms) m = INFINITY;
-    auto time_one = [&](int v, float& best, bool apart = false) {
+    // lead: the fastest of those it competes with so far; one that its first timing leaves more
+    // than a quarter behind is not timed again. fresh: its kernel has not run yet (warm-up)
+    auto time_one = [&](int v, float& best, float lead, bool fresh, bool apart = false) {
         const Sweep32 how = v < 0 ? Sweep32::plain : apart ? Sweep32::apart : Sweep32::pass;
         if (v >= 0) T.variant = v;
-        sweeps32(h, op, 6, how);   // warm-up (and tensor maps)
+        if (fresh) sweeps32(h, op, 6, how);
         for (int rep = 0; rep < 2; ++rep) {   // the faster of two timings
             float t = 0.f;
             CK(h, cudaEventRecord(h->ev[0], h->stream));
@@ -1136,17 +1138,22 @@ void tune_fp32_kernel(rfb_soc_handle* h, const OpPoint& op, bool tb_only = false
             CK(h, cudaEventSynchronize(h->ev[1]));
             CK(h, cudaEventElapsedTime(&t, h->ev[0], h->ev[1]));
             best = std::min(best, t);
+            if (t > 1.25f * lead) break;
         }
     };
-    if (!tb_only) time_one(-1, plain_ms);
-    for (int v : cands) time_one(v, ms[v]);
+    float lead = INFINITY;
+    for (int v : cands) {                                // both shapes of a kernel in a row
+        time_one(v, ms[v], lead, (v & 1) == 0);
+        lead = std::min(lead, ms[v]);
+    }
     float two = INFINITY, three = INFINITY;              // launched apart, as above
     if (local) {
-        for (int v : {1, 2, 3}) time_one(v, two, true);
-        for (int v : {4, 5}) time_one(v, three, true);
+        for (int v : {1, 2, 3}) time_one(v, two, two, false, true);
+        for (int v : {4, 5}) time_one(v, three, std::min(two, three), v == 4, true);
     } else {
-        two = std::min(ms[0], ms[1]);                    // its passes never overlap
+        two = lead;                                      // its passes never overlap
     }
+    if (!tb_only) time_one(-1, plain_ms, std::min(two, three), true);
     T.pass_depth = two <= three ? 2 : 3;
     T.auto_depth = plain_ms <= std::min(two, three) ? 1 : T.pass_depth;
     int bestv = 0;
